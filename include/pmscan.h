@@ -518,6 +518,13 @@ void pm_server_destroy(pm_server *s);
  */
 int pm_selfcheck_host_walk(const pm_set *s, const uint8_t *T, int64_t n, pm_result **out);
 
+/*
+ * The same for the set's sampled-gram tables (the ones its scans on a GPU
+ * take when the launch plan is automatic): a host walk of them. PM_EINVAL for
+ * a set that has none (a pinned launch plan, or patterns too short).
+ */
+int pm_selfcheck_gram_walk(const pm_set *s, const uint8_t *T, int64_t n, pm_result **out);
+
 const char *pm_strerror(int code);
 int pm_last_cuda_error(void);  /* cudaError_t of the last PM_ECUDA, per thread */
 const char *pm_version(void);

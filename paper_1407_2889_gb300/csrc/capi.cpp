@@ -5,6 +5,8 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <system_error>
+#include <thread>
 
 #include <cuda_runtime.h>
 
@@ -118,6 +120,7 @@ void release_device(pm_set *s)
                     s->dwm.hcode, s->dwm.grp_off, s->dwm.grp_ids, s->dwm.poff, s->dwm.fcode, s->dwm.flen,
                     s->dacv.table, s->dacv.cls, s->dacv.omask, s->dacv.orank, s->dacv.out_off, s->dacv.out_ent,
                     s->dac2.table2,
+                    s->dgram.base,
                     s->c_text, s->c_ws, s->c_out, s->c_counts};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -127,6 +130,7 @@ void release_device(pm_set *s)
     s->dwm = DevWm();
     s->dacv = DevAcv();
     s->dac2 = DevAc2();
+    s->dgram = DevGram();
     s->c_text = s->c_ws = s->c_out = s->c_counts = nullptr;
     s->c_text_cap = s->c_ws_cap = s->c_out_cap = 0;
 }
@@ -249,6 +253,91 @@ int upload_wm(pm_set *s)
     return rc;
 }
 
+// The gram tables of a set whose launch plan is automatic: scans then take
+// them instead of the automaton or the shift tables (scan_gram.cu).
+bool plan_is_automatic(const pm_set *s)
+{
+    const pm_params &p = s->params;
+    if (s->algo == PM_ALGO_WM || s->algo == PM_ALGO_WMV) return p.warps_per_cta == 0 && p.ctas_per_sm == 0;
+    return p.placement == PM_PLACE_AUTO && p.smem_table_bytes == 0 && p.warps_per_cta == 0 && p.ctas_per_sm == 0 &&
+           p.counters == 0 && p.ids_place == 0 && p.stride == 0;
+}
+
+int upload_gram(pm_set *s, const DeviceProps &dp)
+{
+    const GramTables &t = s->gram;
+    DevGram &d = s->dgram;
+    if (!t.ok) return PM_OK;
+    int rc = gram_plan(t, dp, d);
+    if (rc || !d.use) return rc;
+    // one allocation and one copy: a small set's compile is mostly these
+    const struct { const void *src; size_t bytes; void **dst; } part[] = {
+        {t.filter.data(), t.filter.size() * 4, reinterpret_cast<void **>(&d.filter)},
+        {t.rank_base.data(), t.rank_base.size() * 4, reinterpret_cast<void **>(&d.rank_base)},
+        {t.dir.data(), t.dir.size() * 4, reinterpret_cast<void **>(&d.dir)},
+        {t.ent.data(), t.ent.size() * sizeof(GramEntry), &d.ent},
+        {t.pats.data(), t.pats.size() * 4, reinterpret_cast<void **>(&d.pats)},
+        {t.code.data(), t.code.size() * 4, reinterpret_cast<void **>(&d.code)},
+        {t.grp_off.data(), t.grp_off.size() * 4, reinterpret_cast<void **>(&d.grp_off)},
+        {t.grp_ids.data(), t.grp_ids.size() * 4, reinterpret_cast<void **>(&d.grp_ids)}};
+    size_t total = 0;
+    for (const auto &p : part) total += (p.bytes + 15) & ~size_t(15);
+    try {
+        std::vector<uint8_t> all(total, 0);
+        size_t at = 0;
+        for (const auto &p : part) {
+            if (p.bytes) std::memcpy(all.data() + at, p.src, p.bytes);
+            at += (p.bytes + 15) & ~size_t(15);
+        }
+        rc = upload(&d.base, all.data(), all.size(), s->device_bytes);
+    } catch (const std::bad_alloc &) {
+        return PM_ENOMEM;
+    }
+    if (rc) return rc;
+    size_t at = 0;
+    for (const auto &p : part) {
+        *p.dst = static_cast<uint8_t *>(d.base) + at;
+        at += (p.bytes + 15) & ~size_t(15);
+    }
+    s->dac.gt = s->dwm.gt = s->dacv.gt = &s->gram;
+    s->dac.dg = s->dwm.dg = s->dacv.dg = &s->dgram;
+    return PM_OK;
+}
+
+// Builds the gram tables beside the automaton, on a thread of its own when
+// the set is large enough for that to pay (100,000 32-mers: 65 of 355 ms).
+class GramJob {
+public:
+    GramJob(pm_set *s, const uint8_t *P, const int64_t *off, int64_t d, int32_t m)
+    {
+        if (!plan_is_automatic(s)) return;
+        // The transition-table walk of one-length Aho-Corasick sets costs about
+        // 220 instructions per lane and 16 bytes, whatever matches (d = 8000,
+        // m = 8, where one position in nine matches: 1.38 ms per GiB against
+        // 2.29 for grams of cost 360); the other scans are always slower.
+        const double limit = s->algo == PM_ALGO_AC ? 220.0 : 1e30;
+        auto work = [=]() { rc_ = build_gram(P, off, d, m, limit, s->gram); };
+        if (d >= 2000) {
+            try {
+                thread_ = std::thread(work);
+                return;
+            } catch (const std::exception &) {  // no thread to be had: built here
+            }
+        }
+        work();
+    }
+    ~GramJob() { join(); }
+    int join()
+    {
+        if (thread_.joinable()) thread_.join();
+        return rc_;
+    }
+
+private:
+    std::thread thread_;
+    int rc_ = PM_OK;
+};
+
 int finish_compile(pm_set *s, pm_set **out)
 {
     if (s->host_only) {
@@ -273,6 +362,7 @@ int finish_compile(pm_set *s, pm_set **out)
             s->dac2.use = rc == PM_OK;
         }
     }
+    if (!rc) rc = upload_gram(s, dp);
     if (rc) {
         release_device(s);
         delete s;
@@ -412,11 +502,14 @@ int pm_ac_compile(const uint8_t *P, int64_t d, int32_t m, const pm_params *opt, 
     s->algo = PM_ALGO_AC;
     if (opt) s->params = *opt;
     s->host_only = s->params.host_only != 0;
+    GramJob gram(s, P, nullptr, d, m);
     int rc = build_ac(P, d, m, s->ac);
     if (!rc) {
         build_ac2(s->ac);  // the two-character table of an eligible set
         if (s->params.stride == 2 && s->ac.table2.empty()) rc = PM_ETOOBIG;
     }
+    const int rg = gram.join();
+    if (!rc) rc = rg;
     if (rc) {
         delete s;
         return rc;
@@ -432,7 +525,10 @@ int pm_pfac_compile(const uint8_t *P, int64_t d, int32_t m, const pm_params *opt
     s->algo = PM_ALGO_PFAC;
     if (opt) s->params = *opt;
     s->host_only = s->params.host_only != 0;
+    GramJob gram(s, P, nullptr, d, m);
     int rc = build_pfac(P, d, m, s->ac);
+    const int rg = gram.join();
+    if (!rc) rc = rg;
     if (rc) {
         delete s;
         return rc;
@@ -448,7 +544,10 @@ int pm_acv_compile(const uint8_t *P, const int64_t *offsets, int64_t d, const pm
     s->algo = PM_ALGO_ACV;
     if (opt) s->params = *opt;
     s->host_only = s->params.host_only != 0;
+    GramJob gram(s, P, offsets, d, 0);
     int rc = build_acv(P, offsets, d, s->acv);
+    const int rg = gram.join();
+    if (!rc) rc = rg;
     if (rc) {
         delete s;
         return rc;
@@ -466,7 +565,10 @@ int pm_wmv_compile(const uint8_t *P, const int64_t *offsets, int64_t d, int32_t 
     if (opt) s->params = *opt;
     s->host_only = s->params.host_only != 0;
     const int bp = s->params.wm_prefix_len > 0 ? s->params.wm_prefix_len : 2;
+    GramJob gram(s, P, offsets, d, 0);
     int rc = build_wmv(P, offsets, d, B, bp, s->wm);
+    const int rg = gram.join();
+    if (!rc) rc = rg;
     if (rc) {
         delete s;
         return rc;
@@ -485,7 +587,10 @@ int pm_wm_compile(const uint8_t *P, int64_t d, int32_t m, int32_t B, const pm_pa
     s->host_only = s->params.host_only != 0;
     int bp = s->params.wm_prefix_len > 0 ? s->params.wm_prefix_len : 2;
     if (bp > m) bp = m;
+    GramJob gram(s, P, nullptr, d, m);
     int rc = build_wm(P, d, m, B, bp, s->wm);
+    const int rg = gram.join();
+    if (!rc) rc = rg;
     if (rc) {
         delete s;
         return rc;
@@ -685,15 +790,19 @@ static int tune_wm(pm_set *s, const uint8_t *d_text, int64_t n, bool list, int32
     pm_params best_p = s->params;
     float best_t = -1.0f;
     std::vector<std::pair<int, int>> tried;   // (warps, hist_smem)
-    for (int w : {0, 24, 20, 16, 12, 8}) {
+    // -1: the gram scan, where the set has it (its parameters are the automatic ones)
+    for (int w : {-1, 0, 24, 20, 16, 12, 8}) {
+        if (w < 0 && !s->dgram.use) continue;
         pm_params p = s->params;
-        p.warps_per_cta = w;
+        p.warps_per_cta = w < 0 ? 0 : w;
         DevWm plan = saved;
         if (wm_plan(t, p, dp, plan) != PM_OK) continue;
+        plan.gt = w < 0 ? &s->gram : nullptr;
+        plan.dg = w < 0 ? &s->dgram : nullptr;
         bool dup = false;
         for (const auto &x : tried) dup = dup || (x.first == plan.warps && x.second == plan.hist_smem);
         if (dup) continue;
-        tried.push_back({plan.warps, plan.hist_smem});
+        if (w >= 0) tried.push_back({plan.warps, plan.hist_smem});
         auto run = [&]() {
             return wm_launch(t, plan, d_text, n, list, static_cast<int64_t *>(counts), static_cast<uint64_t *>(occ),
                              n_occ, static_cast<int64_t *>(nocc), ws, st);
@@ -771,6 +880,7 @@ int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t
     }
     // candidate plans: the current one, then placement x warps x counters x ids
     std::vector<pm_params> cand;
+    if (s->dgram.use) cand.push_back(pm_params{});  // the gram scan
     cand.push_back(s->params);
     cand.back().stride = 1;
     for (int place : {PM_PLACE_AUTO, PM_PLACE_HYBRID})
@@ -792,6 +902,9 @@ int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t
     for (const pm_params &p : cand) {
         DevAc plan = saved;
         if (ac_plan(t, p, dp, plan) != PM_OK) continue;
+        const bool gram = s->dgram.use && &p == &cand.front();
+        plan.gt = gram ? &s->gram : nullptr;
+        plan.dg = gram ? &s->dgram : nullptr;
         bool dup = false;
         // a late-ids plan's list mode does not count in the scan kernel, so
         // plans differing only in counters are one candidate there; the
@@ -799,6 +912,7 @@ int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t
         // mode) is kept
         const bool late_list = list && plan.ids_smem == 2;
         for (const Tried &x : tried) {
+            if (x.plan.dg) continue;
             if (late_list && x.plan.ids_smem == 2) {  // only the list-mode launch matters
                 dup = dup || (x.plan.warps_list == plan.warps_list && x.plan.variant_list == plan.variant_list &&
                               x.plan.smem_entries == plan.smem_entries);
@@ -867,7 +981,7 @@ int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t
     s->dac = tried[bi].plan;  // same device tables, new launch plan
     s->dac2.use = false;
     s->params = tried[bi].params;
-    s->params.stride = 1;
+    if (!s->dac.dg) s->params.stride = 1;
     if (best_out) *best_out = s->params;
     if (best_ms) *best_ms = tried[bi].ms;
     return PM_OK;
@@ -1263,6 +1377,29 @@ int pm_scan_batch(const pm_set *const *sets, const uint8_t *const *texts, const 
     return PM_OK;
 }
 
+static int host_result(const std::vector<uint64_t> &occ, const std::vector<int64_t> &counts, pm_result **out)
+{
+    pm_result *r = new_result(int64_t(counts.size()), int64_t(occ.size()), true, false);
+    if (!r) return PM_ENOMEM;
+    if (!occ.empty()) std::memcpy(r->occ, occ.data(), occ.size() * 8);
+    std::memcpy(r->counts, counts.data(), counts.size() * 8);
+    *out = r;
+    return PM_OK;
+}
+
+int pm_selfcheck_gram_walk(const pm_set *s, const uint8_t *T, int64_t n, pm_result **out)
+{
+    if (!s || !out || n < 0 || (n > 0 && !T) || !s->gram.ok) return PM_EINVAL;
+    try {
+        std::vector<uint64_t> occ;
+        std::vector<int64_t> counts;
+        host_walk_gram(s->gram, T, n, occ, counts);
+        return host_result(occ, counts, out);
+    } catch (const std::bad_alloc &) {
+        return PM_ENOMEM;
+    }
+}
+
 int pm_selfcheck_host_walk(const pm_set *s, const uint8_t *T, int64_t n, pm_result **out)
 {
     if (!s || !out || n < 0 || (n > 0 && !T)) return PM_EINVAL;
@@ -1275,12 +1412,7 @@ int pm_selfcheck_host_walk(const pm_set *s, const uint8_t *T, int64_t n, pm_resu
         else if (s->algo == PM_ALGO_ACV) host_walk_acv(s->acv, T, n, occ, counts);
         else if (s->algo == PM_ALGO_WMV) host_walk_wmv(s->wm, T, n, occ, counts);
         else host_walk_wm(s->wm, T, n, occ, counts);
-        pm_result *r = new_result(int64_t(counts.size()), int64_t(occ.size()), true, false);
-        if (!r) return PM_ENOMEM;
-        if (!occ.empty()) std::memcpy(r->occ, occ.data(), occ.size() * 8);
-        std::memcpy(r->counts, counts.data(), counts.size() * 8);
-        *out = r;
-        return PM_OK;
+        return host_result(occ, counts, out);
     } catch (const std::bad_alloc &) {
         return PM_ENOMEM;
     }

@@ -1,0 +1,264 @@
+// gram.cpp -- host-side tables of the sampled-gram scan (scan_gram.cu) and a
+// host walk of them.
+//
+// Every pattern of the set is at least m characters long (m the shortest
+// length). Take a stride s and a gram length q with q <= m - s + 1. Of the s
+// consecutive text positions i .. i + s - 1 after a start i exactly one, t, is
+// a multiple of s, and the q characters at t are the characters k .. k + q - 1
+// of any pattern that occurs at i, k = t - i < s. So it is enough to look at
+// the grams at multiples of s: each pattern enters a table under its first s
+// grams (offset k = 0 .. s - 1), a text gram not in the table rules out s
+// starts at once, and a gram that is in it names the candidates (pattern, k),
+// which are compared with the text byte by byte. This is the block idea of
+// Wu-Manber's SHIFT and HASH tables (Section 3.2, Algorithms 4 and 5) with a
+// fixed shift s, so that no position depends on the one before it.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <new>
+#include <string>
+#include <string_view>
+#include <unordered_map>
+
+#include "pm_internal.h"
+
+namespace pm {
+
+namespace {
+
+inline uint32_t code2(uint32_t b) { return (b >> 1) & 3u; }
+
+// odd multipliers of the gram hash (any odd numbers with mixed bits do)
+constexpr uint32_t kMul[4] = {0x9E3779B1u, 0x5DB3D743u, 0xA54FF53Bu, 0x510E527Fu};
+
+// the gram's hash, and the filter bit it sets: the word by the hash's top
+// bits, the bit by the low bits of the gram's codes (or of a byte gram's hash)
+uint32_t gram_hash(const GramTables &t, const uint8_t *g, uint32_t *bit)
+{
+    uint32_t h = 0;
+    if (t.qw == 0) {
+        for (int j = 0; j < t.q; ++j) h |= code2(g[j]) << (2 * j);
+        const uint32_t x = h * t.K[0];
+        *bit = (x >> (37 - t.fb)) << 5 | (h & 31u);
+        return x;
+    }
+    for (int w = 0; w < t.qw; ++w) {
+        const uint32_t x = uint32_t(g[4 * w]) | uint32_t(g[4 * w + 1]) << 8 | uint32_t(g[4 * w + 2]) << 16 |
+                           uint32_t(g[4 * w + 3]) << 24;
+        h += x * t.K[w];
+    }
+    *bit = (h >> (37 - t.fb)) << 5 | (h & 31u);
+    return h;
+}
+
+}  // namespace
+
+int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, double limit, GramTables &t)
+{
+    t = GramTables();
+    try {
+        const bool var = off != nullptr;
+        auto first = [&](int64_t r) { return var ? off[r] : r * int64_t(m); };
+        auto len_of = [&](int64_t r) { return int(var ? off[r + 1] - off[r] : m); };
+        // (the other compilers refuse bad offsets and sizes: no plan here)
+        if (d > (int64_t(1) << 23) || (var && off[0] != 0) || (!var && m > 255)) return PM_OK;
+        for (int64_t r = 0; var && r < d; ++r)
+            if (off[r + 1] <= off[r] || off[r + 1] - off[r] > 255) return PM_OK;
+        bool present[256] = {};
+        int lo = 1 << 30, hi = 0;
+        for (int64_t r = 0; r < d; ++r) {
+            const int L = len_of(r);
+            lo = std::min(lo, L);
+            hi = std::max(hi, L);
+            const uint8_t *p = P + first(r);
+            for (int j = 0; j < L; ++j) present[p[j]] = true;
+        }
+        int letters = 0;
+        bool packed = true, seen[4] = {};
+        for (uint32_t b = 0; b < 256; ++b) {
+            if (!present[b]) continue;
+            ++letters;
+            if (seen[code2(b)]) packed = false;
+            seen[code2(b)] = true;
+        }
+
+        // Plan: the stride and gram that cost least per 16 text bytes, in
+        // instructions per lane: each probe, each gram that passes the filter
+        // (by chance in the hashed filter, or because so many grams of the
+        // alphabet are in the table), and each entry compared (G / space is
+        // the mean number of entries under a gram of random text; without
+        // that term a set of 8,000 8-mers would take 1-character grams).
+        double best = 1e30;
+        for (int s = 16; s >= 1; s >>= 1) {
+            int q = std::min(16, lo - s + 1);
+            if (!packed) q &= ~3;
+            if (q < (packed ? 3 : 4)) continue;
+            const double G = double(d) * s;
+            if (G > 8.0e6) continue;
+            const double space = std::pow(double(std::max(letters, 2)), double(q));
+            const double natural = 1.0 - std::exp(-G / space);
+            const bool direct = packed && 2 * q <= 18;
+            int fb = direct ? 2 * q : 12;
+            if (!direct)
+                while (fb < 20 && double(1u << fb) < 32.0 * G) ++fb;
+            const double chance = direct ? 0.0 : 1.0 - std::exp(-G / double(1u << fb));
+            const double pass = 1.0 - (1.0 - natural) * (1.0 - chance);
+            const double probes = 16.0 / s;
+            const double cost = 24.0 + probes * ((packed ? 9.0 : 8.0 + q / 4) + 40.0 * pass + 60.0 * G / space);
+            if (cost < best) {
+                best = cost;
+                t.s = s;
+                t.q = q;
+                t.qw = packed ? 0 : q / 4;
+                t.fb = fb;
+                t.rank = direct;
+            }
+        }
+        // too short for any gram, too many patterns, or so many matches that
+        // the automaton is faster
+        if (t.s == 0 || best > limit) {
+            t = GramTables();
+            return PM_OK;
+        }
+        t.var = var;
+        t.d = d;
+        t.m_min = lo;
+        t.m_max = hi;
+        for (int w = 0; w < 4; ++w) t.K[w] = kMul[w];
+        if (packed) t.K[0] = (t.rank ? 1u : kMul[0]) << (32 - 2 * t.q);
+
+        // distinct patterns of a one-length set (groups of equal patterns, as
+        // in the other tables); every pattern of its own in a mixed one
+        std::vector<int64_t> rep;
+        if (!var) {
+            std::unordered_map<std::string_view, uint32_t> index;
+            index.reserve(size_t(d) * 2);
+            std::vector<uint32_t> cls(static_cast<size_t>(d)), mult;
+            for (int64_t r = 0; r < d; ++r) {
+                const std::string_view key(reinterpret_cast<const char *>(P + r * int64_t(m)), size_t(m));
+                const auto it = index.emplace(key, uint32_t(rep.size()));
+                if (it.second) {
+                    rep.push_back(r);
+                    mult.push_back(0);
+                }
+                cls[size_t(r)] = it.first->second;
+                ++mult[it.first->second];
+            }
+            t.code.resize(rep.size());
+            std::vector<uint32_t> fill(rep.size(), 0);
+            t.grp_off.push_back(0);
+            for (size_t c = 0; c < rep.size(); ++c) {
+                t.code[c] = uint32_t(rep[c]);
+                if (mult[c] < 2) continue;
+                t.code[c] = 0x80000000u | uint32_t(t.grp_off.size() - 1);
+                fill[c] = t.grp_off.back();
+                t.grp_off.push_back(t.grp_off.back() + mult[c]);
+            }
+            t.grp_ids.resize(t.grp_off.back());
+            for (int64_t r = 0; r < d; ++r) {
+                const uint32_t c = cls[size_t(r)];
+                if (mult[c] >= 2) t.grp_ids[fill[c]++] = uint32_t(r);
+            }
+        } else {
+            rep.resize(size_t(d));
+            t.code.resize(size_t(d));
+            for (int64_t r = 0; r < d; ++r) {
+                rep[size_t(r)] = r;
+                t.code[size_t(r)] = uint32_t(r);
+            }
+        }
+        const size_t nc = rep.size();
+        t.pw = (hi + 3) / 4;
+        t.pats.assign(nc * size_t(t.pw), 0u);
+        for (size_t c = 0; c < nc; ++c)
+            std::memcpy(reinterpret_cast<uint8_t *>(t.pats.data() + c * size_t(t.pw)), P + first(rep[c]),
+                        size_t(len_of(rep[c])));
+
+        // entries, bucket-major; inside a bucket by (k descending, pattern
+        // ascending), so that the starts t - k come out in ascending order
+        // and equal starts in ascending pattern id
+        const size_t G = nc * size_t(t.s);
+        std::vector<uint32_t> h(G);
+        t.filter.assign(size_t(1) << (t.fb - 5), 0u);
+        for (int k = 0; k < t.s; ++k)
+            for (size_t c = 0; c < nc; ++c) {
+                uint32_t b;
+                h[size_t(k) * nc + c] = gram_hash(t, P + first(rep[c]) + k, &b);
+                t.filter[b >> 5] |= 1u << (b & 31);
+            }
+        auto bucket = [&](uint32_t x) -> uint32_t {
+            if (!t.rank) return x >> (32 - t.db);
+            const uint32_t b = x >> (32 - t.fb);
+            return t.rank_base[b >> 5] + uint32_t(__builtin_popcount(t.filter[b >> 5] & ((1u << (b & 31)) - 1u)));
+        };
+        size_t nb;
+        if (t.rank) {
+            t.rank_base.resize(t.filter.size());
+            uint32_t run = 0;
+            for (size_t w = 0; w < t.filter.size(); ++w) {
+                t.rank_base[w] = run;
+                run += uint32_t(__builtin_popcount(t.filter[w]));
+            }
+            nb = run;
+        } else {
+            t.db = 8;
+            while (t.db < 24 && (size_t(1) << t.db) < G) ++t.db;
+            nb = size_t(1) << t.db;
+        }
+        t.dir.assign(nb + 1, 0u);
+        for (const uint32_t x : h) ++t.dir[bucket(x) + 1];
+        for (size_t b = 0; b < nb; ++b) t.dir[b + 1] += t.dir[b];
+        std::vector<uint32_t> at(t.dir.begin(), t.dir.end() - 1);
+        t.ent.resize(G);
+        for (int k = t.s - 1; k >= 0; --k)
+            for (size_t c = 0; c < nc; ++c) {
+                const uint32_t x = h[size_t(k) * nc + c];
+                GramEntry &e = t.ent[at[bucket(x)]++];
+                e.h = x;
+                e.idx = uint32_t(c);
+                e.k_len = uint32_t(k) | uint32_t(len_of(rep[c])) << 8;
+                e.code = t.code[c];
+            }
+        t.ok = true;
+        return PM_OK;
+    } catch (const std::bad_alloc &) {
+        t = GramTables();
+        return PM_ENOMEM;
+    }
+}
+
+void host_walk_gram(const GramTables &t, const uint8_t *T, int64_t n, std::vector<uint64_t> &occ,
+                    std::vector<int64_t> &counts)
+{
+    occ.clear();
+    counts.assign(size_t(t.d), 0);
+    uint8_t g[16];
+    for (int64_t p = 0; p < n; p += t.s) {
+        for (int j = 0; j < 16; ++j) g[j] = p + j < n ? T[p + j] : uint8_t(0);
+        uint32_t b;
+        const uint32_t x = gram_hash(t, g, &b);
+        if (!((t.filter[b >> 5] >> (b & 31)) & 1u)) continue;
+        uint32_t bk;
+        if (t.rank)
+            bk = t.rank_base[b >> 5] + uint32_t(__builtin_popcount(t.filter[b >> 5] & ((1u << (b & 31)) - 1u)));
+        else bk = x >> (32 - t.db);
+        for (uint32_t e = t.dir[bk]; e < t.dir[bk + 1]; ++e) {
+            const GramEntry &en = t.ent[e];
+            const int64_t start = p - int64_t(en.k_len & 255u), len = int64_t(en.k_len >> 8);
+            if (en.h != x || start < 0 || start + len > n) continue;
+            if (std::memcmp(T + start, t.pats.data() + size_t(en.idx) * size_t(t.pw), size_t(len)) != 0) continue;
+            auto put = [&](uint32_t r) {
+                occ.push_back((uint64_t(start) << 32) | r);
+                ++counts[r];
+            };
+            if (en.code & 0x80000000u) {
+                const uint32_t gi = en.code & 0x7FFFFFFFu;
+                for (uint32_t j = t.grp_off[gi]; j < t.grp_off[gi + 1]; ++j) put(t.grp_ids[j]);
+            } else {
+                put(en.code);
+            }
+        }
+    }
+}
+
+}  // namespace pm

@@ -139,7 +139,47 @@ struct AcvTables {
 };
 constexpr int32_t kAcvMaxLen = 65; // the halo of the scan kernels (64 bytes)
 
+// ---------------------------------------------------------------------------
+// Sampled grams (gram.cpp, scan_gram.cu): the table of a set whose grams are
+// looked up at every s-th text position (see gram.cpp). A gram is q
+// characters: 2-bit codes (byte >> 1) & 3 for alphabets they tell apart (qw
+// 0), else qw words of 4 bytes. Its hash h (for 2-bit grams of at most 18
+// bits the gram itself, shifted to the top) picks a filter bit by its top fb
+// bits and a bucket of entries: by its top db bits, or (rank) the gram's
+// rank among the filter's set bits.
+// ---------------------------------------------------------------------------
+struct GramEntry {
+    uint32_t h;       // the gram's hash
+    uint32_t idx;     // distinct pattern: its bytes are pats[idx * pw ..]
+    uint32_t k_len;   // gram offset k in the pattern | pattern length << 8
+    uint32_t code;    // pattern id, or 0x80000000 | group of equal patterns
+};
+
+struct GramTables {
+    bool ok = false;
+    bool var = false;              // mixed lengths: no groups, code = pattern id
+    bool rank = false;             // buckets by rank in the filter
+    int64_t d = 0;
+    int32_t m_min = 0, m_max = 0;
+    int32_t s = 0, q = 0, qw = 0;  // stride, gram length, words of a byte gram
+    int32_t fb = 0, db = 0, pw = 0;
+    uint32_t K[4] = {};
+    std::vector<uint32_t> filter;     // 2^fb bits
+    std::vector<uint32_t> rank_base;  // rank: set bits before each filter word
+    std::vector<uint32_t> dir;        // first entry of each bucket, and the end
+    std::vector<GramEntry> ent;
+    std::vector<uint32_t> pats;       // pw words per distinct pattern, zero padded
+    std::vector<uint32_t> code;       // code of each distinct pattern
+    std::vector<uint32_t> grp_off, grp_ids;
+};
+
 int build_ac(const uint8_t *P, int64_t d, int32_t m, AcTables &out);
+// off NULL: d rows of length m; else pattern r is P[off[r] .. off[r+1]).
+// t.ok stays false (and PM_OK is returned) when the set has no gram plan or
+// its planned cost (instructions per lane and 16 text bytes) exceeds `limit`.
+int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, double limit, GramTables &t);
+void host_walk_gram(const GramTables &t, const uint8_t *T, int64_t n,
+                    std::vector<uint64_t> &occ, std::vector<int64_t> &counts);
 // pattern r is P[off[r] .. off[r+1]); lengths 1..kAcvMaxLen
 int build_acv(const uint8_t *P, const int64_t *off, int64_t d, AcvTables &out);
 void host_walk_acv(const AcvTables &t, const uint8_t *T, int64_t n,
@@ -177,8 +217,22 @@ constexpr int kWarpTile = kLane * kChunk;
 struct AcLaunch;                    // defined in scan_ac.cu
 struct WmLaunch;
 
+// Device copy and plan of the gram tables.
+struct DevGram {
+    void *base = nullptr;           // the one allocation the others point into
+    uint32_t *filter = nullptr, *rank_base = nullptr, *dir = nullptr;
+    void *ent = nullptr;
+    uint32_t *pats = nullptr, *code = nullptr, *grp_off = nullptr, *grp_ids = nullptr;
+    int32_t warps = 0, hist_smem = 0;
+    bool use = false;               // the tables fit this device
+};
+
 // Everything a launcher needs about the device copy of a set.
 struct DevAc {
+    // gram tables that scans of this plan take instead of the transition
+    // table (sets whose launch plan is automatic), or NULL
+    const GramTables *gt = nullptr;
+    const DevGram *dg = nullptr;
     void *table = nullptr;          // entry_bytes * (n_rows << lw)
     uint32_t *grp_off = nullptr;
     uint32_t *grp_ids = nullptr;
@@ -219,6 +273,8 @@ struct DevAc2 {
 };
 
 struct DevAcv {
+    const GramTables *gt = nullptr;  // as in DevAc
+    const DevGram *dg = nullptr;
     void *table = nullptr;          // entry_bytes * (n_rows << lw), index entries for ACGT sets
     uint8_t *cls = nullptr;
     uint32_t *omask = nullptr, *orank = nullptr, *out_off = nullptr, *out_ent = nullptr;
@@ -229,6 +285,8 @@ struct DevAcv {
 };
 
 struct DevWm {
+    const GramTables *gt = nullptr;  // as in DevAc
+    const DevGram *dg = nullptr;
     uint8_t *shift = nullptr;
     uint32_t *hoff = nullptr;
     uint32_t *hids = nullptr;
@@ -304,7 +362,7 @@ struct ListParts {
     unsigned long long *seg_sum = nullptr;
     uint32_t *tile_ent = nullptr, *tile_out = nullptr;
     void *slots = nullptr;
-    int64_t seg_tiles = 0;
+    int64_t seg_tiles = 0, segs = 0;
 };
 int64_t list_workspace_bytes(int64_t nsub, bool list, int64_t nterms, int slot_entry_bytes);
 void list_workspace_parts(void *d_ws, int64_t nsub, int64_t nterms, int slot_entry_bytes, ListParts &out);
@@ -326,6 +384,38 @@ int expand_launch(void *d_ws, int64_t nsub, int64_t nterms, int slot_entry_bytes
                   const uint32_t *grp_ids, int64_t n_grp_off, int64_t n_grp_ids, uint64_t *d_occ,
                   int64_t occ_cap, int64_t *d_n_occ, const unsigned long long *occ_base,
                   unsigned long long pos_base, void *stream, const ExpandLate *late = nullptr);
+// The same for slots of any tile length: `tile` text bytes and `slot_stride`
+// entries per tile; slot_kind 0 and 1 are the 4- and 8-byte entries above, 2
+// holds (offset << 20) | pattern id (mixed lengths, no groups).
+struct ExpandTiles {
+    int64_t tile = 0, slot_stride = 0, ntiles = 0, seg_tiles = 0;
+    int slot_kind = 0;
+    const void *slots = nullptr;
+    const uint32_t *tile_ent = nullptr, *tile_out = nullptr;
+    const unsigned long long *seg_sum = nullptr;
+};
+int expand_tiles_launch(const ExpandTiles &tl, const uint32_t *grp_off, const uint32_t *grp_ids,
+                        int64_t n_grp_off, int64_t n_grp_ids, uint64_t *d_occ, int64_t occ_cap,
+                        int64_t *d_n_occ, const unsigned long long *occ_base, unsigned long long pos_base,
+                        void *stream);
+// sampled-gram scan (scan_gram.cu) on the workspace of any of the scans: its
+// segment sums zeroed, counts and n_occ zeroed or to be added to
+struct GramWs {
+    uint32_t *tile_ent = nullptr, *tile_out = nullptr;
+    unsigned long long *seg_sum = nullptr;
+    void *slots = nullptr;
+    int64_t segs = 1;
+    int per_pos = 1;                // slot entries per text position
+};
+int gram_plan(const GramTables &t, const DeviceProps &dp, DevGram &dev);
+int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, int64_t n, bool list,
+                int64_t *d_counts, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ, const GramWs &ws,
+                const unsigned long long *occ_base, unsigned long long pos_base, void *stream);
+// gram_launch over a list workspace (list_workspace_parts with these sizes)
+int gram_launch_ws(const GramTables &t, const DevGram &dv, const uint8_t *d_text, int64_t n, bool list,
+                   int64_t *d_counts, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ, void *d_ws,
+                   int64_t nterms, int slot_bytes, int per_pos, const unsigned long long *occ_base,
+                   unsigned long long pos_base, void *stream);
 // two characters per lookup (scan_ac2.cu): plan (PM_ETOOBIG if the set is
 // not eligible or the tables do not fit) and scan on the AC workspace
 int ac2_plan(const AcTables &t, const pm_params &opt, const DeviceProps &dp, DevAc2 &dev);
@@ -453,6 +543,8 @@ struct pm_set {
     pm::AcTables ac;
     pm::WmTables wm;
     pm::AcvTables acv;               // PM_ALGO_ACV
+    pm::GramTables gram;
+    pm::DevGram dgram;
     pm::DevAc dac;
     pm::DevWm dwm;
     pm::DevAcv dacv;

@@ -135,7 +135,7 @@ struct ExpandLateArgs {
     dev::WsHeader *ws;
 };
 
-template <typename SE, int kOffShift, uint32_t kGrp, int CM, bool GS>
+template <typename SE, int kOffShift, uint32_t kGrp, int CM, bool GS, bool ANY>
 __global__ void __launch_bounds__(kExpandThreads)
 expand_kernel(const SE *__restrict__ slots, const uint32_t *__restrict__ tile_ent,
               const uint32_t *__restrict__ tile_out, const unsigned long long *__restrict__ seg_sum,
@@ -143,8 +143,9 @@ expand_kernel(const SE *__restrict__ slots, const uint32_t *__restrict__ tile_en
               const uint32_t *__restrict__ grp_off, const uint32_t *__restrict__ grp_ids,
               unsigned long long *__restrict__ occ, long long occ_cap, long long *n_occ,
               const unsigned long long *occ_base, unsigned long long pos_base, long long ngo, long long ngi,
-              const ExpandLateArgs late)
+              const ExpandLateArgs late, long long any_tile, long long any_stride)
 {
+    const long long tile = ANY ? any_tile : kWarpTile, slot_stride = ANY ? any_stride : kWarpTile;
     typedef typename std::conditional<sizeof(SE) == 4, uint16_t, uint32_t>::type CE;
     constexpr bool LATE = CM != 0;
     extern __shared__ __align__(16) unsigned char esm[];
@@ -177,7 +178,7 @@ expand_kernel(const SE *__restrict__ slots, const uint32_t *__restrict__ tile_en
     unsigned long long mine = 0;
     for (long long q = r0; q < r1; ++q) {
         const uint32_t o = tile_out[t0 + q];
-        s_ent[q] = min(tile_ent[t0 + q], uint32_t(kWarpTile));
+        s_ent[q] = min(tile_ent[t0 + q], uint32_t(slot_stride));
         s_off[q] = o;  // the tile's own total, replaced by its offset below
         mine += o;
     }
@@ -240,7 +241,7 @@ expand_kernel(const SE *__restrict__ slots, const uint32_t *__restrict__ tile_en
     // loads of the next item are in flight while the current one is written.
     auto load = [&](SE (&x)[R], long long qq, uint32_t gg) {
         const uint32_t ent = s_ent[qq];
-        const SE *src = slots + (t0 + qq) * kWarpTile;
+        const SE *src = slots + (t0 + qq) * slot_stride;
 #pragma unroll
         for (int u = 0; u < R; ++u) {
             const uint32_t j = gg + u * 32 + lane;
@@ -280,7 +281,7 @@ expand_kernel(const SE *__restrict__ slots, const uint32_t *__restrict__ tile_en
 #pragma unroll
             for (int u = 0; u < R; ++u) w[u] = (SE)0;
         }
-        const uint32_t tile0 = uint32_t(pos_base + (unsigned long long)(t0 + q) * kWarpTile);
+        const uint32_t tile0 = uint32_t(pos_base + (unsigned long long)(t0 + q) * (unsigned long long)tile);
 #pragma unroll
         for (int u = 0; u < R; ++u) {
             const uint32_t row = g0 + u * 32;
@@ -885,6 +886,10 @@ int ac_enqueue(const AcTables &t, const DevAc &dv, const uint8_t *d_text, int64_
         return PM_OK;
     }
 
+    if (dv.dg)
+        return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, nterms, se, 1,
+                              occ_base, pos_base, st);
+
     // list mode has its own layout (with late ids: no counters, maybe more warps)
     const bool late = list && !pfac && dv.ids_smem == 2;
     const int var = list ? dv.variant_list : dv.variant;
@@ -988,18 +993,20 @@ void list_workspace_parts(void *d_ws, int64_t nsub, int64_t nterms, int slot_ent
     out.slots = w + L.slots;
     const long long segs = ac_segments(nsub, dp.sm_count);
     out.seg_tiles = (nsub + segs - 1) / segs;
+    out.segs = segs;
 }
 
-int expand_launch(void *d_ws, int64_t nsub, int64_t nterms, int slot_entry_bytes, const uint32_t *grp_off,
-                  const uint32_t *grp_ids, int64_t n_grp_off, int64_t n_grp_ids, uint64_t *d_occ,
-                  int64_t occ_cap, int64_t *d_n_occ, const unsigned long long *occ_base,
-                  unsigned long long pos_base, void *stream, const ExpandLate *late)
+namespace {
+
+// one launch of the expand kernel over slots of any tile length (late: the
+// late-ids form, with the workspace whose counters it adds to)
+int expand_enqueue(const ExpandTiles &tl, const uint32_t *grp_off, const uint32_t *grp_ids, int64_t n_grp_off,
+                   int64_t n_grp_ids, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ,
+                   const unsigned long long *occ_base, unsigned long long pos_base, cudaStream_t st,
+                   const ExpandLate *late, void *late_ws)
 {
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    ListParts P;
-    list_workspace_parts(d_ws, nsub, nterms, slot_entry_bytes, P);
-    const long long seg_tiles = P.seg_tiles;
-    const long long nseg = (nsub + seg_tiles - 1) / seg_tiles;
+    const long long seg_tiles = tl.seg_tiles;
+    const long long nseg = (tl.ntiles + seg_tiles - 1) / seg_tiles;
     // shared memory of the expand kernel: 12 bytes per tile of a segment
     // (above 48 KB only for texts of more than about 3 GB), then, while two
     // CTAs still fit an SM: with late ids canon, the match bitmap and its
@@ -1012,7 +1019,6 @@ int expand_launch(void *d_ws, int64_t nsub, int64_t nterms, int slot_entry_bytes
     if (rc) return rc;
     const long long per_cta = std::min<long long>((long long)dp.smem_per_sm / 2 - 2048, dp.smem_optin - 1024);
     long long esmem = (seg_tiles + 1) * 8 + seg_tiles * 4;
-    const bool se4 = slot_entry_bytes == 4;
     ExpandLateArgs la{};
     const bool is_late = late && late->canon;
     if (is_late) {
@@ -1021,17 +1027,18 @@ int expand_launch(void *d_ws, int64_t nsub, int64_t nterms, int slot_entry_bytes
         la.rank = late->rank;
         la.nterms = late->nterms;
         la.nwords = late->nwords;
-        la.ccount = reinterpret_cast<unsigned long long *>(static_cast<char *>(d_ws) + kWsHeader);
+        la.ccount = reinterpret_cast<unsigned long long *>(static_cast<char *>(late_ws) + kWsHeader);
         la.counts = reinterpret_cast<long long *>(late->counts);
-        la.ws = static_cast<dev::WsHeader *>(d_ws);
-        const int ceb = se4 ? 2 : 4;
+        la.ws = static_cast<dev::WsHeader *>(late_ws);
+        const int ceb = tl.slot_kind == 0 ? 2 : 4;
         const long long cb = r16(late->nterms * ceb) + r16(late->nwords * 4) + r16((late->nwords + 1) * ceb);
         const long long x32 = cb + r16(late->nterms * 4), x16 = cb + r16((late->nterms + 1) / 2 * 4);
         la.smem = esmem + x32 <= per_cta ? 1 : esmem + x16 <= per_cta ? 2 : 0;
         esmem += la.smem == 1 ? x32 : la.smem == 2 ? x16 : 0;
     }
     const long long grp_bytes = (n_grp_off + n_grp_ids) * 4;
-    const bool grp_smem = n_grp_off > 0 && (grp_bytes <= (16 << 10) || esmem + grp_bytes <= per_cta);
+    const bool grp_smem =
+        tl.slot_kind != 2 && n_grp_off > 0 && (grp_bytes <= (16 << 10) || esmem + grp_bytes <= per_cta);
     const long long ngo = grp_smem ? n_grp_off : 0, ngi = grp_smem ? n_grp_ids : 0;
     esmem += (ngo + ngi) * 4;
     long long *n_occ = reinterpret_cast<long long *>(d_n_occ);
@@ -1040,32 +1047,68 @@ int expand_launch(void *d_ws, int64_t nsub, int64_t nterms, int slot_entry_bytes
             const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(esmem));
             if (ea != cudaSuccess) return ea;
         }
-        kern<<<unsigned(nseg), kExpandThreads, size_t(esmem), st>>>(slots, P.tile_ent, P.tile_out, P.seg_sum, nseg,
-                                                                   seg_tiles, nsub, grp_off, grp_ids, occ, cap, n_occ,
-                                                                   occ_base, pos_base, ngo, ngi, la);
+        kern<<<unsigned(nseg), kExpandThreads, size_t(esmem), st>>>(
+            slots, tl.tile_ent, tl.tile_out, tl.seg_sum, nseg, seg_tiles, tl.ntiles, grp_off, grp_ids, occ, cap, n_occ,
+            occ_base, pos_base, ngo, ngi, la, tl.tile, tl.slot_stride);
         return cudaGetLastError();
     };
+    const bool any = tl.tile != kWarpTile || tl.slot_stride != kWarpTile;  // never with late ids
     const int cm = !is_late ? 0 : la.smem == 1 ? 1 : la.smem == 2 ? 2 : 3;
     // one instance per slot width, counter mode and group-table placement
     auto pick = [&](auto se_tag) -> cudaError_t {
         typedef decltype(se_tag) SE;
         constexpr int sh = sizeof(SE) == 4 ? 16 : 32;
         constexpr uint32_t grp = sizeof(SE) == 4 ? 0x8000u : 0x80000000u;
-        const SE *sl = static_cast<const SE *>(P.slots);
-        switch (cm * 2 + (grp_smem ? 1 : 0)) {
-            case 0: return go(expand_kernel<SE, sh, grp, 0, false>, sl);
-            case 1: return go(expand_kernel<SE, sh, grp, 0, true>, sl);
-            case 2: return go(expand_kernel<SE, sh, grp, 1, false>, sl);
-            case 3: return go(expand_kernel<SE, sh, grp, 1, true>, sl);
-            case 4: return go(expand_kernel<SE, sh, grp, 2, false>, sl);
-            case 5: return go(expand_kernel<SE, sh, grp, 2, true>, sl);
-            case 6: return go(expand_kernel<SE, sh, grp, 3, false>, sl);
-            default: return go(expand_kernel<SE, sh, grp, 3, true>, sl);
+        const SE *sl = static_cast<const SE *>(tl.slots);
+        switch ((any ? 8 : cm * 2) + (grp_smem ? 1 : 0)) {
+            case 0: return go(expand_kernel<SE, sh, grp, 0, false, false>, sl);
+            case 1: return go(expand_kernel<SE, sh, grp, 0, true, false>, sl);
+            case 2: return go(expand_kernel<SE, sh, grp, 1, false, false>, sl);
+            case 3: return go(expand_kernel<SE, sh, grp, 1, true, false>, sl);
+            case 4: return go(expand_kernel<SE, sh, grp, 2, false, false>, sl);
+            case 5: return go(expand_kernel<SE, sh, grp, 2, true, false>, sl);
+            case 6: return go(expand_kernel<SE, sh, grp, 3, false, false>, sl);
+            case 7: return go(expand_kernel<SE, sh, grp, 3, true, false>, sl);
+            case 8: return go(expand_kernel<SE, sh, grp, 0, false, true>, sl);
+            default: return go(expand_kernel<SE, sh, grp, 0, true, true>, sl);
         }
     };
-    const cudaError_t e = se4 ? pick(uint32_t(0)) : pick(0ull);
+    cudaError_t e;
+    if (tl.slot_kind == 2) e = go(expand_kernel<uint32_t, 20, 0u, 0, false, true>, static_cast<const uint32_t *>(tl.slots));
+    else e = tl.slot_kind == 0 ? pick(uint32_t(0)) : pick(0ull);
     if (e != cudaSuccess) { set_cuda_error(int(e)); cudaGetLastError(); return PM_ECUDA; }
     return PM_OK;
+}
+
+}  // namespace
+
+int expand_launch(void *d_ws, int64_t nsub, int64_t nterms, int slot_entry_bytes, const uint32_t *grp_off,
+                  const uint32_t *grp_ids, int64_t n_grp_off, int64_t n_grp_ids, uint64_t *d_occ,
+                  int64_t occ_cap, int64_t *d_n_occ, const unsigned long long *occ_base,
+                  unsigned long long pos_base, void *stream, const ExpandLate *late)
+{
+    ListParts P;
+    list_workspace_parts(d_ws, nsub, nterms, slot_entry_bytes, P);
+    ExpandTiles tl;
+    tl.tile = kWarpTile;
+    tl.slot_stride = kWarpTile;
+    tl.ntiles = nsub;
+    tl.seg_tiles = P.seg_tiles;
+    tl.slot_kind = slot_entry_bytes == 4 ? 0 : 1;
+    tl.slots = P.slots;
+    tl.tile_ent = P.tile_ent;
+    tl.tile_out = P.tile_out;
+    tl.seg_sum = P.seg_sum;
+    return expand_enqueue(tl, grp_off, grp_ids, n_grp_off, n_grp_ids, d_occ, occ_cap, d_n_occ, occ_base, pos_base,
+                          static_cast<cudaStream_t>(stream), late, d_ws);
+}
+
+int expand_tiles_launch(const ExpandTiles &tl, const uint32_t *grp_off, const uint32_t *grp_ids,
+                        int64_t n_grp_off, int64_t n_grp_ids, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ,
+                        const unsigned long long *occ_base, unsigned long long pos_base, void *stream)
+{
+    return expand_enqueue(tl, grp_off, grp_ids, n_grp_off, n_grp_ids, d_occ, occ_cap, d_n_occ, occ_base, pos_base,
+                          static_cast<cudaStream_t>(stream), nullptr, nullptr);
 }
 
 int64_t ac_workspace_bytes(const AcTables &t, int64_t n, bool list)

@@ -1,0 +1,606 @@
+// scan_gram.cu -- sampled-gram scan on sm_103a: one table lookup per s text
+// positions (the tables are described in gram.cpp).
+//
+// A warp takes rows of 512 text bytes, 16 per lane, two rows per load batch
+// with the next batch in flight. The lane's 16 characters become one 32-bit
+// word of 2-bit codes (one multiply-add per 4 bytes); with the next lane's
+// word that gives the gram at any offset by one funnel shift, and its hash by
+// one multiply. A filter bit in shared memory drops almost every gram. No
+// lookup depends on another one, so a lane has 16 / s of them in flight: the
+// walk of the transition table, by contrast, is one dependent shared-memory
+// access per character.
+//
+// Grams that pass are packed into the warp's queue in text order and taken 32
+// at a time: bucket, entries, byte comparison with the text (which also
+// settles bytes outside the alphabet). The matches of a tile go to its slot
+// in text order, and the expand kernel of the other scans writes the keys.
+//
+// Bound: instruction issue (54-78 % of the issue slots; DRAM 20-40 % of its
+// peak). 256 MiB of EST-shaped text, list mode, this scan against the one
+// it replaces: 20,000 32-mers 0.10 ms (s = 16) against 1.64 (hybrid
+// transition table), 100,000 32-mers 0.20 against 2.46, 8,000 16-mers
+// compiled as Wu-Manber 0.13 (s = 4) against 2.10, 8,000 patterns of 8-16
+// characters 0.71 (s = 1) against 1.41; counts of 1,000 16-mers 0.075 (s =
+// 8) against 0.18.
+#include <type_traits>
+
+#include "scan_common.cuh"
+
+namespace pm {
+namespace {
+
+using dev::kFull;
+
+constexpr int kRow = 512;        // text bytes per warp row
+constexpr int kMaxWarps = 32;
+
+// rows per load batch: enough bytes in flight, at most 16 grams a lane
+__host__ __device__ constexpr int rows_of(int s) { return s >= 8 ? 4 : s >= 2 ? 2 : 1; }
+// the shortest tile, whole batches and at least kWarpTile bytes
+__host__ __device__ constexpr int min_tile(int s) { return s >= 8 ? 4096 : 3072; }
+
+struct GramArgs {
+    const uint8_t *text;
+    long long n;
+    int aligned;
+    uint32_t K[4];
+    int fshift, wshift, bshift;   // 32 - fb, 32 - (fb - 5), 32 - db
+    int fwords;                   // filter words
+    const uint32_t *filter_g;
+    const uint32_t *rank_g;
+    const uint32_t *dir;
+    const uint4 *ent;
+    const uint32_t *pats;
+    int pw;
+    const uint32_t *code;
+    const uint32_t *grp_off, *grp_ids;
+    int ncodes;
+    int tile;                     // text bytes per tile (a multiple of kRow * rows_of(S))
+    long long ntiles;
+    int list, hist_smem;
+    int slot_kind;                // 0: (off << 16) | code16, 1: (off << 32) | code, 2: (off << 20) | r
+    long long slot_stride;        // entries per tile
+    void *slots;
+    uint32_t *tile_ent, *tile_out;
+    unsigned long long *seg_sum;
+    long long seg_tiles;
+    long long *counts;
+    long long *n_occ;
+};
+
+__host__ __device__ constexpr int qcap(int s) { return 32 + rows_of(s) * kRow / s; }
+
+// bytes [off, off + 16) of the text, zeros from n on
+__device__ __forceinline__ uint4 load16(const GramArgs &a, long long off)
+{
+    if (a.aligned && off + 16 <= a.n) return __ldg(reinterpret_cast<const uint4 *>(a.text + off));
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (off + 20 <= a.n) {
+        // unaligned text: five aligned words (the last one ends inside the text)
+        const uint8_t *p = a.text + off;
+        const uint32_t sh = uint32_t(reinterpret_cast<uintptr_t>(p) & 3u) * 8u;
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(p - (sh >> 3));
+        if (off >= 3) {
+            const uint32_t w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3), w4 = __ldg(w + 4);
+            v.x = __funnelshift_r(w0, w1, sh);
+            v.y = __funnelshift_r(w1, w2, sh);
+            v.z = __funnelshift_r(w2, w3, sh);
+            v.w = __funnelshift_r(w3, w4, sh);
+            return v;
+        }
+    }
+    uint32_t b[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+        if (off + j < a.n) b[j >> 2] |= uint32_t(a.text[off + j]) << (8 * (j & 3));
+    return make_uint4(b[0], b[1], b[2], b[3]);
+}
+
+// the 2-bit codes (byte >> 1) & 3 of 16 bytes, first character lowest: the
+// multiply gathers a word's four codes in its top byte
+__device__ __forceinline__ uint32_t pack16(const uint4 &v)
+{
+    constexpr uint32_t M = 0x06060606u, G = 0x00820820u;
+    const uint32_t p0 = (v.x & M) * G, p1 = (v.y & M) * G, p2 = (v.z & M) * G, p3 = (v.w & M) * G;
+    return __byte_perm(__byte_perm(p0, p1, 0x0073), __byte_perm(p2, p3, 0x0073), 0x5410);
+}
+
+// pattern bytes against the text at p; `room`: whole words around them lie
+// inside the text
+__device__ __forceinline__ bool same_bytes(const uint8_t *p, int len, const uint32_t *pat, bool room)
+{
+    if (room) {
+        const uint32_t lead = uint32_t(reinterpret_cast<uintptr_t>(p) & 3u), sh = lead * 8u;
+        const uint32_t *w = reinterpret_cast<const uint32_t *>(p - lead);
+        uint32_t cur = __ldg(w);
+        for (int left = len; left > 0; left -= 4) {
+            const uint32_t nxt = __ldg(++w);
+            uint32_t x = __funnelshift_r(cur, nxt, sh) ^ __ldg(pat++);
+            if (left < 4) x &= (1u << (8 * left)) - 1u;
+            if (x) return false;
+            cur = nxt;
+        }
+        return true;
+    }
+    for (int j = 0; j < len; ++j)
+        if (p[j] != uint8_t(__ldg(pat + (j >> 2)) >> (8 * (j & 3)))) return false;
+    return true;
+}
+
+// S: stride; QW: 0 2-bit grams, else words of a byte gram; RANK: buckets by
+// rank in the filter (the queue holds (offset << 18) | gram), else by hash
+// (offsets and hashes side by side).
+template <int S, int QW, bool RANK>
+__global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const GramArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int NP = 16 / S;       // probes per lane and row
+    constexpr int R = rows_of(S);
+    constexpr int QCAP = qcap(S);
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+
+    uint32_t *s_filter = reinterpret_cast<uint32_t *>(smem);
+    uint32_t *s_rank = s_filter + ((a.fwords + 3) & ~3);
+    uint32_t *s_hist = s_rank + (RANK ? (a.fwords + 3) & ~3 : 0);
+    uint32_t *q32 = s_hist + (a.hist_smem ? (a.ncodes + 3) & ~3 : 0) + warp * (RANK ? QCAP : QCAP + QCAP / 2);
+    uint16_t *q16 = reinterpret_cast<uint16_t *>(q32 + QCAP);
+
+    {   // the tables are padded to 16 bytes
+        uint4 *f4 = reinterpret_cast<uint4 *>(s_filter), *r4 = reinterpret_cast<uint4 *>(s_rank);
+        for (int i = threadIdx.x; i < (a.fwords + 3) / 4; i += blockDim.x) {
+            f4[i] = __ldg(reinterpret_cast<const uint4 *>(a.filter_g) + i);
+            if (RANK) r4[i] = __ldg(reinterpret_cast<const uint4 *>(a.rank_g) + i);
+        }
+    }
+    if (a.hist_smem)
+        for (int i = threadIdx.x; i < a.ncodes; i += blockDim.x) s_hist[i] = 0u;
+    __syncthreads();
+
+    const uint32_t ntiles = uint32_t(a.ntiles);
+    const uint32_t G = gridDim.x * (blockDim.x >> 5);
+    const int ngroups = a.tile / (kRow * R);
+    uint32_t st = blockIdx.x * (blockDim.x >> 5) + warp;
+    unsigned long long my_total = 0;
+    const uint32_t K0 = a.K[0];
+
+    uint4 v[R + 1];                  // a batch's rows, and the 16 bytes after them (lane 0)
+    auto load = [&](uint32_t t, int g) {
+        const long long base = (long long)t * a.tile + g * (kRow * R);
+        if (a.aligned && base + kRow * R + 16 <= a.n) {
+            const uint4 *p = reinterpret_cast<const uint4 *>(a.text + base) + lane;
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = __ldg(p + 32 * r);
+            if (lane == 0) v[R] = __ldg(p + 32 * R);
+        } else {
+#pragma unroll
+            for (int r = 0; r <= R; ++r)
+                if (r < R || lane == 0) v[r] = load16(a, base + lane * 16 + r * kRow);
+        }
+    };
+    if (st < ntiles) load(st, 0);
+    int g = 0;
+    uint32_t ent = 0, outs = 0;      // the tile's entries (uniform) and this lane's keys
+    uint32_t qn = 0;                 // queue length (uniform)
+
+    while (st < ntiles) {
+        const bool last = g + 1 == ngroups;
+        const uint32_t stn = last ? st + G : st;
+        const int gn = last ? 0 : g + 1;
+
+        // ---- the batch's grams: hash, and the word that names the bit ----
+        uint32_t lo[R], hi[R];           // 2-bit grams: 16 characters and the 16 after them
+        uint32_t H[QW == 0 ? 1 : R * NP];
+        if (QW == 0) {
+            uint32_t c[R + 1];
+#pragma unroll
+            for (int r = 0; r <= R; ++r) c[r] = pack16(v[r]);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                lo[r] = c[r];
+                hi[r] = __shfl_sync(kFull, lane == 0 ? c[r + 1] : c[r], (lane + 1) & 31);
+            }
+        } else {
+            constexpr int NX = (16 - S + 4 * QW - 1) / 4 - 3;  // words of the next lane a gram may reach
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                uint32_t x[8];
+                x[0] = v[r].x; x[1] = v[r].y; x[2] = v[r].z; x[3] = v[r].w;
+                if (NX > 0) x[4] = __shfl_sync(kFull, lane == 0 ? v[r + 1].x : v[r].x, (lane + 1) & 31);
+                if (NX > 1) x[5] = __shfl_sync(kFull, lane == 0 ? v[r + 1].y : v[r].y, (lane + 1) & 31);
+                if (NX > 2) x[6] = __shfl_sync(kFull, lane == 0 ? v[r + 1].z : v[r].z, (lane + 1) & 31);
+                if (NX > 3) x[7] = __shfl_sync(kFull, lane == 0 ? v[r + 1].w : v[r].w, (lane + 1) & 31);
+#pragma unroll
+                for (int k = 0; k < NP; ++k) {
+                    uint32_t h = 0u;
+#pragma unroll
+                    for (int j = 0; j < QW; ++j) {
+                        const int o = S * k + 4 * j;
+                        const uint32_t y = (o & 3) == 0 ? x[o >> 2]
+                                                        : __funnelshift_r(x[o >> 2], x[(o >> 2) + 1], 8 * (o & 3));
+                        h += y * a.K[j];
+                    }
+                    H[QW == 0 ? 0 : r * NP + k] = h;
+                }
+            }
+        }
+        // the rows are in registers as grams: the next batch's loads
+        if (stn < ntiles) load(stn, gn);
+
+        // ---- a filter bit per probe, the first one lowest ----
+        uint32_t mask[R], any = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            uint32_t m = 0;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) {
+                const uint32_t win = QW == 0 ? (k == 0 ? lo[r] : __funnelshift_r(lo[r], hi[r], 2 * S * k))
+                                             : H[QW == 0 ? 0 : r * NP + k];
+                const uint32_t h = QW == 0 ? win * K0 : win;
+                const uint32_t w = s_filter[h >> a.wshift];
+                m = __funnelshift_r(m, __funnelshift_r(w, 0u, win), 1);  // bit `win mod 32` of w, appended
+            }
+            mask[r] = m >> (32 - NP);
+            any |= mask[r];
+        }
+        // ---- passing grams -> queue, row by row, lane by lane (text order) ----
+        if (__any_sync(kFull, any != 0u)) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                uint32_t m = mask[r], at = qn;
+                if (NP <= 2) {
+#pragma unroll
+                    for (int k = 0; k < NP; ++k) {
+                        const uint32_t bal = __ballot_sync(kFull, (m >> k) & 1u);
+                        at += __popc(bal & lt);
+                        qn += __popc(bal);
+                    }
+                } else {
+                    const uint32_t cnt = __popc(m);
+                    const uint32_t inc = dev::warp_incl_scan(cnt, lane);
+                    at += inc - cnt;
+                    qn += __shfl_sync(kFull, inc, 31);
+                }
+                const uint32_t off0 = uint32_t(g * R + r) * kRow + uint32_t(lane) * 16u;
+                if (QW == 0 && NP > 1) {
+                    while (m) {
+                        const uint32_t k = uint32_t(__ffs(int(m))) - 1u;
+                        m &= m - 1u;
+                        const uint32_t h = __funnelshift_r(lo[r], hi[r], 2 * S * k) * K0;
+                        if (RANK) {
+                            q32[at] = ((off0 + S * k) << 18) | (h >> a.fshift);
+                        } else {
+                            q32[at] = h;
+                            q16[at] = uint16_t(off0 + S * k);
+                        }
+                        ++at;
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < NP; ++k)
+                        if ((m >> k) & 1u) {
+                            const uint32_t h = QW == 0 ? lo[r] * K0 : H[QW == 0 ? 0 : r * NP + k];
+                            if (RANK) {
+                                q32[at] = ((off0 + S * k) << 18) | (h >> a.fshift);
+                            } else {
+                                q32[at] = h;
+                                q16[at] = uint16_t(off0 + S * k);
+                            }
+                            ++at;
+                        }
+                }
+            }
+            __syncwarp();
+        }
+        // ---- full batches of 32 (at the tile's end the rest too) ----
+        if (qn >= 32u || (last && qn > 0u)) {
+            const long long tile0 = (long long)st * a.tile;
+            const uint8_t *tp = a.text + tile0;
+            // starts relative to the tile, inside the text
+            const int low = tile0 == 0 ? 0 : -S;
+            const int rem = int(min(a.n - tile0, 1LL << 30));
+            int done = 0;
+            do {
+                const int i = done + lane;
+                uint32_t e0 = 0, e1 = 0, h = 0, off = 0;
+                if (i < int(qn)) {
+                    h = q32[i];
+                    uint32_t bk;
+                    if (RANK) {
+                        off = h >> 18;
+                        const uint32_t b = h & 0x3FFFFu;
+                        h = b << a.fshift;
+                        bk = s_rank[b >> 5] + __popc(s_filter[b >> 5] & ((1u << (b & 31u)) - 1u));
+                    } else {
+                        off = q16[i];
+                        bk = h >> a.bshift;
+                    }
+                    e0 = __ldg(a.dir + bk);
+                    e1 = __ldg(a.dir + bk + 1);
+                }
+                done += 32;
+                // does entry e match here?
+                auto match = [&](const uint4 &en) -> bool {
+                    const int start = int(off) - int(en.z & 255u), len = int(en.z >> 8);
+                    if (en.x != h || start < low || start + len > rem) return false;
+                    const bool room = start >= low + 3 && start + ((len + 3) & ~3) + 4 <= rem;
+                    return same_bytes(tp + start, len, a.pats + (size_t)en.y * a.pw, room);
+                };
+                // matches of this lane's gram: counted, then written behind
+                // those of the lanes before it
+                uint32_t nh = 0, val = 0, mark = 0;
+                for (uint32_t e = e0; e < e1; ++e) {
+                    const uint4 en = __ldg(a.ent + e);
+                    if (!match(en)) continue;
+                    uint32_t mult = 1u;
+                    if (a.hist_smem) atomicAdd(&s_hist[en.y], 1u);
+                    if (en.w & 0x80000000u) {
+                        const uint32_t gi = en.w & 0x7FFFFFFFu;
+                        const uint32_t j0 = __ldg(a.grp_off + gi), j1 = __ldg(a.grp_off + gi + 1);
+                        mult = j1 - j0;
+                        if (!a.hist_smem)
+                            for (uint32_t j = j0; j < j1; ++j)
+                                atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + __ldg(a.grp_ids + j), 1ull);
+                    } else if (!a.hist_smem) {
+                        atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + en.w, 1ull);
+                    }
+                    outs += mult;
+                    if (nh == 0) {
+                        val = en.w;
+                        mark = en.z & 255u;
+                    }
+                    ++nh;
+                }
+                if (a.list && __any_sync(kFull, nh != 0u)) {
+                    uint32_t k = ent;
+                    if (__any_sync(kFull, nh > 1u)) {
+                        const uint32_t inc = dev::warp_incl_scan(nh, lane);
+                        k += inc - nh;
+                        ent += __shfl_sync(kFull, inc, 31);
+                    } else {
+                        const uint32_t bal = __ballot_sync(kFull, nh != 0u);
+                        k += __popc(bal & lt);
+                        ent += __popc(bal);
+                    }
+                    auto put = [&](uint32_t gk, uint32_t code) {
+                        // start in the tile, shifted by S - 1 so that it is never negative
+                        const uint32_t o = off + uint32_t(S - 1) - gk;
+                        const long long p = (long long)st * a.slot_stride + k;
+                        if (a.slot_kind == 0)
+                            static_cast<uint32_t *>(a.slots)[p] = (o << 16) | ((code >> 16) & 0x8000u) | (code & 0x7FFFu);
+                        else if (a.slot_kind == 1)
+                            static_cast<unsigned long long *>(a.slots)[p] = ((unsigned long long)o << 32) | code;
+                        else
+                            static_cast<uint32_t *>(a.slots)[p] = (o << 20) | code;
+                        ++k;
+                    };
+                    if (nh == 1u) {
+                        put(mark, val);
+                    } else if (nh > 1u) {
+                        for (uint32_t e = e0; e < e1; ++e) {
+                            const uint4 en = __ldg(a.ent + e);
+                            if (match(en)) put(en.z & 255u, en.w);
+                        }
+                    }
+                }
+            } while (int(qn) - done >= 32 || (last && int(qn) - done > 0));
+            // the rest (fewer than 32) moves to the front
+            const int left = max(int(qn) - done, 0);
+            uint32_t h = 0, o = 0;
+            if (lane < left) {
+                h = q32[done + lane];
+                if (!RANK) o = q16[done + lane];
+            }
+            __syncwarp();
+            if (lane < left) {
+                q32[lane] = h;
+                if (!RANK) q16[lane] = uint16_t(o);
+            }
+            __syncwarp();
+            qn = uint32_t(left);
+        }
+        if (last) {
+            if (a.list) {
+                uint32_t o_tot = outs;
+                if (ent != 0u) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) o_tot += __shfl_xor_sync(kFull, o_tot, o);
+                }
+                if (lane == 0) {
+                    a.tile_ent[st] = ent;
+                    a.tile_out[st] = o_tot;
+                    if (o_tot) atomicAdd(&a.seg_sum[st / uint32_t(a.seg_tiles)], (unsigned long long)o_tot);
+                }
+            } else {
+                my_total += outs;
+            }
+            ent = 0;
+            outs = 0;
+        }
+        st = stn;
+        g = gn;
+    }
+
+    if (!a.list) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) my_total += __shfl_down_sync(kFull, my_total, o);
+        if (lane == 0 && my_total) atomicAdd(reinterpret_cast<unsigned long long *>(a.n_occ), my_total);
+    }
+    if (!a.hist_smem) return;
+    __syncthreads();
+    for (int c = threadIdx.x; c < a.ncodes; c += blockDim.x) {
+        const uint32_t x = s_hist[c];
+        if (!x) continue;
+        const uint32_t code = __ldg(a.code + c);
+        if (code & 0x80000000u) {
+            const uint32_t gi = code & 0x7FFFFFFFu;
+            for (uint32_t j = a.grp_off[gi]; j < a.grp_off[gi + 1]; ++j)
+                atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + a.grp_ids[j], (unsigned long long)x);
+        } else {
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + code, (unsigned long long)x);
+        }
+    }
+}
+
+typedef void (*GramKernel)(const GramArgs);
+
+template <int QW, bool RANK>
+GramKernel by_stride(int s)
+{
+    switch (s) {
+    case 1: return gram_scan_kernel<1, QW, RANK>;
+    case 2: return gram_scan_kernel<2, QW, RANK>;
+    case 4: return gram_scan_kernel<4, QW, RANK>;
+    case 8: return gram_scan_kernel<8, QW, RANK>;
+    default: return gram_scan_kernel<16, QW, RANK>;
+    }
+}
+
+GramKernel kernel_of(const GramTables &t)
+{
+    switch (t.qw) {
+    case 0: return t.rank ? by_stride<0, true>(t.s) : by_stride<0, false>(t.s);
+    case 1: return by_stride<1, false>(t.s);
+    case 2: return by_stride<2, false>(t.s);
+    case 3: return by_stride<3, false>(t.s);
+    default: return by_stride<4, false>(t.s);
+    }
+}
+
+long long up4(long long x) { return (x + 3) & ~3LL; }
+
+long long table_words(const GramTables &t)
+{
+    return up4((long long)t.filter.size()) * (t.rank ? 2 : 1);
+}
+
+long long queue_words(const GramTables &t) { return t.rank ? qcap(t.s) : qcap(t.s) + qcap(t.s) / 2; }
+
+}  // namespace
+
+int gram_plan(const GramTables &t, const DeviceProps &dp, DevGram &dev)
+{
+    dev.use = false;
+    if (!t.ok) return PM_OK;
+    const long long budget = (long long)dp.smem_optin - 1024;
+    const long long nc = (long long)t.code.size();
+    // counters in shared memory if they fit beside 24 warps' queues
+    for (int hist : {1, 0})
+        for (int w : {32, 24, 16}) {
+            const long long need = 4 * (table_words(t) + (hist ? up4(nc) : 0) + w * queue_words(t));
+            if (need > budget || (hist && w < 24)) continue;
+            dev.warps = w;
+            dev.hist_smem = hist;
+            dev.use = true;
+            return PM_OK;
+        }
+    return PM_OK;
+}
+
+int gram_slot_bytes(const GramTables &t)
+{
+    if (t.var) return t.d <= (1 << 20) ? 4 : 8;
+    return t.d < 32768 ? 4 : 8;
+}
+
+int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, int64_t n, bool list,
+                int64_t *d_counts, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ, const GramWs &ws,
+                const unsigned long long *occ_base, unsigned long long pos_base, void *stream)
+{
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    DeviceProps dp;
+    int rc = device_props(dp);
+    if (rc) return rc;
+    GramArgs a;
+    a.text = d_text;
+    a.n = n;
+    a.aligned = (reinterpret_cast<uintptr_t>(d_text) & 15) == 0;
+    for (int j = 0; j < 4; ++j) a.K[j] = t.K[j];
+    a.fshift = 32 - t.fb;
+    a.wshift = 37 - t.fb;
+    a.bshift = 32 - t.db;
+    a.fwords = int(t.filter.size());
+    a.filter_g = dv.filter;
+    a.rank_g = dv.rank_base;
+    a.dir = dv.dir;
+    a.ent = static_cast<const uint4 *>(dv.ent);
+    a.pats = dv.pats;
+    a.pw = t.pw;
+    a.code = dv.code;
+    a.grp_off = dv.grp_off;
+    a.grp_ids = dv.grp_ids;
+    a.ncodes = int(t.code.size());
+    a.list = list ? 1 : 0;
+    a.hist_smem = dv.hist_smem;
+    a.counts = reinterpret_cast<long long *>(d_counts);
+    a.n_occ = reinterpret_cast<long long *>(d_n_occ);
+    // Tiles: long ones waste fewer lanes on a tile's last batch, short ones
+    // spread a short text over the SMs. The workspace holds one count per
+    // kWarpTile bytes, so a tile is longer than that; a mixed-length slot has
+    // 12 bits for the start, a ranked gram's queue entry 14.
+    int warps = dv.warps;
+    const long long lanes = (long long)dp.sm_count * warps;
+    int tile = min_tile(t.s);
+    static_assert(min_tile(1) >= kWarpTile && min_tile(8) >= kWarpTile, "one count per kWarpTile bytes");
+    const int most = t.var ? tile : 2 * 4096;
+    while (2 * tile <= most && (n + 2 * tile - 1) / (2 * tile) >= lanes) tile *= 2;
+    a.tile = tile;
+    a.ntiles = (n + tile - 1) / tile;
+    const int per_pos = t.var ? ws.per_pos : 1;
+    const int se = gram_slot_bytes(t);
+    a.slot_kind = se == 8 ? 1 : t.var ? 2 : 0;
+    a.slot_stride = (long long)tile * per_pos;
+    a.slots = ws.slots;
+    a.tile_ent = ws.tile_ent;
+    a.tile_out = ws.tile_out;
+    a.seg_sum = ws.seg_sum;
+    a.seg_tiles = (a.ntiles + ws.segs - 1) / ws.segs;
+
+    const GramKernel fn = kernel_of(t);
+    // a short text: fewer warps per CTA, spread over every SM (at least 8,
+    // which load the tables)
+    const long long spread = (a.ntiles + dp.sm_count - 1) / dp.sm_count;
+    if (spread < warps) warps = int(spread < 8 ? 8 : spread);
+    const long long smem = 4 * (table_words(t) + (dv.hist_smem ? up4(a.ncodes) : 0) + (long long)warps * queue_words(t));
+    rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), smem);
+    if (rc) return rc;
+    long long grid = dp.sm_count;
+    const long long want = (a.ntiles + warps - 1) / warps;
+    if (want < grid) grid = want;
+    fn<<<dim3(unsigned(grid)), dim3(unsigned(warps * 32)), size_t(smem), st>>>(a);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
+    if (!list) return PM_OK;
+    ExpandTiles tl;
+    tl.tile = tile;
+    tl.slot_stride = a.slot_stride;
+    tl.ntiles = a.ntiles;
+    tl.seg_tiles = a.seg_tiles;
+    tl.slot_kind = a.slot_kind;
+    tl.slots = ws.slots;
+    tl.tile_ent = ws.tile_ent;
+    tl.tile_out = ws.tile_out;
+    tl.seg_sum = ws.seg_sum;
+    return expand_tiles_launch(tl, dv.grp_off, dv.grp_ids, (int64_t)t.grp_off.size(), (int64_t)t.grp_ids.size(),
+                               d_occ, occ_cap, d_n_occ, occ_base, pos_base - (unsigned long long)(t.s - 1), stream);
+}
+
+int gram_launch_ws(const GramTables &t, const DevGram &dv, const uint8_t *d_text, int64_t n, bool list,
+                   int64_t *d_counts, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ, void *d_ws,
+                   int64_t nterms, int slot_bytes, int per_pos, const unsigned long long *occ_base,
+                   unsigned long long pos_base, void *stream)
+{
+    ListParts L;
+    list_workspace_parts(d_ws, warp_tiles(n), nterms, slot_bytes, L);
+    GramWs ws;
+    ws.tile_ent = L.tile_ent;
+    ws.tile_out = L.tile_out;
+    ws.seg_sum = L.seg_sum;
+    ws.slots = L.slots;
+    ws.segs = L.segs;
+    ws.per_pos = per_pos;
+    return gram_launch(t, dv, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, ws, occ_base, pos_base, stream);
+}
+
+}  // namespace pm

@@ -621,6 +621,10 @@ int wm_launch(const WmTables &t, const DevWm &dv, const uint8_t *d_text, int64_t
     if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
     if (n < t.m || ntiles == 0) return PM_OK;
 
+    if (dv.dg)
+        return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, 0, se * per_pos,
+                              per_pos, nullptr, 0, stream);
+
     typedef void (*K)(const WmArgs);
     const int nv = wm_nv(t.m);
     const bool wide = t.m > 16;

@@ -35,7 +35,7 @@ EXPORTED = [
     "pm_batch_set_warps", "pm_batch_set_placement", "pm_batch_placement", "pm_batch_capture", "pm_batch_replay",
     "pm_tune", "pm_server_create", "pm_server_submit", "pm_server_wait", "pm_server_get_stats",
     "pm_server_reset_stats", "pm_server_destroy",
-    "pm_selfcheck_host_walk", "pm_strerror", "pm_last_cuda_error", "pm_version",
+    "pm_selfcheck_host_walk", "pm_selfcheck_gram_walk", "pm_strerror", "pm_last_cuda_error", "pm_version",
 ]
 
 
@@ -196,6 +196,8 @@ def lib():
         L.pm_server_destroy.argtypes = [vp]
         L.pm_selfcheck_host_walk.restype = ctypes.c_int
         L.pm_selfcheck_host_walk.argtypes = [vp, vp, i64, ctypes.POINTER(ctypes.POINTER(pm_result))]
+        L.pm_selfcheck_gram_walk.restype = ctypes.c_int
+        L.pm_selfcheck_gram_walk.argtypes = [vp, vp, i64, ctypes.POINTER(ctypes.POINTER(pm_result))]
         L.pm_strerror.restype = ctypes.c_char_p
         L.pm_strerror.argtypes = [ctypes.c_int]
         L.pm_last_cuda_error.restype = ctypes.c_int
@@ -558,6 +560,14 @@ def pm_selfcheck_host_walk(h: int, T):
     rp = ctypes.POINTER(pm_result)()
     _check(lib().pm_selfcheck_host_walk(h, T.ctypes.data, T.size, ctypes.byref(rp)),
            "pm_selfcheck_host_walk")
+    return _take_result(rp)
+
+
+def pm_selfcheck_gram_walk(h: int, T):
+    T = np.ascontiguousarray(T, dtype=np.uint8)
+    rp = ctypes.POINTER(pm_result)()
+    _check(lib().pm_selfcheck_gram_walk(h, T.ctypes.data, T.size, ctypes.byref(rp)),
+           "pm_selfcheck_gram_walk")
     return _take_result(rp)
 
 

@@ -1,0 +1,77 @@
+"""GPU parity of the sampled-gram scan where it can go wrong: texts that end
+inside a row, a batch or a tile, unaligned texts, bytes outside the alphabet,
+every stride, list and counts, and texts in which every gram passes."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # collected on CPU-only machines, never run there
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1407_2889_gb300 import pmscan as pm  # noqa: E402
+
+THREADS = os.cpu_count() or 4
+
+
+def _check(s, T, want, off=0):
+    buf = torch.zeros(T.size + 16, dtype=torch.uint8, device="cuda")
+    d_text = buf[off:off + T.size]
+    d_text.copy_(torch.from_numpy(T))
+    occ, cnt = s.scan(d_text)
+    assert np.array_equal(occ, want[0]) and np.array_equal(cnt, want[1])
+    assert np.array_equal(s.scan(d_text, counts_only=True)[1], want[1])
+
+
+@pytest.mark.parametrize("alphabet", [b"ACGT", b"ACDEFGHIKLMNPQRSTVWY"])
+@pytest.mark.parametrize("m", [4, 8, 9, 10, 13, 16, 20, 31, 65])
+def test_text_ends(alphabet, m):
+    rng = np.random.default_rng(41 + m)
+    A = np.frombuffer(alphabet, np.uint8)
+    base = A[rng.integers(0, A.size, 40000)]
+    base[rng.integers(0, base.size, 300)] = ord("N")
+    P = A[rng.integers(0, A.size, (90, m))]
+    for r in range(0, 90, 2):
+        P[r] = base[r * 37:r * 37 + m]
+    P[5] = P[4]
+    s = pm.PatternSet.ac(P)
+    for n in (m, 511, 512, 513, 2047, 3072, 3073, 4096 + 15, 8192, 24575, 40000):
+        T = base[:n].copy()
+        T[n - m:] = P[4]  # an occurrence at the very end
+        for off in (0, 1, 6):
+            _check(s, T, oracle.dictionary(T, P, threads=THREADS), off)
+    s.close()
+
+
+@pytest.mark.parametrize("m", [8, 16, 32])
+def test_every_gram_passes(m):
+    T = np.full(70001, ord("A"), np.uint8)
+    P = np.full((3, m), ord("A"), np.uint8)
+    P[2, -1] = ord("C")
+    want = oracle.dictionary(T, P, threads=THREADS)
+    for s in (pm.PatternSet.ac(P), pm.PatternSet.wm(P, 2), pm.PatternSet.pfac(P)):
+        _check(s, T, want)
+        s.close()
+    V = [b"A" * k for k in range(max(4, m - 12), m + 1)]
+    want = oracle.dictionary_var(T, V, threads=THREADS)
+    for s in (pm.PatternSet.acv(V), pm.PatternSet.wmv(V, 2)):
+        _check(s, T, want)
+        s.close()
+
+
+@pytest.mark.parametrize("d,m", [(40000, 12), (70000, 24)])
+def test_wide_codes_and_device_counters(d, m):
+    rng = np.random.default_rng(d)
+    A = np.frombuffer(b"ACGT", np.uint8)
+    T = A[rng.integers(0, 4, 300000)]
+    P = A[rng.integers(0, 4, (d, m))]
+    P[::3] = T[(np.arange(0, d, 3) * 4)[:, None] + np.arange(m)[None, :]]
+    P[1] = P[0]
+    s = pm.PatternSet.ac(P)
+    _check(s, T, oracle.dictionary(T, P, threads=THREADS))
+    s.close()
