@@ -260,7 +260,7 @@ bool plan_is_automatic(const pm_set *s)
     const pm_params &p = s->params;
     if (s->algo == PM_ALGO_WM || s->algo == PM_ALGO_WMV) return p.warps_per_cta == 0 && p.ctas_per_sm == 0;
     return p.placement == PM_PLACE_AUTO && p.smem_table_bytes == 0 && p.warps_per_cta == 0 && p.ctas_per_sm == 0 &&
-           p.counters == 0 && p.ids_place == 0 && p.stride == 0;
+           p.counters == 0 && p.ids_place == 0 && p.stride <= 1;
 }
 
 int upload_gram(pm_set *s, const DeviceProps &dp)
@@ -279,7 +279,9 @@ int upload_gram(pm_set *s, const DeviceProps &dp)
         {t.pats.data(), t.pats.size() * 4, reinterpret_cast<void **>(&d.pats)},
         {t.code.data(), t.code.size() * 4, reinterpret_cast<void **>(&d.code)},
         {t.grp_off.data(), t.grp_off.size() * 4, reinterpret_cast<void **>(&d.grp_off)},
-        {t.grp_ids.data(), t.grp_ids.size() * 4, reinterpret_cast<void **>(&d.grp_ids)}};
+        {t.grp_ids.data(), t.grp_ids.size() * 4, reinterpret_cast<void **>(&d.grp_ids)},
+        {t.id_off.data(), t.id_off.size() * 2, reinterpret_cast<void **>(&d.id_off)},
+        {t.ids.data(), t.ids.size() * 2, reinterpret_cast<void **>(&d.ids)}};
     size_t total = 0;
     for (const auto &p : part) total += (p.bytes + 15) & ~size_t(15);
     try {
@@ -981,7 +983,7 @@ int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t
     s->dac = tried[bi].plan;  // same device tables, new launch plan
     s->dac2.use = false;
     s->params = tried[bi].params;
-    if (!s->dac.dg) s->params.stride = 1;
+    s->params.stride = 1;
     if (best_out) *best_out = s->params;
     if (best_ms) *best_ms = tried[bi].ms;
     return PM_OK;

@@ -171,6 +171,12 @@ struct GramTables {
     std::vector<uint32_t> pats;       // pw words per distinct pattern, zero padded
     std::vector<uint32_t> code;       // code of each distinct pattern
     std::vector<uint32_t> grp_off, grp_ids;
+    // Dense form (one-length sets of fewer than 2^15 patterns, s = 1, q = m):
+    // the gram is the pattern, so its rank is the distinct pattern's number,
+    // whose ids are ids[id_off[c] .. id_off[c + 1]). lut: the byte of code c in byte c.
+    bool dense = false;
+    uint32_t lut = 0;
+    std::vector<uint16_t> id_off, ids;
 };
 
 int build_ac(const uint8_t *P, int64_t d, int32_t m, AcTables &out);
@@ -223,7 +229,8 @@ struct DevGram {
     uint32_t *filter = nullptr, *rank_base = nullptr, *dir = nullptr;
     void *ent = nullptr;
     uint32_t *pats = nullptr, *code = nullptr, *grp_off = nullptr, *grp_ids = nullptr;
-    int32_t warps = 0, hist_smem = 0;
+    uint16_t *id_off = nullptr, *ids = nullptr;
+    int32_t warps = 0, hist_smem = 0, pair = 0;
     bool use = false;               // the tables fit this device
 };
 

@@ -159,44 +159,8 @@ expand_kernel(const SE *__restrict__ slots, const uint32_t *__restrict__ tile_en
     const long long nt = max(0LL, min(seg_tiles, nsub - t0));
     if (nt == 0 && !LATE) return;
 
-    // base of the segment: sum of the earlier segments
-    unsigned long long part = 0;
-    for (long long q = tid; q < seg; q += kExpandThreads) part += seg_sum[q];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
-    if (lane == 0) s_red[warp] = part;
-    __syncthreads();
-    // a chunk of a longer scan writes after the keys of the chunks before it
-    unsigned long long seg_base = occ_base ? *occ_base : 0ull;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) seg_base += s_red[w];
-    __syncthreads();
-
-    // per-tile offsets: each thread scans a run of consecutive tiles
-    const long long per = (nt + kExpandThreads - 1) / kExpandThreads;
-    const long long r0 = min(nt, (long long)tid * per), r1 = min(nt, r0 + per);
-    unsigned long long mine = 0;
-    for (long long q = r0; q < r1; ++q) {
-        const uint32_t o = tile_out[t0 + q];
-        s_ent[q] = min(tile_ent[t0 + q], uint32_t(slot_stride));
-        s_off[q] = o;  // the tile's own total, replaced by its offset below
-        mine += o;
-    }
-    unsigned long long inc = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long u = __shfl_up_sync(kFull, inc, o);
-        if (lane >= o) inc += u;
-    }
-    if (lane == 31) s_red[warp] = inc;
-    __syncthreads();
-    unsigned long long run = seg_base + inc - mine;
-    for (int w = 0; w < warp; ++w) run += s_red[w];
-    for (long long q = r0; q < r1; ++q) {
-        const unsigned long long o = s_off[q];
-        s_off[q] = run;
-        run += o;
-    }
+    const unsigned long long run = dev::segment_offsets<kExpandThreads>(tile_ent, tile_out, seg_sum, seg, t0, nt, occ_base,
+                                                                        uint32_t(slot_stride), s_off, s_ent, s_red);
     if (tid == kExpandThreads - 1 && nt > 0 && t0 + nt == nsub) *n_occ = (long long)run;  // the last tile's CTA
     // small group tables move to shared memory (GS): their loads sit on a
     // row's critical path

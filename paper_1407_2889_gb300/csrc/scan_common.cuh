@@ -138,5 +138,58 @@ __device__ __forceinline__ void count_pattern(uint32_t r, uint32_t *s_hist, long
     else atomicAdd(reinterpret_cast<unsigned long long *>(g_counts) + r, 1ull);
 }
 
+// Output offsets of a segment of nt warp tiles (from tile t0 on), by the whole
+// CTA of THREADS threads: s_off[q] gets the number of keys before tile t0 + q
+// (those of the segments before this one, number seg, and *base included),
+// s_ent[q] its entries (at most max_ent). Returns, on the last thread, the
+// keys up to the segment's end. s_red: THREADS / 32 words.
+template <int THREADS>
+__device__ __forceinline__ unsigned long long
+segment_offsets(const uint32_t *tile_ent, const uint32_t *tile_out, const unsigned long long *seg_sum, long long seg,
+                long long t0, long long nt, const unsigned long long *base, uint32_t max_ent,
+                unsigned long long *s_off, uint32_t *s_ent, unsigned long long *s_red)
+{
+    constexpr int NW = THREADS / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // base of the segment: sum of the earlier segments
+    unsigned long long part = 0;
+    for (long long q = tid; q < seg; q += THREADS) part += seg_sum[q];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
+    if (lane == 0) s_red[warp] = part;
+    __syncthreads();
+    // a chunk of a longer scan writes after the keys of the chunks before it
+    unsigned long long seg_base = base ? *base : 0ull;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) seg_base += s_red[w];
+    __syncthreads();
+    // per-tile offsets: each thread scans a run of consecutive tiles
+    const long long per = (nt + THREADS - 1) / THREADS;
+    const long long r0 = min(nt, (long long)tid * per), r1 = min(nt, r0 + per);
+    unsigned long long mine = 0;
+    for (long long q = r0; q < r1; ++q) {
+        const uint32_t o = tile_out[t0 + q];
+        s_ent[q] = min(tile_ent[t0 + q], max_ent);
+        s_off[q] = o;  // the tile's own total, replaced by its offset below
+        mine += o;
+    }
+    unsigned long long inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long u = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += u;
+    }
+    if (lane == 31) s_red[warp] = inc;
+    __syncthreads();
+    unsigned long long run = seg_base + inc - mine;
+    for (int w = 0; w < warp; ++w) run += s_red[w];
+    for (long long q = r0; q < r1; ++q) {
+        const unsigned long long o = s_off[q];
+        s_off[q] = run;
+        run += o;
+    }
+    return run;
+}
+
 }  // namespace dev
 }  // namespace pm

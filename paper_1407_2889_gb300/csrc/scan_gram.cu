@@ -22,16 +22,17 @@
 // compiled as Wu-Manber 0.13 (s = 4) against 2.10, 8,000 patterns of 8-16
 // characters 0.71 (s = 1) against 1.41; counts of 1,000 16-mers 0.075 (s =
 // 8) against 0.18.
+#include <algorithm>
 #include <type_traits>
 
-#include "scan_common.cuh"
+#include "gram_device.cuh"
 
 namespace pm {
 namespace {
 
 using dev::kFull;
+using namespace gramdev;
 
-constexpr int kRow = 512;        // text bytes per warp row
 constexpr int kMaxWarps = 32;
 
 // rows per load batch: enough bytes in flight, at most 16 grams a lane
@@ -69,63 +70,6 @@ struct GramArgs {
 };
 
 __host__ __device__ constexpr int qcap(int s) { return 32 + rows_of(s) * kRow / s; }
-
-// bytes [off, off + 16) of the text, zeros from n on
-__device__ __forceinline__ uint4 load16(const GramArgs &a, long long off)
-{
-    if (a.aligned && off + 16 <= a.n) return __ldg(reinterpret_cast<const uint4 *>(a.text + off));
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (off + 20 <= a.n) {
-        // unaligned text: five aligned words (the last one ends inside the text)
-        const uint8_t *p = a.text + off;
-        const uint32_t sh = uint32_t(reinterpret_cast<uintptr_t>(p) & 3u) * 8u;
-        const uint32_t *w = reinterpret_cast<const uint32_t *>(p - (sh >> 3));
-        if (off >= 3) {
-            const uint32_t w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3), w4 = __ldg(w + 4);
-            v.x = __funnelshift_r(w0, w1, sh);
-            v.y = __funnelshift_r(w1, w2, sh);
-            v.z = __funnelshift_r(w2, w3, sh);
-            v.w = __funnelshift_r(w3, w4, sh);
-            return v;
-        }
-    }
-    uint32_t b[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-        if (off + j < a.n) b[j >> 2] |= uint32_t(a.text[off + j]) << (8 * (j & 3));
-    return make_uint4(b[0], b[1], b[2], b[3]);
-}
-
-// the 2-bit codes (byte >> 1) & 3 of 16 bytes, first character lowest: the
-// multiply gathers a word's four codes in its top byte
-__device__ __forceinline__ uint32_t pack16(const uint4 &v)
-{
-    constexpr uint32_t M = 0x06060606u, G = 0x00820820u;
-    const uint32_t p0 = (v.x & M) * G, p1 = (v.y & M) * G, p2 = (v.z & M) * G, p3 = (v.w & M) * G;
-    return __byte_perm(__byte_perm(p0, p1, 0x0073), __byte_perm(p2, p3, 0x0073), 0x5410);
-}
-
-// pattern bytes against the text at p; `room`: whole words around them lie
-// inside the text
-__device__ __forceinline__ bool same_bytes(const uint8_t *p, int len, const uint32_t *pat, bool room)
-{
-    if (room) {
-        const uint32_t lead = uint32_t(reinterpret_cast<uintptr_t>(p) & 3u), sh = lead * 8u;
-        const uint32_t *w = reinterpret_cast<const uint32_t *>(p - lead);
-        uint32_t cur = __ldg(w);
-        for (int left = len; left > 0; left -= 4) {
-            const uint32_t nxt = __ldg(++w);
-            uint32_t x = __funnelshift_r(cur, nxt, sh) ^ __ldg(pat++);
-            if (left < 4) x &= (1u << (8 * left)) - 1u;
-            if (x) return false;
-            cur = nxt;
-        }
-        return true;
-    }
-    for (int j = 0; j < len; ++j)
-        if (p[j] != uint8_t(__ldg(pat + (j >> 2)) >> (8 * (j & 3)))) return false;
-    return true;
-}
 
 // S: stride; QW: 0 2-bit grams, else words of a byte gram; RANK: buckets by
 // rank in the filter (the queue holds (offset << 18) | gram), else by hash
@@ -176,7 +120,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
         } else {
 #pragma unroll
             for (int r = 0; r <= R; ++r)
-                if (r < R || lane == 0) v[r] = load16(a, base + lane * 16 + r * kRow);
+                if (r < R || lane == 0) v[r] = load16(a.text, a.n, a.aligned, base + lane * 16 + r * kRow);
         }
     };
     if (st < ntiles) load(st, 0);
@@ -443,7 +387,408 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
     }
 }
 
+// ---------------------------------------------------------------------------
+// Dense form: one-length sets whose m-gram is looked up at every position (s =
+// 1, q = m <= 9), where a gram in the table is a match unless a byte outside
+// the alphabet hides in it. There are no buckets and no pattern bytes: the
+// gram's rank in the filter is the distinct pattern's number, and the window
+// is compared with the gram spelled out in letters.
+//
+// What bounds it is instruction issue, then the shared-memory pipe (32 random
+// words cost about 3.5 wavefronts), so PAIR takes two positions per lookup: a
+// word of the pair table, picked by the characters 2 .. m of an (m + 1)-gram,
+// holds for each pair of first characters whether the two m-grams in it are in
+// the set. 64 KB at m = 8; longer grams test the filter's bits. 1 GiB of
+// EST-shaped text, 8,000 8-mers (one position in nine matches), list mode: 1.13
+// ms, with the transition table 1.38, with sampled grams 2.29; 128 MiB, 1,000
+// 8-mers (PFAC): 93 us, sampled 185. 256 MiB of the first: 73 % of the issue
+// slots and 78 % of the shared-memory and L1 pipe in use.
+// ---------------------------------------------------------------------------
+struct DenseArgs {
+    GramArgs a;
+    int pwords;                   // pair table words, 4^(m - 1)
+    uint32_t pmask;               // (pwords - 1) * 4
+    uint32_t gmask;               // 4^m - 1
+    int m;
+    uint32_t lut;                 // the byte of code c in byte c
+    const uint16_t *id_off, *ids; // each distinct pattern's ids
+};
+
+constexpr int kDenseQueue = 32 + 2 * kRow;   // queue entries: two rows, and a rest of fewer than 32
+
+// MW: words of a window (m <= 4 MW)
+template <bool PAIR, int MW>
+__global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_dense_kernel(const DenseArgs da)
+{
+    const GramArgs &a = da.a;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int nwarps = blockDim.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+
+    uint32_t *s_pair = reinterpret_cast<uint32_t *>(smem);
+    uint2 *s_mr = reinterpret_cast<uint2 *>(s_pair + (PAIR ? da.pwords : 0));   // filter word, rank
+    uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_mr + a.fwords);
+    uint32_t *s_exp = s_hist + a.ncodes;                                        // four characters spelled out
+    uint16_t *q16 = reinterpret_cast<uint16_t *>(s_exp + 256) + warp * kDenseQueue;
+    uint8_t *s_ext = reinterpret_cast<uint8_t *>(q16 + (nwarps - warp) * kDenseQueue);  // min(keys - 1, 3)
+
+    for (int i = threadIdx.x; i < a.fwords; i += blockDim.x)
+        s_mr[i] = make_uint2(__ldg(a.filter_g + i), __ldg(a.rank_g + i));
+    for (int i = threadIdx.x; i < a.ncodes; i += blockDim.x) {
+        s_hist[i] = 0u;
+        s_ext[i] = uint8_t(min(int(__ldg(da.id_off + i + 1)) - int(__ldg(da.id_off + i)) - 1, 3));
+    }
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
+        uint32_t x = 0;
+        for (int j = 0; j < 4; ++j) x |= ((da.lut >> (8 * ((i >> (2 * j)) & 3))) & 0xFFu) << (8 * j);
+        s_exp[i] = x;
+    }
+    __syncthreads();
+    if (PAIR) {
+        // Word w, bits 2p and 2p + 1: the (m + 1)-gram x = 16 w + p starts with
+        // the m-gram x mod 4^m and ends with x / 4, so the word interleaves 16
+        // filter bits with 4 others, each of them four times.
+        for (int i = threadIdx.x; i < da.pwords; i += blockDim.x) {
+            const uint32_t b = (uint32_t(i) << 4) & da.gmask;
+            uint32_t f = (s_mr[b >> 5].x >> (b & 16u)) & 0xFFFFu;
+            f = (f | f << 8) & 0x00FF00FFu;
+            f = (f | f << 4) & 0x0F0F0F0Fu;
+            f = (f | f << 2) & 0x33333333u;
+            f = (f | f << 1) & 0x55555555u;
+            const uint32_t e = uint32_t(i) << 2, n = s_mr[e >> 5].x >> (e & 31u);
+            s_pair[i] = f | ((n & 1u) | (n & 2u) << 7 | (n & 4u) << 14 | (n & 8u) << 21) * 0xAAu;
+        }
+        __syncthreads();
+    }
+
+    // A warp takes a run of consecutive tiles, so that a row's characters
+    // after the last lane are the next row's, packed once.
+    const int m = da.m;
+    const uint32_t gmask = da.gmask, pmask = da.pmask;
+    const uint32_t tail = (m & 3) ? (1u << (8 * (m & 3))) - 1u : 0xFFFFFFFFu;  // bytes of the last word compared
+    const uint32_t W = gridDim.x * nwarps, w = blockIdx.x * nwarps + warp;
+    const uint32_t ntiles = uint32_t(a.ntiles), each = ntiles / W, extra = ntiles % W;
+    uint32_t st = w * each + min(w, extra);
+    const uint32_t st_end = st + each + (w < extra ? 1u : 0u);
+    const uint32_t nrows = uint32_t(a.tile) / kRow;          // even
+    const uint32_t nfull = a.aligned ? uint32_t(a.n / kRow) : 0u;   // rows wholly inside an aligned text
+    unsigned long long my_total = 0;
+
+    auto load = [&](uint32_t row) -> uint4 {
+        if (row < nfull) return __ldg(reinterpret_cast<const uint4 *>(a.text + (long long)row * kRow) + lane);
+        return load16(a.text, a.n, a.aligned, (long long)row * kRow + lane * 16);
+    };
+    // a bit per position whose m-gram is in the set: position k at bit 31 - k
+    auto probe = [&](uint32_t lo, uint32_t hi) -> uint32_t {
+        uint32_t mask = 0;
+        if (PAIR) {
+#pragma unroll
+            for (int k = 0; k < 16; k += 2) {
+                const uint32_t at = __funnelshift_r(lo, hi, 2 * k + 2) & pmask;
+                const uint32_t e = *reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(s_pair) + at);
+                const uint32_t win = k == 0 ? lo : __funnelshift_r(lo, hi, 2 * k);
+                mask = __funnelshift_r(mask, __funnelshift_r(e, 0u, win << 1), 2);  // bits 2 (win mod 16) and + 1
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const uint32_t win = k == 0 ? lo : __funnelshift_r(lo, hi, 2 * k);
+                const uint32_t e = s_mr[(win & gmask) >> 5].x;
+                mask = __funnelshift_r(mask, __funnelshift_r(e, 0u, win), 1);
+            }
+        }
+        return __brev(mask & 0xFFFF0000u) << 16;
+    };
+
+    uint32_t c0 = 0;
+    uint4 v1, v2;
+    uint32_t row = st * nrows;
+    if (st < st_end) {
+        c0 = pack16(load(row));
+        v1 = load(row + 1);
+        v2 = load(row + 2);
+    }
+    uint32_t r = 0, ent = 0, outs = 0;
+    int qn = 0;
+    while (st < st_end) {
+        const uint32_t c1 = pack16(v1), c2 = pack16(v2);
+        const bool last = r + 2 == nrows;
+        if (!last || st + 1 < st_end) {
+            v1 = load(row + 3);
+            v2 = load(row + 4);
+        }
+        const uint32_t h0 = __shfl_sync(kFull, lane == 0 ? c1 : c0, (lane + 1) & 31);
+        const uint32_t h1 = __shfl_sync(kFull, lane == 0 ? c2 : c1, (lane + 1) & 31);
+        uint32_t m0 = probe(c0, h0), m1 = probe(c1, h1);
+        c0 = c2;
+
+        // ---- hits -> queue (offsets in the tile), lane by lane: both rows'
+        // counts in one scan ----
+        {
+            const uint32_t cnt = __popc(m0) | __popc(m1) << 16;
+            const uint32_t inc = dev::warp_incl_scan(cnt, lane), tot = __shfl_sync(kFull, inc, 31);
+            uint32_t at = uint32_t(qn) + ((inc - cnt) & 0xFFFFu);
+            uint32_t off = r * kRow + uint32_t(lane) * 16u;
+            while (m0) {
+                const uint32_t k = __clz(int(m0));
+                m0 &= 0x7FFFFFFFu >> k;
+                q16[at++] = uint16_t(off + k);
+            }
+            at = uint32_t(qn) + (tot & 0xFFFFu) + ((inc - cnt) >> 16);
+            off += kRow;
+            while (m1) {
+                const uint32_t k = __clz(int(m1));
+                m1 &= 0x7FFFFFFFu >> k;
+                q16[at++] = uint16_t(off + k);
+            }
+            qn += int(tot & 0xFFFFu) + int(tot >> 16);
+            __syncwarp();
+        }
+        // ---- full batches of 32 (at the tile's end the rest too) ----
+        if (qn >= 32 || (last && qn > 0)) {
+            const long long tile0 = (long long)st * a.tile;
+            const uint8_t *tp = a.text + tile0;
+            uint32_t *dst = static_cast<uint32_t *>(a.slots) + (long long)st * a.slot_stride;
+            // offsets whose words (up to three after the first) lie inside an aligned text
+            const int safe = a.aligned ? int(min(a.n - tile0, 1LL << 30)) - 16 : -1;
+            const int fits = int(min(a.n - tile0, 1LL << 30)) - m;
+            int done = 0;
+            do {
+                const bool in = done + lane < qn;
+                const int off = in ? int(q16[done + lane]) : 0;
+                done += 32;
+                bool ok = in;
+                uint32_t gram;
+                if (off <= safe) {
+                    const uint32_t *wp = reinterpret_cast<const uint32_t *>(tp) + (off >> 2);
+                    const uint32_t sh = uint32_t(off) * 8u;   // the funnel shift takes it modulo 32
+                    uint32_t y[3], p[3];
+                    uint32_t cur = __ldg(wp);
+#pragma unroll
+                    for (int j = 0; j < MW; ++j) {
+                        const uint32_t nxt = __ldg(wp + j + 1);
+                        y[j] = __funnelshift_r(cur, nxt, sh);
+                        p[j] = (y[j] & 0x06060606u) * 0x00820820u;   // four codes in the top byte (pack16)
+                        y[j] ^= s_exp[p[j] >> 24];
+                        cur = nxt;
+                    }
+                    y[MW - 1] &= tail;
+                    gram = MW == 1 ? p[0] >> 24 : __byte_perm(p[0], p[1], 0x0073) & 0xFFFFu;
+                    if (MW == 3) gram |= (p[2] >> 24) << 16;
+                    ok = ok && (MW == 1 ? y[0] : MW == 2 ? y[0] | y[1] : y[0] | y[1] | y[2]) == 0u;
+                } else {
+                    gram = 0u;
+                    ok = ok && off <= fits;
+                    for (int j = 0; ok && j < m; ++j) {
+                        const uint32_t b = tp[off + j], c = (b >> 1) & 3u;
+                        ok = b == ((da.lut >> (8 * c)) & 0xFFu);
+                        gram |= c << (2 * j);
+                    }
+                }
+                gram &= gmask;
+                const uint2 mr = s_mr[gram >> 5];
+                const uint32_t c = mr.y + __popc(mr.x & ~(kFull << (gram & 31u)));
+                const uint32_t bal = __ballot_sync(kFull, ok);
+                if (ok) {
+                    const uint32_t ext = s_ext[c];
+                    atomicAdd(&s_hist[c], 1u);
+                    outs += ext + 1u;
+                    if (ext == 3u) outs += uint32_t(__ldg(da.id_off + c + 1) - __ldg(da.id_off + c)) - 4u;
+                    if (a.list) dst[ent + __popc(bal & lt)] = uint32_t(off) << 18 | ext << 16 | c;
+                }
+                ent += __popc(bal);
+            } while (qn - done >= 32 || (last && qn > done));
+            const int left = max(qn - done, 0);
+            const uint32_t q = lane < left ? q16[done + lane] : 0u;
+            __syncwarp();
+            if (lane < left) q16[lane] = uint16_t(q);
+            __syncwarp();
+            qn = left;
+        }
+        row += 2;
+        r += 2;
+        if (last) {
+            if (a.list) {
+                uint32_t o_tot = outs;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) o_tot += __shfl_xor_sync(kFull, o_tot, o);
+                if (lane == 0) {
+                    a.tile_ent[st] = ent;
+                    a.tile_out[st] = o_tot;
+                    if (o_tot) atomicAdd(&a.seg_sum[st / uint32_t(a.seg_tiles)], (unsigned long long)o_tot);
+                }
+            } else {
+                my_total += outs;
+            }
+            ent = 0;
+            outs = 0;
+            r = 0;
+            ++st;
+        }
+    }
+
+    if (!a.list) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) my_total += __shfl_down_sync(kFull, my_total, o);
+        if (lane == 0 && my_total) atomicAdd(reinterpret_cast<unsigned long long *>(a.n_occ), my_total);
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < a.ncodes; c += blockDim.x) {
+        const uint32_t x = s_hist[c];
+        if (!x) continue;
+        const uint32_t j1 = __ldg(da.id_off + c + 1);
+        for (uint32_t j = __ldg(da.id_off + c); j < j1; ++j)
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + __ldg(da.ids + j), (unsigned long long)x);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Keys of the dense form. An entry is (start in the tile << 18) | (min(keys -
+// 1, 3) << 16) | distinct pattern; id_off / ids list each distinct pattern's
+// ids. CTA b owns segment b's tiles, a warp takes a tile in rows of 32 entries,
+// eight rows loaded together and the next eight in flight. A key's place in a
+// row comes from two ballots of the entries' key counts, so the tables are read
+// for the ids only; the row is issue-bound, and looking the counts up (as the
+// expand kernel of the other scans does) took twice the instructions.
+// ---------------------------------------------------------------------------
+constexpr int kDenseExpandThreads = 512;
+
+template <bool SM>
+__global__ void __launch_bounds__(kDenseExpandThreads)
+dense_expand_kernel(const uint32_t *__restrict__ slots, const uint32_t *__restrict__ tile_ent,
+                    const uint32_t *__restrict__ tile_out, const unsigned long long *__restrict__ seg_sum,
+                    long long seg_tiles, long long ntiles, uint32_t tile, const uint16_t *__restrict__ id_off,
+                    const uint16_t *__restrict__ ids, int nc, int d, unsigned long long *__restrict__ occ,
+                    long long occ_cap, long long *n_occ, const unsigned long long *occ_base,
+                    unsigned long long pos_base)
+{
+    constexpr int T = kDenseExpandThreads, NW = T / 32, R = 8;
+    extern __shared__ __align__(16) unsigned char esm[];
+    unsigned long long *s_off = reinterpret_cast<unsigned long long *>(esm);
+    uint32_t *s_ent = reinterpret_cast<uint32_t *>(s_off + seg_tiles);
+    uint16_t *s_io = reinterpret_cast<uint16_t *>(s_ent + seg_tiles), *s_id = s_io + nc + 1;
+    __shared__ unsigned long long s_red[NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    const long long t0 = (long long)blockIdx.x * seg_tiles;
+    const int nt = int(max(0LL, min(seg_tiles, ntiles - t0)));
+    if (nt == 0) return;
+    if (SM) {
+        for (int i = tid; i <= nc; i += T) s_io[i] = __ldg(id_off + i);
+        for (int i = tid; i < d; i += T) s_id[i] = __ldg(ids + i);
+    }
+    const unsigned long long run = dev::segment_offsets<T>(tile_ent, tile_out, seg_sum, blockIdx.x, t0, nt, occ_base,
+                                                           tile, s_off, s_ent, s_red);
+    if (tid == T - 1 && t0 + nt == ntiles) *n_occ = (long long)run;
+    __syncthreads();
+    auto first_of = [&](uint32_t c) -> uint32_t { return SM ? s_io[c] : __ldg(id_off + c); };
+    auto id_at = [&](uint32_t j) -> uint32_t { return SM ? s_id[j] : __ldg(ids + j); };
+
+    const unsigned long long cap = (unsigned long long)occ_cap;
+    uint32_t x[R], y[R];
+    auto load = [&](uint32_t (&z)[R], int q, uint32_t g) {
+        const uint32_t ent = s_ent[q];
+        const uint32_t *src = slots + (t0 + q) * tile + g + lane;
+#pragma unroll
+        for (int u = 0; u < R; ++u) z[u] = g + u * 32 + lane < ent ? __ldcs(src + u * 32) : 0u;
+    };
+    int q = warp;
+    while (q < nt && s_ent[q] == 0) q += NW;
+    uint32_t g = 0, pos = 0, room = 0;
+    unsigned long long *out = occ;
+    if (q < nt) load(x, q, 0);
+    while (q < nt) {
+        const uint32_t ent = s_ent[q];
+        if (g == 0) {  // 32-bit key offsets from the tile's base, clipped to the capacity left after it
+            const unsigned long long b = s_off[q];
+            out = occ + b;
+            room = b < cap ? uint32_t(min(cap - b, 0xFFFFFFFFull)) : 0u;
+            pos = 0;
+        }
+        int qn = q;
+        uint32_t gn = g + R * 32;
+        if (gn >= ent) {
+            gn = 0;
+            do qn += NW;
+            while (qn < nt && s_ent[qn] == 0);
+        }
+        if (qn < nt) load(y, qn, gn);
+        const uint32_t tile0 = uint32_t(pos_base) + uint32_t(t0 + q) * tile;
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+            const uint32_t row = g + u * 32;
+            if (row >= ent) break;
+            const uint32_t cnt = min(ent - row, 32u);
+            const bool valid = uint32_t(lane) < cnt;
+            const uint32_t v = x[u], c = v & 0xFFFFu;
+            const uint32_t hi = tile0 + (v >> 18);
+            const uint32_t e0 = __ballot_sync(kFull, v & 0x10000u), e1 = __ballot_sync(kFull, v & 0x20000u);
+            const uint32_t j = first_of(c);
+            if ((e0 & e1) == 0u) {
+                const uint32_t o = pos + lane + __popc(e0 & lt) + 2u * __popc(e1 & lt);
+                if (valid && o < room) out[o] = (unsigned long long)hi << 32 | id_at(j);
+                if ((v & 0x30000u) && o + 1u < room) out[o + 1u] = (unsigned long long)hi << 32 | id_at(j + 1u);
+                if ((v & 0x20000u) && o + 2u < room) out[o + 2u] = (unsigned long long)hi << 32 | id_at(j + 2u);
+                pos += cnt + __popc(e0) + 2u * __popc(e1);
+            } else {  // four or more equal patterns
+                const uint32_t n = valid ? first_of(c + 1u) - j : 0u;
+                const uint32_t inc = dev::warp_incl_scan(n, lane);
+                const uint32_t o = pos + inc - n;
+                for (uint32_t k = 0; k < n; ++k)
+                    if (o + k < room) out[o + k] = (unsigned long long)hi << 32 | id_at(j + k);
+                pos += __shfl_sync(kFull, inc, 31);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < R; ++u) x[u] = y[u];
+        q = qn;
+        g = gn;
+    }
+}
+
+// shared memory of the dense form (mirrors the kernel's carve-up)
+long long dense_smem(const GramTables &t, bool pair, int warps)
+{
+    const long long nc = (long long)t.code.size();
+    return 4 * ((pair ? 1LL << (2 * (t.q - 1)) : 0) + 2 * (long long)t.filter.size() + nc + 256) +
+           2 * (long long)warps * kDenseQueue + nc;
+}
+
+typedef void (*DenseKernel)(const DenseArgs);
+
+DenseKernel dense_kernel_of(const GramTables &t, bool pair)
+{
+    if (t.q <= 4) return pair ? gram_dense_kernel<true, 1> : gram_dense_kernel<false, 1>;
+    if (t.q <= 8) return pair ? gram_dense_kernel<true, 2> : gram_dense_kernel<false, 2>;
+    return gram_dense_kernel<false, 3>;
+}
+
+int dense_expand(const GramTables &t, const DevGram &dv, const GramArgs &a, const GramWs &ws, const DeviceProps &dp,
+                 uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ, const unsigned long long *occ_base,
+                 unsigned long long pos_base, cudaStream_t st)
+{
+    const int nc = int(t.code.size());
+    const long long base = a.seg_tiles * 12, tab = 2 * ((long long)nc + 1 + t.d);
+    const long long per_cta = std::min<long long>((long long)dp.smem_per_sm / 2 - 2048, dp.smem_optin - 1024);
+    const bool sm = base + tab <= per_cta;
+    const long long smem = base + (sm ? tab : 0);
+    const auto fn = sm ? dense_expand_kernel<true> : dense_expand_kernel<false>;
+    const int rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), smem);
+    if (rc) return rc;
+    fn<<<unsigned((a.ntiles + a.seg_tiles - 1) / a.seg_tiles), kDenseExpandThreads, size_t(smem), st>>>(
+        static_cast<const uint32_t *>(ws.slots), ws.tile_ent, ws.tile_out, ws.seg_sum, a.seg_tiles, a.ntiles,
+        uint32_t(a.tile), dv.id_off, dv.ids, nc, int(t.d), reinterpret_cast<unsigned long long *>(d_occ),
+        d_occ ? occ_cap : 0, reinterpret_cast<long long *>(d_n_occ), occ_base, pos_base);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
+    return PM_OK;
+}
+
 typedef void (*GramKernel)(const GramArgs);
+
+inline long long up4w(long long x) { return (x + 3) & ~3LL; }
 
 template <int QW, bool RANK>
 GramKernel by_stride(int s)
@@ -468,11 +813,9 @@ GramKernel kernel_of(const GramTables &t)
     }
 }
 
-long long up4(long long x) { return (x + 3) & ~3LL; }
-
 long long table_words(const GramTables &t)
 {
-    return up4((long long)t.filter.size()) * (t.rank ? 2 : 1);
+    return up4w((long long)t.filter.size()) * (t.rank ? 2 : 1);
 }
 
 long long queue_words(const GramTables &t) { return t.rank ? qcap(t.s) : qcap(t.s) + qcap(t.s) / 2; }
@@ -485,10 +828,22 @@ int gram_plan(const GramTables &t, const DeviceProps &dp, DevGram &dev)
     if (!t.ok) return PM_OK;
     const long long budget = (long long)dp.smem_optin - 1024;
     const long long nc = (long long)t.code.size();
+    if (t.dense) {
+        for (int w : {32, 28, 24, 20, 16})
+            for (bool pair : {true, false}) {
+                if ((pair && t.q > 8) || dense_smem(t, pair, w) > budget) continue;
+                dev.warps = w;
+                dev.hist_smem = 1;
+                dev.pair = pair ? 1 : 0;
+                dev.use = true;
+                return PM_OK;
+            }
+        return PM_OK;
+    }
     // counters in shared memory if they fit beside 24 warps' queues
     for (int hist : {1, 0})
         for (int w : {32, 24, 16}) {
-            const long long need = 4 * (table_words(t) + (hist ? up4(nc) : 0) + w * queue_words(t));
+            const long long need = 4 * (table_words(t) + (hist ? up4w(nc) : 0) + w * queue_words(t));
             if (need > budget || (hist && w < 24)) continue;
             dev.warps = w;
             dev.hist_smem = hist;
@@ -557,21 +912,44 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
     a.seg_sum = ws.seg_sum;
     a.seg_tiles = (a.ntiles + ws.segs - 1) / ws.segs;
 
-    const GramKernel fn = kernel_of(t);
     // a short text: fewer warps per CTA, spread over every SM (at least 8,
     // which load the tables)
     const long long spread = (a.ntiles + dp.sm_count - 1) / dp.sm_count;
     if (spread < warps) warps = int(spread < 8 ? 8 : spread);
-    const long long smem = 4 * (table_words(t) + (dv.hist_smem ? up4(a.ncodes) : 0) + (long long)warps * queue_words(t));
-    rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), smem);
-    if (rc) return rc;
     long long grid = dp.sm_count;
     const long long want = (a.ntiles + warps - 1) / warps;
     if (want < grid) grid = want;
-    fn<<<dim3(unsigned(grid)), dim3(unsigned(warps * 32)), size_t(smem), st>>>(a);
+    const dim3 gd{unsigned(grid)}, bd{unsigned(warps * 32)};
+    if (t.dense) {
+        DenseArgs da;
+        da.a = a;
+        // a short text does not repay the pair table (1 MiB against 100 8-mers:
+        // 21.5 us without it, 22.0 with)
+        const bool pair = dv.pair && n >= (int64_t(8) << 20);
+        da.pwords = 1 << (2 * (t.q - 1));
+        da.pmask = uint32_t(da.pwords - 1) * 4u;
+        da.gmask = (1u << (2 * t.q)) - 1u;
+        da.m = t.q;
+        da.lut = t.lut;
+        da.id_off = dv.id_off;
+        da.ids = dv.ids;
+        const long long smem = dense_smem(t, pair, warps);
+        const DenseKernel fn = dense_kernel_of(t, pair);
+        rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), smem);
+        if (rc) return rc;
+        fn<<<gd, bd, size_t(smem), st>>>(da);
+    } else {
+        const GramKernel fn = kernel_of(t);
+        const long long smem =
+            4 * (table_words(t) + (dv.hist_smem ? up4w(a.ncodes) : 0) + (long long)warps * queue_words(t));
+        rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), smem);
+        if (rc) return rc;
+        fn<<<gd, bd, size_t(smem), st>>>(a);
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
     if (!list) return PM_OK;
+    if (t.dense) return dense_expand(t, dv, a, ws, dp, d_occ, occ_cap, d_n_occ, occ_base, pos_base, st);
     ExpandTiles tl;
     tl.tile = tile;
     tl.slot_stride = a.slot_stride;
