@@ -20,9 +20,10 @@ INCLUDE = os.path.join(ROOT, "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CU_SOURCES = ["scan_ac.cu", "scan_ac_wide.cu", "scan_ac_wide_counts.cu", "scan_wm.cu", "scan_batch.cu", "scan_acv.cu",
-              "scan_ac2.cu", "scan_gram.cu"]
+              "scan_ac2.cu", "scan_gram.cu", "scan_gram_batch.cu"]
 CPP_SOURCES = ["compile.cpp", "gram.cpp", "capi.cpp", "serve.cpp"]
-HEADERS = ["pm_internal.h", "scan_common.cuh", "ac_device.cuh", "ac_scan_kernel.cuh", "gram_device.cuh"]
+HEADERS = ["pm_internal.h", "scan_common.cuh", "ac_device.cuh", "ac_scan_kernel.cuh", "gram_device.cuh",
+           "batch_device.cuh", "scan_gram_batch.cuh"]
 
 
 def _nvcc() -> str:

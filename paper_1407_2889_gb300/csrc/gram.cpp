@@ -51,6 +51,14 @@ uint32_t gram_hash(const GramTables &t, const uint8_t *g, uint32_t *bit)
     return h;
 }
 
+// the 2-bit codes of up to 16 of len characters, first one lowest
+uint32_t codes(const uint8_t *p, int64_t len)
+{
+    uint32_t x = 0;
+    for (int j = 0; j < 16 && j < len; ++j) x |= code2(p[j]) << (2 * j);
+    return x;
+}
+
 }  // namespace
 
 int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, double limit, GramTables &t)
@@ -126,6 +134,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, doubl
             return PM_OK;
         }
         t.var = var;
+        t.cost = best;
         t.d = d;
         t.m_min = lo;
         t.m_max = hi;
@@ -173,7 +182,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, doubl
             }
         }
         const size_t nc = rep.size();
-        t.pw = (hi + 3) / 4;
+        t.pw = (hi + 15) / 16 * 4;   // whole 16-byte blocks
         t.pats.assign(nc * size_t(t.pw), 0u);
         for (size_t c = 0; c < nc; ++c)
             std::memcpy(reinterpret_cast<uint8_t *>(t.pats.data() + c * size_t(t.pw)), P + first(rep[c]),
@@ -220,6 +229,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, doubl
                 const uint32_t x = h[size_t(k) * nc + c];
                 GramEntry &e = t.ent[at[bucket(x)]++];
                 e.h = x;
+                if (t.qw == 0) e.h = codes(P + first(rep[c]) + k, len_of(rep[c]) - k);
                 e.idx = uint32_t(c);
                 e.k_len = uint32_t(k) | uint32_t(len_of(rep[c])) << 8;
                 e.code = t.code[c];
@@ -266,7 +276,8 @@ void host_walk_gram(const GramTables &t, const uint8_t *T, int64_t n, std::vecto
         for (uint32_t e = t.dir[bk]; e < t.dir[bk + 1]; ++e) {
             const GramEntry &en = t.ent[e];
             const int64_t start = p - int64_t(en.k_len & 255u), len = int64_t(en.k_len >> 8);
-            if (en.h != x || start < 0 || start + len > n) continue;
+            if (start < 0 || start + len > n) continue;
+            if (t.qw != 0 ? en.h != x : en.h != codes(T + p, start + len - p)) continue;
             if (std::memcmp(T + start, t.pats.data() + size_t(en.idx) * size_t(t.pw), size_t(len)) != 0) continue;
             auto put = [&](uint32_t r) {
                 occ.push_back((uint64_t(start) << 32) | r);

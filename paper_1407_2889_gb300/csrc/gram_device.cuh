@@ -1,4 +1,5 @@
-// gram_device.cuh -- device building blocks of the sampled-gram scan: text loads, 2-bit packing, pattern comparison, and the shape
+// gram_device.cuh -- device building blocks of the sampled-gram scans (plain
+// and batched): text loads, 2-bit packing, pattern comparison, and the shape
 // of a warp's work.
 #pragma once
 
@@ -46,26 +47,114 @@ __device__ __forceinline__ uint32_t pack16(const uint4 &v)
     return __byte_perm(__byte_perm(p0, p1, 0x0073), __byte_perm(p2, p3, 0x0073), 0x5410);
 }
 
-// pattern bytes against the text at p; `room`: whole words around them lie
-// inside the text
+// Text bytes that must follow a window's start, inside the text, for the word
+// path of same_bytes: its 16-byte blocks and the word after them.
+__device__ __forceinline__ int compare_span(int len) { return ((len + 15) & ~15) + 4; }
+
+// pattern bytes (a row of zero-padded 16-byte blocks) against the text at p;
+// `room`: compare_span(len) bytes from p on, and the three before it, are the
+// text's. A block's loads are independent: one at a time, a 62-byte pattern
+// took 16 dependent trips to L2 (158 KB of text with 5,000 matches of such
+// patterns: 607 us on one CTA).
 __device__ __forceinline__ bool same_bytes(const uint8_t *p, int len, const uint32_t *pat, bool room)
 {
     if (room) {
         const uint32_t lead = uint32_t(reinterpret_cast<uintptr_t>(p) & 3u), sh = lead * 8u;
         const uint32_t *w = reinterpret_cast<const uint32_t *>(p - lead);
-        uint32_t cur = __ldg(w);
-        for (int left = len; left > 0; left -= 4) {
-            const uint32_t nxt = __ldg(++w);
-            uint32_t x = __funnelshift_r(cur, nxt, sh) ^ __ldg(pat++);
-            if (left < 4) x &= (1u << (8 * left)) - 1u;
-            if (x) return false;
-            cur = nxt;
+        const uint4 *row = reinterpret_cast<const uint4 *>(pat);
+#pragma unroll 2
+        for (int left = len; left > 0; left -= 16, w += 4, ++row) {
+            const uint4 q = __ldg(row);
+            const uint32_t t0 = __ldg(w), t1 = __ldg(w + 1), t2 = __ldg(w + 2);
+            uint32_t x = __funnelshift_r(t0, t1, sh) ^ q.x, y = __funnelshift_r(t1, t2, sh) ^ q.y;
+            if (left < 8) {
+                if (left < 4) x &= (1u << (8 * left)) - 1u;
+                y &= left <= 4 ? 0u : (1u << (8 * (left - 4))) - 1u;
+            }
+            if (left > 8) {
+                const uint32_t t3 = __ldg(w + 3), t4 = __ldg(w + 4);
+                uint32_t z = __funnelshift_r(t2, t3, sh) ^ q.z, v = __funnelshift_r(t3, t4, sh) ^ q.w;
+                if (left < 16) {
+                    if (left < 12) z &= (1u << (8 * (left - 8))) - 1u;
+                    v &= left <= 12 ? 0u : (1u << (8 * (left - 12))) - 1u;
+                }
+                x |= z | v;
+            }
+            if (x | y) return false;
         }
         return true;
     }
     for (int j = 0; j < len; ++j)
         if (p[j] != uint8_t(__ldg(pat + (j >> 2)) >> (8 * (j & 3)))) return false;
     return true;
+}
+
+// One batch of 32 passing grams: lane l has the entries e0 .. e0 + cnt - 1 for
+// the gram at offset pos of the tile (cnt 0: none); win: the codes of the 16
+// characters there, or (RAW) the byte gram's hash. Each lane first compares its
+// entries' codes (16 of the pattern's characters, or the hash) with win, which
+// leaves few to compare byte by byte. When a gram still has several, the (gram,
+// entry) pairs are dealt out to the lanes in order, 32 at a time, so that one
+// long list does not hold up the warp. emit(ok, entry, pos) is called by the
+// whole warp; the pairs that match have ok set, and ascend by lane and call in
+// output order.
+struct GramTile {
+    const uint4 *ent;
+    const uint32_t *pats;
+    int pw;
+    const uint8_t *text;             // the tile's first byte
+    int low, rem;                    // starts from low on, ends up to rem, are inside the text
+};
+
+template <bool RAW>
+__device__ __forceinline__ bool same_code(const uint4 &en, uint32_t win)
+{
+    if (RAW) return en.x == win;
+    const uint32_t nc = (en.z >> 8) - (en.z & 255u);   // characters from the gram on
+    return ((en.x ^ win) & (nc >= 16u ? kFull : ~(kFull << (2u * nc)))) == 0u;
+}
+
+template <bool RAW, class Emit>
+__device__ __forceinline__ void verify_batch(const GramTile &g, uint32_t e0, uint32_t cnt, uint32_t win, int pos,
+                                             Emit &&emit)
+{
+    const int lane = threadIdx.x & 31;
+    uint32_t nm = 0, first = 0;
+    for (uint32_t k = 0; k < cnt; ++k) {
+        if (!same_code<RAW>(__ldg(g.ent + e0 + k), win)) continue;
+        if (nm++ == 0) first = e0 + k;
+    }
+    if (!__any_sync(kFull, nm != 0u)) return;
+    auto one = [&](bool in, uint32_t e, uint32_t w, int p) {
+        uint4 en = make_uint4(0u, 0u, 0u, 0u);
+        bool ok = false;
+        if (in) {
+            en = __ldg(g.ent + e);
+            const int start = p - int(en.z & 255u), len = int(en.z >> 8);
+            ok = same_code<RAW>(en, w) && start >= g.low && start + len <= g.rem;
+            if (ok)
+                ok = same_bytes(g.text + start, len, g.pats + (size_t)en.y * g.pw,
+                                start >= g.low + 3 && start + compare_span(len) <= g.rem);
+        }
+        if (__any_sync(kFull, ok)) emit(ok, en, p);
+    };
+    if (!__any_sync(kFull, nm > 1u)) {
+        one(nm != 0u, first, win, pos);
+        return;
+    }
+    if (nm == 0u) cnt = 0u;
+    const uint32_t inc = dev::warp_incl_scan(cnt, lane), total = __shfl_sync(kFull, inc, 31);
+    const uint32_t shift = e0 - (inc - cnt);   // pair x of this lane's gram is entry shift + x
+    for (uint32_t x0 = 0; x0 < total; x0 += 32) {
+        const uint32_t x = x0 + lane;
+        int o = 0;                             // the first lane whose pairs reach past x
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1)
+            if (__shfl_sync(kFull, inc, o + s - 1) <= x) o += s;
+        const uint32_t e = x + __shfl_sync(kFull, shift, o), w = __shfl_sync(kFull, win, o);
+        const int p = __shfl_sync(kFull, pos, o);
+        one(x < total, e, w, p);
+    }
 }
 
 }  // namespace gramdev

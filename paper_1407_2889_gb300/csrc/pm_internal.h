@@ -149,7 +149,7 @@ constexpr int32_t kAcvMaxLen = 65; // the halo of the scan kernels (64 bytes)
 // rank among the filter's set bits.
 // ---------------------------------------------------------------------------
 struct GramEntry {
-    uint32_t h;       // the gram's hash
+    uint32_t h;       // codes of the pattern's characters from the gram on (up to 16), or the byte gram's hash
     uint32_t idx;     // distinct pattern: its bytes are pats[idx * pw ..]
     uint32_t k_len;   // gram offset k in the pattern | pattern length << 8
     uint32_t code;    // pattern id, or 0x80000000 | group of equal patterns
@@ -164,11 +164,12 @@ struct GramTables {
     int32_t s = 0, q = 0, qw = 0;  // stride, gram length, words of a byte gram
     int32_t fb = 0, db = 0, pw = 0;
     uint32_t K[4] = {};
+    double cost = 0.0;             // planned instructions per lane and 16 text bytes
     std::vector<uint32_t> filter;     // 2^fb bits
     std::vector<uint32_t> rank_base;  // rank: set bits before each filter word
     std::vector<uint32_t> dir;        // first entry of each bucket, and the end
     std::vector<GramEntry> ent;
-    std::vector<uint32_t> pats;       // pw words per distinct pattern, zero padded
+    std::vector<uint32_t> pats;       // pw words (16-byte blocks) per distinct pattern, zero padded
     std::vector<uint32_t> code;       // code of each distinct pattern
     std::vector<uint32_t> grp_off, grp_ids;
     // Dense form (one-length sets of fewer than 2^15 patterns, s = 1, q = m):
@@ -496,6 +497,12 @@ struct BatchDesc {                 // one instance, in processing order
     long long pstat_off, done_off;
     long long spill_off, spill_cap;
     int part, nparts;
+    // gram items (gram_batch_kernel): the set's gram tables (see GramTables)
+    int gram, tile;                // tile: text bytes a warp takes at a time
+    int g_s, g_rank, g_fwords, g_pw;
+    uint32_t g_k, g_fshift, g_wshift, g_bshift;
+    const uint32_t *g_filter, *g_rank_base, *g_dir, *g_pats, *g_code, *g_grp_off, *g_grp_ids;
+    const void *g_ent;
 };
 
 struct BatchShape {                // launch shape and shared-memory split
@@ -534,11 +541,13 @@ inline int64_t batch_ws_bytes(int64_t ccount_words) { return kWsHeader + 8 * cco
 // whatever the rest of the batch (list: the instance's keys are listed).
 int64_t batch_words_bound(const BatchInst &I, const BatchShape &sh, bool list);
 // Queue items of a batch of k instances fit at most this many descriptors.
-inline int64_t batch_items_bound(int64_t k, const BatchShape &sh) { return 2 * k + 4 * int64_t(sh.sm_count) + 16; }
+inline int64_t batch_items_bound(int64_t k, const BatchShape &sh) { return 2 * k + 12 * int64_t(sh.sm_count) + 16; }
 int batch_prepare_launch(const BatchShape &sh);  // host-side set-up, before any capture
+// n_gram: how many items, from the first on, are gram items
+int batch_gram_items(const std::vector<BatchDesc> &items);
 int batch_launch_raw(const BatchDesc *d_desc, int k, const uint8_t *text, int64_t *counts,
                      uint64_t *occ, int64_t *n_occ, void *ws, int64_t ccount_total,
-                     const BatchShape &sh, bool list, void *stream);
+                     const BatchShape &sh, bool list, void *stream, int n_gram);
 
 }  // namespace pm
 

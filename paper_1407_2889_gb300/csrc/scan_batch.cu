@@ -23,6 +23,8 @@
 #include <vector>
 
 #include "ac_device.cuh"
+#include "batch_device.cuh"
+#include "scan_gram_batch.cuh"
 
 namespace pm {
 
@@ -40,22 +42,6 @@ constexpr int kBatchPool = 40;                  // hit pool slots per lane, u16 
 constexpr int kBatchPoolBytes = (kBatchPool + 1) * 32 * 2;
 constexpr int kBatchStage = 128;              // u64 entries
 constexpr int kBatchMaxM = 16 * kBatchHV + 1;
-
-struct BatchArgs {
-    const BatchDesc *desc;
-    int k;
-    const uint8_t *text;
-    long long *counts;
-    unsigned long long *occ;
-    long long *n_occ;
-    dev::WsHeader *ws;
-    unsigned long long *ccount;
-    unsigned long long *spill;     // key staging of split instances' parts
-    int list;
-    int region_bytes;              // per-CTA shared memory for table, ids and counters
-};
-
-__host__ __device__ constexpr long long rr16(long long x) { return (x + 15) & ~15LL; }
 
 __host__ __device__ inline long long batch_warp_bytes()
 {
@@ -136,7 +122,6 @@ __device__ void run_instance(const BatchArgs &a, const BatchDesc &D, const CtaSm
     E *pl = reinterpret_cast<E *>(S.pool) + lane;
     const uint32_t cap = kBatchPoolBytes / (32 * sizeof(E)) - 1;  // the last slot absorbs overflow
     const int m = D.m;
-    const bool split = D.nparts > 1;
     auto count_terminal = [&](uint32_t c) {
         if (s_hist) atomicAdd(&s_hist[c], 1u);
         else atomicAdd(&g_hist[c], 1ull);
@@ -343,82 +328,7 @@ __device__ void run_instance(const BatchArgs &a, const BatchDesc &D, const CtaSm
         }
     };
 
-    if (!split) {
-        const unsigned long long total = pass(true, a.list != 0, 0ull);
-        if (threadIdx.x == 0) a.n_occ[D.out_slot] = (long long)total;
-        write_counts(s_hist == nullptr);
-        __syncthreads();
-        return;
-    }
-
-    // ---- a part of a split instance ----------------------------------------
-    __shared__ unsigned long long s_base;
-    __shared__ int s_last;
-    unsigned long long *pstat = a.ccount + D.pstat_off;  // (1 << 63) | part total
-    const bool staged = a.list && D.spill_cap > 0;
-    if (staged) {
-        odst = a.spill + D.spill_off;
-        ocap = (unsigned long long)D.spill_cap;
-    }
-    const unsigned long long total = pass(true, staged, 0ull);
-    if (threadIdx.x == 0) {
-        dev::st_relaxed(&pstat[D.part], (1ull << 63) | total);
-        unsigned long long base = 0;
-        if (a.list) {
-            // the parts before this one were taken earlier by running CTAs,
-            // and publish their totals without waiting for anything
-            const long long t0c = clock64();
-            for (int q = 0; q < D.part; ++q) {
-                unsigned long long v = dev::ld_relaxed(&pstat[q]);
-                while (!(v >> 63)) {
-                    if (clock64() - t0c > dev::kSpinLimit) {
-                        dev::set_status(a.ws, dev::kErrTimeoutWait);
-                        break;
-                    }
-                    __nanosleep(128);
-                    v = dev::ld_relaxed(&pstat[q]);
-                }
-                base += v & ~(1ull << 63);
-            }
-        }
-        s_base = base;
-    }
-    __syncthreads();
-    if (a.list) {
-        odst = a.occ + D.occ_off;
-        ocap = (unsigned long long)D.occ_cap;
-        const unsigned long long b0 = s_base;
-        if (staged && total <= (unsigned long long)D.spill_cap) {
-            // this CTA's own stores, ordered by the barrier above
-            const unsigned long long *sp = a.spill + D.spill_off;
-            const unsigned long long nkeep = b0 < ocap ? min(total, ocap - b0) : 0ull;
-            for (unsigned long long i = threadIdx.x; i < nkeep; i += blockDim.x) odst[b0 + i] = sp[i];
-        } else if (b0 < ocap) {
-            (void)pass(false, true, b0);
-        }
-    }
-    // counters into the instance's device counters; the last part writes
-    // the instance's counts and its total
-    if (s_hist)
-        for (int c = threadIdx.x; c < D.nterms; c += blockDim.x)
-            if (s_hist[c]) atomicAdd(&g_hist[c], (unsigned long long)s_hist[c]);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned int *done = reinterpret_cast<unsigned int *>(a.ccount + D.done_off);
-        s_last = atomicAdd(done, 1u) == unsigned(D.nparts - 1);
-    }
-    __syncthreads();
-    if (s_last) {
-        __threadfence();
-        write_counts(true);
-        if (threadIdx.x == 0) {
-            unsigned long long all = 0;
-            for (int q = 0; q < D.nparts; ++q) all += dev::ld_acquire(&pstat[q]) & ~(1ull << 63);
-            a.n_occ[D.out_slot] = (long long)all;
-        }
-    }
-    __syncthreads();
+    run_item(a, D, s_hist, g_hist, odst, ocap, pass, write_counts);
 }
 
 __global__ void __launch_bounds__(512, 1) ac_batch_kernel(const BatchArgs a)
@@ -482,15 +392,23 @@ constexpr long long kSpillBytes = 32;               // text bytes per staged key
 constexpr int kBatchMaxWarps = 16;
 
 struct InstLayout {
-    int smem_entries, ids_off, hist_off;
+    int smem_entries = 0, ids_off = -1, hist_off = -1;
+    bool gram = false;     // gram_batch_kernel's item; hist_off as for the others
+    int tile = 0;          // gram: text bytes a warp takes at a time
 };
 
 // Where an instance's tables go inside the region. Everything when it fits;
 // otherwise counters and ids stay in shared memory only while each takes at
 // most a quarter of the region, and the table gets the rest (its
 // breadth-first prefix: the rows a walk visits most).
-static InstLayout layout_of(const AcTables &t, int region, int policy)
+static InstLayout layout_of(const pm_set *s, int region, int policy)
 {
+    const AcTables &t = s->ac;
+    if (s->dac.dg) {  // sets that take the gram scan take it here too, where their tables fit
+        InstLayout G;
+        G.gram = gram_batch_layout(s->gram, G.hist_off, G.tile);
+        if (G.gram) return G;
+    }
     const int eb = t.entry_bytes;
     const long long entries = (long long)t.n_rows << t.lw;
     const long long nw = (long long)t.flag_mask.size(), nt = (long long)t.canon.size();
@@ -575,6 +493,8 @@ static void fill_desc(const BatchInst &I, const InstLayout &L, long long coff, B
     D.t_hi = (I.text_len + kWarpTile - 1) / kWarpTile;
     D.part = 0;
     D.nparts = 1;
+    D.gram = 0;
+    if (L.gram) gram_batch_fill(I.set->gram, I.set->dgram, L.tile, D);
 }
 
 int64_t batch_fill(const BatchInst *inst, int k, const BatchShape &sh, BatchDesc *out)
@@ -583,7 +503,7 @@ int64_t batch_fill(const BatchInst *inst, int k, const BatchShape &sh, BatchDesc
     for (int q = 0; q < k; ++q) {
         const BatchInst &I = inst[q];
         const AcTables &t = I.set->ac;
-        const InstLayout L = layout_of(t, sh.region_bytes, sh.policy);
+        const InstLayout L = layout_of(I.set, sh.region_bytes, sh.policy);
         const int64_t nt = int64_t(t.canon.size());
         const int64_t coff = ccount;
         if (L.hist_off < 0) ccount += nt;
@@ -600,22 +520,30 @@ int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool lis
     if (k <= 0) return 0;
     std::vector<InstLayout> lay(static_cast<size_t>(k));
     std::vector<double> cost(static_cast<size_t>(k));
-    double total = 0.0;
+    double total[2] = {0.0, 0.0};   // the two kernels run one after the other
     for (int q = 0; q < k; ++q) {
         const AcTables &t = inst[q].set->ac;
-        lay[size_t(q)] = layout_of(t, sh.region_bytes, sh.policy);
+        const InstLayout L = layout_of(inst[q].set, sh.region_bytes, sh.policy);
+        lay[size_t(q)] = L;
         // a table read partly through L2 costs several times more per byte;
-        // every instance also pays for loading its tables
+        // every instance also pays for loading its tables. Gram items by their
+        // planned instructions per byte, a filter load about a third of a
+        // sparse scan of as many bytes
         const long long entries = (long long)t.n_rows << t.lw;
-        const double w = lay[size_t(q)].smem_entries >= entries ? 1.0 : 4.0;
-        cost[size_t(q)] = double(inst[q].text_len) * w + 4.0 * double(lay[size_t(q)].smem_entries * t.entry_bytes);
-        total += cost[size_t(q)];
+        if (L.gram)
+            cost[size_t(q)] = double(inst[q].text_len) * (30.0 + inst[q].set->gram.cost) +
+                              30.0 * 4.0 * double(inst[q].set->gram.filter.size()) + 1.0e6;
+        else
+            cost[size_t(q)] = double(inst[q].text_len) * (L.smem_entries >= entries ? 1.0 : 4.0) +
+                              4.0 * double(L.smem_entries * t.entry_bytes);
+        total[L.gram ? 0 : 1] += cost[size_t(q)];
     }
     std::vector<int> order(static_cast<size_t>(k));
     std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return cost[size_t(x)] > cost[size_t(y)]; });
-    // about four items per CTA: an instance above that share is split
-    const double share = total / (4.0 * double(std::max(sh.sm_count, 1)));
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+        if (lay[size_t(x)].gram != lay[size_t(y)].gram) return lay[size_t(x)].gram;
+        return cost[size_t(x)] > cost[size_t(y)];
+    });
     int64_t ccount = 0, spill = 0;
     for (const int q : order) {
         const BatchInst &I = inst[q];
@@ -623,6 +551,9 @@ int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool lis
         const int64_t nt = int64_t(I.set->ac.canon.size());
         const long long ntiles = (I.text_len + kWarpTile - 1) / kWarpTile;
         long long parts = 1;
+        // about four items per CTA (eight gram items, which cost less): an
+        // instance above that share is split
+        const double share = total[L.gram ? 0 : 1] / ((L.gram ? 8.0 : 4.0) * double(std::max(sh.sm_count, 1)));
         if (cost[size_t(q)] > share && share > 0.0) {
             parts = (long long)std::ceil(cost[size_t(q)] / share);
             parts = std::min(parts, ntiles / (2LL * sh.warps));  // at least two rounds of tiles each
@@ -646,6 +577,7 @@ int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool lis
             D.nparts = int(parts);
             D.pstat_off = pstat;
             D.done_off = done;
+            if (D.gram) D.tile = gram_batch_tile(D, L.tile);
             if (parts > 1 && list) {
                 // one key per kSpillBytes text bytes, at most the instance's capacity
                 const long long bytes = std::min(D.t_hi * kWarpTile, (long long)I.text_len) - D.t_lo * kWarpTile;
@@ -663,7 +595,7 @@ int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool lis
 int64_t batch_words_bound(const BatchInst &I, const BatchShape &sh, bool list)
 {
     const AcTables &t = I.set->ac;
-    const InstLayout L = layout_of(t, sh.region_bytes, sh.policy);
+    const InstLayout L = layout_of(I.set, sh.region_bytes, sh.policy);
     const long long ntiles = (I.text_len + kWarpTile - 1) / kWarpTile;
     const long long parts = std::max(1LL, ntiles / (2LL * std::max(sh.warps, 1)));
     int64_t w = (L.hist_off < 0 || parts > 1) ? int64_t(t.canon.size()) : 0;
@@ -672,6 +604,13 @@ int64_t batch_words_bound(const BatchInst &I, const BatchShape &sh, bool list)
         if (list) w += std::min<int64_t>(parts * I.occ_cap, (I.text_len + kSpillBytes - 1) / kSpillBytes + parts);
     }
     return w;
+}
+
+int batch_gram_items(const std::vector<BatchDesc> &items)
+{
+    int g = 0;
+    while (size_t(g) < items.size() && items[size_t(g)].gram) ++g;
+    return g;
 }
 
 static int ensure_batch_attr(long long smem_bytes)
@@ -690,14 +629,18 @@ static int ensure_batch_attr(long long smem_bytes)
     return PM_OK;
 }
 
-int batch_prepare_launch(const BatchShape &sh) { return ensure_batch_attr(sh.smem_bytes); }
+int batch_prepare_launch(const BatchShape &sh)
+{
+    const int rc = gram_batch_attr();
+    return rc ? rc : ensure_batch_attr(sh.smem_bytes);
+}
 
 // A memset of the queue, status and global counters, then the persistent
 // kernel. Nothing else touches the host, so the pair can be captured in a
 // graph (batch_prepare_launch must have run for the shape).
 int batch_launch_raw(const BatchDesc *d_desc, int k, const uint8_t *text, int64_t *counts,
                      uint64_t *occ, int64_t *n_occ, void *ws, int64_t ccount_total,
-                     const BatchShape &sh, bool list, void *stream)
+                     const BatchShape &sh, bool list, void *stream, int n_gram)
 {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemsetAsync(ws, 0, size_t(batch_ws_bytes(ccount_total)), st);
@@ -715,7 +658,15 @@ int batch_launch_raw(const BatchDesc *d_desc, int k, const uint8_t *text, int64_
     a.spill = a.ccount + ccount_total;
     a.list = list ? 1 : 0;
     a.region_bytes = sh.region_bytes;
-    const int grid = std::min(sh.sm_count, k);
+    // the gram items come first in the queue order
+    if (n_gram > 0) {
+        a.k = n_gram;
+        const int rc = gram_batch_enqueue(a, std::min(sh.sm_count, n_gram), stream);
+        if (rc || n_gram == k) return rc;
+        a.desc = d_desc + n_gram;
+        a.k = k - n_gram;
+    }
+    const int grid = std::min(sh.sm_count, a.k);
     ac_batch_kernel<<<dim3(unsigned(grid)), dim3(unsigned(sh.warps * 32)), size_t(sh.smem_bytes), st>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
@@ -729,6 +680,7 @@ struct pm_batch {
     int32_t k = 0;
     std::vector<int64_t> occ_off, count_off;
     std::vector<pm::BatchInst> inst;  // as given
+    int32_t n_gram = 0;               // of them, the first n_gram are gram items
     int32_t n_items = 0;              // queue items (instances, or parts of large ones)
     int64_t desc_cap = 0;             // descriptors the device array holds
     pm::BatchDesc *d_desc = nullptr;
@@ -752,6 +704,7 @@ static int apply_plan(pm_batch *b, int warps, int policy)
     std::vector<BatchDesc> h;
     b->ccount_total = batch_items(b->inst.data(), b->k, b->shape, !(b->flags & PM_COUNTS_ONLY), h, nullptr);
     b->n_items = int32_t(h.size());
+    b->n_gram = batch_gram_items(h);
     if (h.empty()) return PM_OK;
     cudaError_t e = cudaSuccess;
     if (b->desc_cap < int64_t(h.size())) {
@@ -781,7 +734,7 @@ struct BatchBufs {
 static int batch_enqueue(const pm_batch *b, const BatchBufs &o, cudaStream_t st)
 {
     return batch_launch_raw(b->d_desc, b->n_items, o.text, o.counts, o.occ, o.n_occ, o.ws, b->ccount_total,
-                            b->shape, !(b->flags & PM_COUNTS_ONLY), st);
+                            b->shape, !(b->flags & PM_COUNTS_ONLY), st, b->n_gram);
 }
 
 static int batch_check(const pm_batch *b, const BatchBufs &o, int64_t ws_bytes)

@@ -27,7 +27,8 @@ struct WsHeader {           // lives at the start of the workspace
     uint32_t done_expand;   // expand CTAs that finished (late ids: the last one finalises counts)
     uint32_t pad0;
     unsigned long long queue;  // batched scan: next instance to take
-    unsigned long long pad1[29];
+    unsigned long long queue2; // batched gram scan: next item to take
+    unsigned long long pad1[28];
 };
 static_assert(sizeof(WsHeader) <= kWsHeader, "workspace header too large");
 

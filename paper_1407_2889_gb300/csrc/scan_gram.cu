@@ -72,8 +72,8 @@ struct GramArgs {
 __host__ __device__ constexpr int qcap(int s) { return 32 + rows_of(s) * kRow / s; }
 
 // S: stride; QW: 0 2-bit grams, else words of a byte gram; RANK: buckets by
-// rank in the filter (the queue holds (offset << 18) | gram), else by hash
-// (offsets and hashes side by side).
+// rank in the filter, else by hash. The queue holds each passing gram's offset
+// and the codes of the 16 characters from it on (a byte gram's hash).
 template <int S, int QW, bool RANK>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const GramArgs a)
 {
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
     uint32_t *s_filter = reinterpret_cast<uint32_t *>(smem);
     uint32_t *s_rank = s_filter + ((a.fwords + 3) & ~3);
     uint32_t *s_hist = s_rank + (RANK ? (a.fwords + 3) & ~3 : 0);
-    uint32_t *q32 = s_hist + (a.hist_smem ? (a.ncodes + 3) & ~3 : 0) + warp * (RANK ? QCAP : QCAP + QCAP / 2);
+    uint32_t *q32 = s_hist + (a.hist_smem ? (a.ncodes + 3) & ~3 : 0) + warp * (QCAP + QCAP / 2);
     uint16_t *q16 = reinterpret_cast<uint16_t *>(q32 + QCAP);
 
     {   // the tables are padded to 16 bytes
@@ -211,27 +211,15 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
                     while (m) {
                         const uint32_t k = uint32_t(__ffs(int(m))) - 1u;
                         m &= m - 1u;
-                        const uint32_t h = __funnelshift_r(lo[r], hi[r], 2 * S * k) * K0;
-                        if (RANK) {
-                            q32[at] = ((off0 + S * k) << 18) | (h >> a.fshift);
-                        } else {
-                            q32[at] = h;
-                            q16[at] = uint16_t(off0 + S * k);
-                        }
-                        ++at;
+                        q32[at] = __funnelshift_r(lo[r], hi[r], 2 * S * k);
+                        q16[at++] = uint16_t(off0 + S * k);
                     }
                 } else {
 #pragma unroll
                     for (int k = 0; k < NP; ++k)
                         if ((m >> k) & 1u) {
-                            const uint32_t h = QW == 0 ? lo[r] * K0 : H[QW == 0 ? 0 : r * NP + k];
-                            if (RANK) {
-                                q32[at] = ((off0 + S * k) << 18) | (h >> a.fshift);
-                            } else {
-                                q32[at] = h;
-                                q16[at] = uint16_t(off0 + S * k);
-                            }
-                            ++at;
+                            q32[at] = QW == 0 ? lo[r] : H[QW == 0 ? 0 : r * NP + k];
+                            q16[at++] = uint16_t(off0 + S * k);
                         }
                 }
             }
@@ -240,106 +228,72 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
         // ---- full batches of 32 (at the tile's end the rest too) ----
         if (qn >= 32u || (last && qn > 0u)) {
             const long long tile0 = (long long)st * a.tile;
-            const uint8_t *tp = a.text + tile0;
             // starts relative to the tile, inside the text
-            const int low = tile0 == 0 ? 0 : -S;
-            const int rem = int(min(a.n - tile0, 1LL << 30));
+            const GramTile view{a.ent, a.pats, a.pw, a.text + tile0, tile0 == 0 ? 0 : -S,
+                                int(min(a.n - tile0, 1LL << 30))};
             int done = 0;
             do {
                 const int i = done + lane;
-                uint32_t e0 = 0, e1 = 0, h = 0, off = 0;
+                uint32_t e0 = 0, e1 = 0, win = 0, off = 0;
                 if (i < int(qn)) {
-                    h = q32[i];
+                    win = q32[i];
+                    off = q16[i];
+                    const uint32_t h = QW == 0 ? win * K0 : win;
                     uint32_t bk;
                     if (RANK) {
-                        off = h >> 18;
-                        const uint32_t b = h & 0x3FFFFu;
-                        h = b << a.fshift;
-                        bk = s_rank[b >> 5] + __popc(s_filter[b >> 5] & ((1u << (b & 31u)) - 1u));
+                        const uint32_t b = h >> a.fshift;
+                        bk = s_rank[b >> 5] + __popc(s_filter[b >> 5] & ~(kFull << (b & 31u)));
                     } else {
-                        off = q16[i];
                         bk = h >> a.bshift;
                     }
                     e0 = __ldg(a.dir + bk);
                     e1 = __ldg(a.dir + bk + 1);
                 }
                 done += 32;
-                // does entry e match here?
-                auto match = [&](const uint4 &en) -> bool {
-                    const int start = int(off) - int(en.z & 255u), len = int(en.z >> 8);
-                    if (en.x != h || start < low || start + len > rem) return false;
-                    const bool room = start >= low + 3 && start + ((len + 3) & ~3) + 4 <= rem;
-                    return same_bytes(tp + start, len, a.pats + (size_t)en.y * a.pw, room);
-                };
-                // matches of this lane's gram: counted, then written behind
-                // those of the lanes before it
-                uint32_t nh = 0, val = 0, mark = 0;
-                for (uint32_t e = e0; e < e1; ++e) {
-                    const uint4 en = __ldg(a.ent + e);
-                    if (!match(en)) continue;
-                    uint32_t mult = 1u;
-                    if (a.hist_smem) atomicAdd(&s_hist[en.y], 1u);
-                    if (en.w & 0x80000000u) {
-                        const uint32_t gi = en.w & 0x7FFFFFFFu;
-                        const uint32_t j0 = __ldg(a.grp_off + gi), j1 = __ldg(a.grp_off + gi + 1);
-                        mult = j1 - j0;
-                        if (!a.hist_smem)
-                            for (uint32_t j = j0; j < j1; ++j)
-                                atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + __ldg(a.grp_ids + j), 1ull);
-                    } else if (!a.hist_smem) {
-                        atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + en.w, 1ull);
-                    }
-                    outs += mult;
-                    if (nh == 0) {
-                        val = en.w;
-                        mark = en.z & 255u;
-                    }
-                    ++nh;
-                }
-                if (a.list && __any_sync(kFull, nh != 0u)) {
-                    uint32_t k = ent;
-                    if (__any_sync(kFull, nh > 1u)) {
-                        const uint32_t inc = dev::warp_incl_scan(nh, lane);
-                        k += inc - nh;
-                        ent += __shfl_sync(kFull, inc, 31);
-                    } else {
-                        const uint32_t bal = __ballot_sync(kFull, nh != 0u);
-                        k += __popc(bal & lt);
-                        ent += __popc(bal);
-                    }
-                    auto put = [&](uint32_t gk, uint32_t code) {
-                        // start in the tile, shifted by S - 1 so that it is never negative
-                        const uint32_t o = off + uint32_t(S - 1) - gk;
-                        const long long p = (long long)st * a.slot_stride + k;
-                        if (a.slot_kind == 0)
-                            static_cast<uint32_t *>(a.slots)[p] = (o << 16) | ((code >> 16) & 0x8000u) | (code & 0x7FFFu);
-                        else if (a.slot_kind == 1)
-                            static_cast<unsigned long long *>(a.slots)[p] = ((unsigned long long)o << 32) | code;
-                        else
-                            static_cast<uint32_t *>(a.slots)[p] = (o << 20) | code;
-                        ++k;
-                    };
-                    if (nh == 1u) {
-                        put(mark, val);
-                    } else if (nh > 1u) {
-                        for (uint32_t e = e0; e < e1; ++e) {
-                            const uint4 en = __ldg(a.ent + e);
-                            if (match(en)) put(en.z & 255u, en.w);
+                verify_batch<QW != 0>(view, e0, e1 - e0, win, int(off), [&](bool ok, const uint4 &en, int pos) {
+                    const uint32_t bal = __ballot_sync(kFull, ok);
+                    if (ok) {
+                        uint32_t mult = 1u;
+                        if (a.hist_smem) atomicAdd(&s_hist[en.y], 1u);
+                        if (en.w & 0x80000000u) {
+                            const uint32_t gi = en.w & 0x7FFFFFFFu;
+                            const uint32_t j0 = __ldg(a.grp_off + gi), j1 = __ldg(a.grp_off + gi + 1);
+                            mult = j1 - j0;
+                            if (!a.hist_smem)
+                                for (uint32_t j = j0; j < j1; ++j)
+                                    atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + __ldg(a.grp_ids + j),
+                                              1ull);
+                        } else if (!a.hist_smem) {
+                            atomicAdd(reinterpret_cast<unsigned long long *>(a.counts) + en.w, 1ull);
+                        }
+                        outs += mult;
+                        if (a.list) {
+                            // start in the tile, shifted by S - 1 so that it is never negative
+                            const uint32_t o = uint32_t(pos + (S - 1)) - (en.z & 255u), code = en.w;
+                            const long long p = (long long)st * a.slot_stride + (ent + __popc(bal & lt));
+                            if (a.slot_kind == 0)
+                                static_cast<uint32_t *>(a.slots)[p] =
+                                    (o << 16) | ((code >> 16) & 0x8000u) | (code & 0x7FFFu);
+                            else if (a.slot_kind == 1)
+                                static_cast<unsigned long long *>(a.slots)[p] = ((unsigned long long)o << 32) | code;
+                            else
+                                static_cast<uint32_t *>(a.slots)[p] = (o << 20) | code;
                         }
                     }
-                }
+                    ent += __popc(bal);
+                });
             } while (int(qn) - done >= 32 || (last && int(qn) - done > 0));
             // the rest (fewer than 32) moves to the front
             const int left = max(int(qn) - done, 0);
             uint32_t h = 0, o = 0;
             if (lane < left) {
                 h = q32[done + lane];
-                if (!RANK) o = q16[done + lane];
+                o = q16[done + lane];
             }
             __syncwarp();
             if (lane < left) {
                 q32[lane] = h;
-                if (!RANK) q16[lane] = uint16_t(o);
+                q16[lane] = uint16_t(o);
             }
             __syncwarp();
             qn = uint32_t(left);
@@ -818,7 +772,7 @@ long long table_words(const GramTables &t)
     return up4w((long long)t.filter.size()) * (t.rank ? 2 : 1);
 }
 
-long long queue_words(const GramTables &t) { return t.rank ? qcap(t.s) : qcap(t.s) + qcap(t.s) / 2; }
+long long queue_words(const GramTables &t) { return qcap(t.s) + qcap(t.s) / 2; }
 
 }  // namespace
 
@@ -893,7 +847,7 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
     // Tiles: long ones waste fewer lanes on a tile's last batch, short ones
     // spread a short text over the SMs. The workspace holds one count per
     // kWarpTile bytes, so a tile is longer than that; a mixed-length slot has
-    // 12 bits for the start, a ranked gram's queue entry 14.
+    // 12 bits for the start.
     int warps = dv.warps;
     const long long lanes = (long long)dp.sm_count * warps;
     int tile = min_tile(t.s);

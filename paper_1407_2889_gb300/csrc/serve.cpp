@@ -391,7 +391,7 @@ int launch_slot(pm_server *s, Slot &sl)
     if (kb > 0) {
         rc = batch_launch_raw(sl.d_desc, kb, base, reinterpret_cast<int64_t *>(base),
                               reinterpret_cast<uint64_t *>(base), sl.d_nocc, sl.d_ws, words, s->shape,
-                              true, sl.st);
+                              true, sl.st, batch_gram_items(items));
         if (rc == PM_OK) {
             e = cudaMemcpyAsync(sl.h_bstat, sl.d_ws, 4, cudaMemcpyDeviceToHost, sl.st);
             if (e != cudaSuccess) { set_cuda_error(int(e)); rc = PM_ECUDA; }
@@ -561,7 +561,7 @@ int rerun_one(pm_server *s, Slot &sl, Req &r, uint64_t *occ)
         if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
         uint8_t *base = s->arena.base();
         rc = batch_launch_raw(sl.d_desc, int(items.size()), base, reinterpret_cast<int64_t *>(base), occ,
-                              sl.d_nocc, sl.d_ws, words, s->shape, true, sl.st);
+                              sl.d_nocc, sl.d_ws, words, s->shape, true, sl.st, batch_gram_items(items));
     }
     if (rc) return rc;
     e = cudaMemcpyAsync(sl.h_nocc, sl.d_nocc, 8, cudaMemcpyDeviceToHost, sl.st);
