@@ -219,20 +219,29 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, doubl
             while (t.db < 24 && (size_t(1) << t.db) < G) ++t.db;
             nb = size_t(1) << t.db;
         }
-        t.dir.assign(nb + 1, 0u);
-        for (const uint32_t x : h) ++t.dir[bucket(x) + 1];
-        for (size_t b = 0; b < nb; ++b) t.dir[b + 1] += t.dir[b];
-        std::vector<uint32_t> at(t.dir.begin(), t.dir.end() - 1);
+        std::vector<uint32_t> at(nb + 1, 0u);
+        for (const uint32_t x : h) ++at[bucket(x) + 1];
+        for (size_t b = 0; b < nb; ++b) at[b + 1] += at[b];
+        t.dir.assign(2 * (nb + 1), 0u);
+        for (size_t b = 0; b <= nb; ++b) {
+            const uint32_t cnt = b < nb ? at[b + 1] - at[b] : 0u;
+            t.dir[2 * b] = at[b] | std::min(cnt, 255u) << 24;
+        }
         t.ent.resize(G);
         for (int k = t.s - 1; k >= 0; --k)
             for (size_t c = 0; c < nc; ++c) {
-                const uint32_t x = h[size_t(k) * nc + c];
-                GramEntry &e = t.ent[at[bucket(x)]++];
-                e.h = x;
-                if (t.qw == 0) e.h = codes(P + first(rep[c]) + k, len_of(rep[c]) - k);
-                e.idx = uint32_t(c);
-                e.k_len = uint32_t(k) | uint32_t(len_of(rep[c])) << 8;
-                e.code = t.code[c];
+                const uint32_t x = h[size_t(k) * nc + c], b = bucket(x), e = at[b]++;
+                GramEntry &en = t.ent[e];
+                en.h = x;
+                if (t.qw == 0) en.h = codes(P + first(rep[c]) + k, len_of(rep[c]) - k);
+                en.idx = uint32_t(c);
+                en.k_len = uint32_t(k) | uint32_t(len_of(rep[c])) << 8;
+                en.code = t.code[c];
+                const uint32_t i = e - (t.dir[2 * b] & 0xFFFFFFu);
+                for (uint32_t u = i; u < 4 && !t.rank; ++u) {
+                    t.dir[2 * b + 1] &= ~(0xFFu << (8 * u));
+                    t.dir[2 * b + 1] |= ((x >> (24 - t.db)) & 0xFFu) << (8 * u);
+                }
             }
         if (t.dense) {
             for (uint32_t c = 0; c < 4; ++c) {
@@ -273,7 +282,16 @@ void host_walk_gram(const GramTables &t, const uint8_t *T, int64_t n, std::vecto
         if (t.rank)
             bk = t.rank_base[b >> 5] + uint32_t(__builtin_popcount(t.filter[b >> 5] & ((1u << (b & 31)) - 1u)));
         else bk = x >> (32 - t.db);
-        for (uint32_t e = t.dir[bk]; e < t.dir[bk + 1]; ++e) {
+        const uint32_t first = t.dir[2 * bk] & 0xFFFFFFu;
+        uint32_t cnt = t.dir[2 * bk] >> 24;
+        if (!t.rank && cnt <= 4) {
+            bool any = false;
+            for (int u = 0; u < 4; ++u)
+                any = any || ((t.dir[2 * bk + 1] >> (8 * u)) & 0xFFu) == ((x >> (24 - t.db)) & 0xFFu);
+            if (!any) continue;
+        }
+        if (cnt == 255) cnt = (t.dir[2 * bk + 2] & 0xFFFFFFu) - first;
+        for (uint32_t e = first; e < first + cnt; ++e) {
             const GramEntry &en = t.ent[e];
             const int64_t start = p - int64_t(en.k_len & 255u), len = int64_t(en.k_len >> 8);
             if (start < 0 || start + len > n) continue;

@@ -167,7 +167,10 @@ struct GramTables {
     double cost = 0.0;             // planned instructions per lane and 16 text bytes
     std::vector<uint32_t> filter;     // 2^fb bits
     std::vector<uint32_t> rank_base;  // rank: set bits before each filter word
-    std::vector<uint32_t> dir;        // first entry of each bucket, and the end
+    // Per bucket: first entry | min(entries, 255) << 24 (255: up to the next
+    // bucket's first), and the bits of the hash below the bucket's (8 of them)
+    // of its first four entries, repeating the last; one bucket more at the end.
+    std::vector<uint32_t> dir;
     std::vector<GramEntry> ent;
     std::vector<uint32_t> pats;       // pw words (16-byte blocks) per distinct pattern, zero padded
     std::vector<uint32_t> code;       // code of each distinct pattern

@@ -49,7 +49,7 @@ struct GramArgs {
     int fwords;                   // filter words
     const uint32_t *filter_g;
     const uint32_t *rank_g;
-    const uint32_t *dir;
+    const uint2 *dir;
     const uint4 *ent;
     const uint32_t *pats;
     int pw;
@@ -190,21 +190,30 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
         }
         // ---- passing grams -> queue, row by row, lane by lane (text order) ----
         if (__any_sync(kFull, any != 0u)) {
+            // Each lane's place: with one gram a row from ballots, else from one
+            // scan of all rows' counts. A row's count stays below the next field
+            // (32 lanes x NP; four rows only up to two grams each).
+            constexpr int F = R == 4 ? 8 : 16;
+            uint32_t ex = 0, tot = 0;
+            if (NP > 1) {
+                uint32_t cnt = 0;
+#pragma unroll
+                for (int r = 0; r < R; ++r) cnt |= uint32_t(__popc(mask[r])) << (F * r);
+                const uint32_t inc = dev::warp_incl_scan(cnt, lane);
+                ex = inc - cnt;
+                tot = __shfl_sync(kFull, inc, 31);
+            }
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 uint32_t m = mask[r], at = qn;
-                if (NP <= 2) {
-#pragma unroll
-                    for (int k = 0; k < NP; ++k) {
-                        const uint32_t bal = __ballot_sync(kFull, (m >> k) & 1u);
-                        at += __popc(bal & lt);
-                        qn += __popc(bal);
-                    }
+                if (NP == 1) {
+                    const uint32_t bal = __ballot_sync(kFull, m);
+                    at += __popc(bal & lt);
+                    qn += __popc(bal);
                 } else {
-                    const uint32_t cnt = __popc(m);
-                    const uint32_t inc = dev::warp_incl_scan(cnt, lane);
-                    at += inc - cnt;
-                    qn += __shfl_sync(kFull, inc, 31);
+                    constexpr uint32_t M = (1u << F) - 1u;
+                    at += (ex >> (F * r)) & M;
+                    qn += (tot >> (F * r)) & M;
                 }
                 const uint32_t off0 = uint32_t(g * R + r) * kRow + uint32_t(lane) * 16u;
                 if (QW == 0 && NP > 1) {
@@ -234,7 +243,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
             int done = 0;
             do {
                 const int i = done + lane;
-                uint32_t e0 = 0, e1 = 0, win = 0, off = 0;
+                uint32_t e0 = 0, cnt = 0, win = 0, off = 0;
                 if (i < int(qn)) {
                     win = q32[i];
                     off = q16[i];
@@ -246,11 +255,10 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
                     } else {
                         bk = h >> a.bshift;
                     }
-                    e0 = __ldg(a.dir + bk);
-                    e1 = __ldg(a.dir + bk + 1);
+                    e0 = bucket_entries<RANK>(a.dir, bk, h >> (a.bshift - 8), cnt);
                 }
                 done += 32;
-                verify_batch<QW != 0>(view, e0, e1 - e0, win, int(off), [&](bool ok, const uint4 &en, int pos) {
+                verify_batch<QW != 0>(view, e0, cnt, win, int(off), [&](bool ok, const uint4 &en, int pos) {
                     const uint32_t bal = __ballot_sync(kFull, ok);
                     if (ok) {
                         uint32_t mult = 1u;
@@ -832,7 +840,7 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
     a.fwords = int(t.filter.size());
     a.filter_g = dv.filter;
     a.rank_g = dv.rank_base;
-    a.dir = dv.dir;
+    a.dir = reinterpret_cast<const uint2 *>(dv.dir);
     a.ent = static_cast<const uint4 *>(dv.ent);
     a.pats = dv.pats;
     a.pw = t.pw;

@@ -152,7 +152,7 @@ __device__ __noinline__ void run_gram(const BatchArgs &a, const BatchDesc &D, un
             const bool last = r0 + R >= rows;
             int done = 0;
             while (int(qn) - done >= 32 || (last && int(qn) > done)) {
-                uint32_t win = 0, e0 = 0, e1 = 0;
+                uint32_t win = 0, e0 = 0, cnt = 0;
                 int pos = 0;
                 if (done + lane < int(qn)) {
                     win = q32[done + lane];
@@ -165,11 +165,10 @@ __device__ __noinline__ void run_gram(const BatchArgs &a, const BatchDesc &D, un
                     } else {
                         bk = h >> D.g_bshift;
                     }
-                    e0 = __ldg(D.g_dir + bk);
-                    e1 = __ldg(D.g_dir + bk + 1);
+                    e0 = bucket_entries<RANK>(reinterpret_cast<const uint2 *>(D.g_dir), bk, h >> (D.g_bshift - 8), cnt);
                 }
                 done += 32;
-                verify_batch<false>(view, e0, e1 - e0, win, pos, [&](bool ok, const uint4 &en, int p) {
+                verify_batch<false>(view, e0, cnt, win, pos, [&](bool ok, const uint4 &en, int p) {
                     const uint32_t bal = __ballot_sync(kFull, ok);
                     uint32_t j0 = 0, kk = 0;
                     if (ok) {
