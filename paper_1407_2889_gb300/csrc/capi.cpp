@@ -313,12 +313,8 @@ public:
     GramJob(pm_set *s, const uint8_t *P, const int64_t *off, int64_t d, int32_t m)
     {
         if (!plan_is_automatic(s)) return;
-        // The transition-table walk of one-length Aho-Corasick sets costs about
-        // 220 instructions per lane and 16 bytes, whatever matches (d = 8000,
-        // m = 8, where one position in nine matches: 1.38 ms per GiB against
-        // 2.29 for grams of cost 360); the other scans are always slower.
-        const double limit = s->algo == PM_ALGO_AC ? 220.0 : 1e30;
-        auto work = [=]() { rc_ = build_gram(P, off, d, m, limit, s->gram); };
+        const bool limited = s->algo == PM_ALGO_AC;
+        auto work = [=]() { rc_ = build_gram(P, off, d, m, limited, s->gram); };
         if (d >= 2000) {
             try {
                 thread_ = std::thread(work);

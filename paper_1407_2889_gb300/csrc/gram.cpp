@@ -61,8 +61,13 @@ uint32_t codes(const uint8_t *p, int64_t len)
 
 }  // namespace
 
-int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, double limit, GramTables &t)
+int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool limited, GramTables &t)
 {
+    // What the transition-table walk of a one-length Aho-Corasick set costs in
+    // the same unit (about 4.6 us per GiB each): tables of fewer than about
+    // 2,000 patterns in shared memory 0.8 ms per GiB, larger ones past it 3 ms,
+    // general alphabets 4.4 ms. The other scans are always slower.
+    const double small = limited ? 170.0 : 1e30, large = limited ? 650.0 : 1e30, general = limited ? 900.0 : 1e30;
     t = GramTables();
     try {
         const bool var = off != nullptr;
@@ -95,9 +100,13 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, doubl
         // (by chance in the hashed filter, or because so many grams of the
         // alphabet are in the table), and each entry compared (G / space is
         // the mean number of entries under a gram of random text; without
-        // that term a set of 8,000 8-mers would take 1-character grams). The
-        // dense form's cost is fitted to 1,000 and 8,000 8-mers; its base is set
-        // so that 100 8-mers stay sampled (1 MiB: 19.1 us against 21.5).
+        // that term a set of 8,000 8-mers would take 1-character grams). With 40
+        // and 60 in place of 60 and 130, 2,000 12-mers over 20 letters took
+        // 4-character grams (58 us per 64 MiB against 46 with 8) and 1,000
+        // patterns of 8-16 characters every second position (155 us per 128
+        // MiB against 129). The dense form's cost is fitted to 1,000 and 8,000
+        // 8-mers; its base is set so that 100 8-mers stay sampled (1 MiB: 18.7
+        // us against 21.5).
         double best = 1e30;
         for (int s = 16; s >= 1; s >>= 1) {
             int q = std::min(16, lo - s + 1);
@@ -115,8 +124,8 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, doubl
             const double chance = direct ? 0.0 : 1.0 - std::exp(-G / double(1u << fb));
             const double pass = 1.0 - (1.0 - natural) * (1.0 - chance);
             const double probes = 16.0 / s;
-            const double cost = dense ? 110.0 + probes * 74.0 * pass
-                                      : 24.0 + probes * ((packed ? 9.0 : 8.0 + q / 4) + 40.0 * pass + 60.0 * G / space);
+            const double cost = dense ? 125.0 + probes * 74.0 * pass
+                                      : 24.0 + probes * ((packed ? 9.0 : 8.0 + q / 4) + 60.0 * pass + 130.0 * G / space);
             if (cost < best) {
                 best = cost;
                 t.s = s;
@@ -127,9 +136,9 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, doubl
                 t.dense = dense;
             }
         }
-        // too short for any gram, too many patterns, or so many matches that
+        // too short for any gram, too many patterns, or so many candidates that
         // the automaton is faster
-        if (t.s == 0 || (best > limit && !t.dense)) {
+        if (t.s == 0 || (!t.dense && best > (packed ? (d < 2000 ? small : large) : general))) {
             t = GramTables();
             return PM_OK;
         }

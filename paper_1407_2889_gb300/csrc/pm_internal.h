@@ -185,9 +185,9 @@ struct GramTables {
 
 int build_ac(const uint8_t *P, int64_t d, int32_t m, AcTables &out);
 // off NULL: d rows of length m; else pattern r is P[off[r] .. off[r+1]).
-// t.ok stays false (and PM_OK is returned) when the set has no gram plan or
-// its planned cost (instructions per lane and 16 text bytes) exceeds `limit`.
-int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, double limit, GramTables &t);
+// t.ok stays false (and PM_OK is returned) when the set has no gram plan or,
+// `limited`, when walking its transition table is planned to be faster.
+int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool limited, GramTables &t);
 void host_walk_gram(const GramTables &t, const uint8_t *T, int64_t n,
                     std::vector<uint64_t> &occ, std::vector<int64_t> &counts);
 // pattern r is P[off[r] .. off[r+1]); lengths 1..kAcvMaxLen
@@ -422,10 +422,12 @@ int gram_plan(const GramTables &t, const DeviceProps &dp, DevGram &dev);
 int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, int64_t n, bool list,
                 int64_t *d_counts, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ, const GramWs &ws,
                 const unsigned long long *occ_base, unsigned long long pos_base, void *stream);
-// gram_launch over a list workspace (list_workspace_parts with these sizes)
+// A whole scan over a list workspace (list_workspace_parts with these sizes):
+// zeroes what must start at zero (first: counts, total, header and segment
+// sums; else the segment sums only, of a later chunk of a longer scan).
 int gram_launch_ws(const GramTables &t, const DevGram &dv, const uint8_t *d_text, int64_t n, bool list,
                    int64_t *d_counts, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ, void *d_ws,
-                   int64_t nterms, int slot_bytes, int per_pos, const unsigned long long *occ_base,
+                   int64_t nterms, int slot_bytes, int per_pos, bool first, const unsigned long long *occ_base,
                    unsigned long long pos_base, void *stream);
 // two characters per lookup (scan_ac2.cu): plan (PM_ETOOBIG if the set is
 // not eligible or the tables do not fit) and scan on the AC workspace

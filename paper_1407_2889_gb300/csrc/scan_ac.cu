@@ -146,6 +146,7 @@ expand_kernel(const SE *__restrict__ slots, const uint32_t *__restrict__ tile_en
               const ExpandLateArgs late, long long any_tile, long long any_stride)
 {
     const long long tile = ANY ? any_tile : kWarpTile, slot_stride = ANY ? any_stride : kWarpTile;
+    if (ANY) dev::grid_wait();
     typedef typename std::conditional<sizeof(SE) == 4, uint16_t, uint32_t>::type CE;
     constexpr bool LATE = CM != 0;
     extern __shared__ __align__(16) unsigned char esm[];
@@ -827,6 +828,9 @@ int ac_enqueue(const AcTables &t, const DevAc &dv, const uint8_t *d_text, int64_
     DeviceProps dp;
     int rc = device_props(dp);
     if (rc) return rc;
+    if (dv.dg && n >= t.m && nsub > 0)
+        return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, nterms, se, 1,
+                              first, occ_base, pos_base, st);
     const AcWsLayout L = ac_ws_layout(nsub, list, nterms, se, dp.sm_count);
     // every segment non-empty: at most ac_segments() of them
     const long long seg_tiles = (nsub + ac_segments(nsub, dp.sm_count) - 1) / ac_segments(nsub, dp.sm_count);
@@ -849,10 +853,6 @@ int ac_enqueue(const AcTables &t, const DevAc &dv, const uint8_t *d_text, int64_
         if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
         return PM_OK;
     }
-
-    if (dv.dg)
-        return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, nterms, se, 1,
-                              occ_base, pos_base, st);
 
     // list mode has its own layout (with late ids: no counters, maybe more warps)
     const bool late = list && !pfac && dv.ids_smem == 2;
@@ -1006,17 +1006,21 @@ int expand_enqueue(const ExpandTiles &tl, const uint32_t *grp_off, const uint32_
     const long long ngo = grp_smem ? n_grp_off : 0, ngi = grp_smem ? n_grp_ids : 0;
     esmem += (ngo + ngi) * 4;
     long long *n_occ = reinterpret_cast<long long *>(d_n_occ);
+    const bool any = tl.tile != kWarpTile || tl.slot_stride != kWarpTile;  // the gram scans: never with late ids
     auto go = [&](auto kern, const auto *slots) -> cudaError_t {
         if (esmem > (48 << 10)) {
             const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(esmem));
             if (ea != cudaSuccess) return ea;
         }
+        if (any)
+            return dev::launch_dependent(kern, dim3(unsigned(nseg)), dim3(kExpandThreads), size_t(esmem), st, slots,
+                                         tl.tile_ent, tl.tile_out, tl.seg_sum, nseg, seg_tiles, tl.ntiles, grp_off, grp_ids,
+                                         occ, cap, n_occ, occ_base, pos_base, ngo, ngi, la, tl.tile, tl.slot_stride);
         kern<<<unsigned(nseg), kExpandThreads, size_t(esmem), st>>>(
             slots, tl.tile_ent, tl.tile_out, tl.seg_sum, nseg, seg_tiles, tl.ntiles, grp_off, grp_ids, occ, cap, n_occ,
             occ_base, pos_base, ngo, ngi, la, tl.tile, tl.slot_stride);
         return cudaGetLastError();
     };
-    const bool any = tl.tile != kWarpTile || tl.slot_stride != kWarpTile;  // never with late ids
     const int cm = !is_late ? 0 : la.smem == 1 ? 1 : la.smem == 2 ? 2 : 3;
     // one instance per slot width, counter mode and group-table placement
     auto pick = [&](auto se_tag) -> cudaError_t {

@@ -516,6 +516,9 @@ int acv_launch(const AcvTables &v, const DevAcv &dv, const uint8_t *d_text, int6
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long nsub = warp_tiles(n);
     const int se = acv_slot_bytes(v);
+    if (dv.dg && n >= v.m_min && nsub > 0)
+        return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, 0, se * v.K,
+                              v.K, true, nullptr, 0, stream);
     ListParts L;
     list_workspace_parts(d_ws, nsub, 0, se * v.K, L);
     cudaError_t e = cudaMemsetAsync(d_counts, 0, size_t(v.ac.d) * sizeof(int64_t), st);
@@ -523,9 +526,6 @@ int acv_launch(const AcvTables &v, const DevAcv &dv, const uint8_t *d_text, int6
     if (e == cudaSuccess) e = cudaMemsetAsync(d_ws, 0, size_t(list ? L.zeroed_bytes : kWsHeader), st);
     if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
     if (n < v.m_min || nsub == 0) return PM_OK;
-    if (dv.dg)
-        return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, 0, se * v.K,
-                              v.K, nullptr, 0, stream);
 
     const AcvKernel fn = kAcvVariants[dv.variant].fn;
     int rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), dv.smem_bytes);

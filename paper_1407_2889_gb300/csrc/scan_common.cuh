@@ -192,5 +192,29 @@ segment_offsets(const uint32_t *tile_ent, const uint32_t *tile_out, const unsign
     return run;
 }
 
+// Kernels of one scan follow one another in a stream and each starts with work
+// that does not need the one before (table loads): launched as programmatic
+// dependents they do that work while the other still runs. Every such kernel
+// calls grid_wait() before it reads or writes what earlier kernels touch, and
+// the kernels before it let it start early with grid_trigger().
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, P(args)...);
+}
+
 }  // namespace dev
 }  // namespace pm

@@ -100,7 +100,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
     }
     if (a.hist_smem)
         for (int i = threadIdx.x; i < a.ncodes; i += blockDim.x) s_hist[i] = 0u;
+    dev::grid_trigger();
     __syncthreads();
+    dev::grid_wait();   // the zeroed counts and sums
 
     const uint32_t ntiles = uint32_t(a.ntiles);
     const uint32_t G = gridDim.x * (blockDim.x >> 5);
@@ -424,6 +426,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_dense_kernel(const Den
         }
         __syncthreads();
     }
+    // no grid_trigger: expand CTAs that start while scan CTAs still run crowd on
+    // the SMs that finish first (1.24 ms per GiB in place of 1.13)
+    dev::grid_wait();   // the zeroed counts and sums
 
     // A warp takes a run of consecutive tiles, so that a row's characters
     // after the last lane are the next row's, packed once.
@@ -641,6 +646,7 @@ dense_expand_kernel(const uint32_t *__restrict__ slots, const uint32_t *__restri
         for (int i = tid; i <= nc; i += T) s_io[i] = __ldg(id_off + i);
         for (int i = tid; i < d; i += T) s_id[i] = __ldg(ids + i);
     }
+    dev::grid_wait();   // the scan's tiles and slots
     const unsigned long long run = dev::segment_offsets<T>(tile_ent, tile_out, seg_sum, blockIdx.x, t0, nt, occ_base,
                                                            tile, s_off, s_ent, s_red);
     if (tid == T - 1 && t0 + nt == ntiles) *n_occ = (long long)run;
@@ -718,6 +724,21 @@ long long dense_smem(const GramTables &t, bool pair, int warps)
            2 * (long long)warps * kDenseQueue + nc;
 }
 
+// Zeroes what a scan adds to: one launch in place of three memsets, which cost
+// about 1.5 us each, and the scan kernel loads its tables meanwhile.
+struct ZeroArgs {
+    unsigned long long *p[3];
+    long long n[3];               // 8-byte words
+};
+
+__global__ void __launch_bounds__(256) gram_zero_kernel(const ZeroArgs z, int64_t *n_occ)
+{
+    dev::grid_trigger();
+    if (n_occ && blockIdx.x == 0 && threadIdx.x == 0) *n_occ = 0;
+    for (int k = 0; k < 3; ++k)
+        for (long long i = blockIdx.x * 256LL + threadIdx.x; i < z.n[k]; i += gridDim.x * 256LL) z.p[k][i] = 0ull;
+}
+
 typedef void (*DenseKernel)(const DenseArgs);
 
 DenseKernel dense_kernel_of(const GramTables &t, bool pair)
@@ -739,11 +760,11 @@ int dense_expand(const GramTables &t, const DevGram &dv, const GramArgs &a, cons
     const auto fn = sm ? dense_expand_kernel<true> : dense_expand_kernel<false>;
     const int rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), smem);
     if (rc) return rc;
-    fn<<<unsigned((a.ntiles + a.seg_tiles - 1) / a.seg_tiles), kDenseExpandThreads, size_t(smem), st>>>(
+    const cudaError_t e = dev::launch_dependent(
+        fn, dim3(unsigned((a.ntiles + a.seg_tiles - 1) / a.seg_tiles)), dim3(kDenseExpandThreads), size_t(smem), st,
         static_cast<const uint32_t *>(ws.slots), ws.tile_ent, ws.tile_out, ws.seg_sum, a.seg_tiles, a.ntiles,
         uint32_t(a.tile), dv.id_off, dv.ids, nc, int(t.d), reinterpret_cast<unsigned long long *>(d_occ),
-        d_occ ? occ_cap : 0, reinterpret_cast<long long *>(d_n_occ), occ_base, pos_base);
-    const cudaError_t e = cudaGetLastError();
+        (long long)(d_occ ? occ_cap : 0), reinterpret_cast<long long *>(d_n_occ), occ_base, pos_base);
     if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
     return PM_OK;
 }
@@ -882,6 +903,7 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
     const long long want = (a.ntiles + warps - 1) / warps;
     if (want < grid) grid = want;
     const dim3 gd{unsigned(grid)}, bd{unsigned(warps * 32)};
+    cudaError_t e = cudaSuccess;
     if (t.dense) {
         DenseArgs da;
         da.a = a;
@@ -899,17 +921,16 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
         const DenseKernel fn = dense_kernel_of(t, pair);
         rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), smem);
         if (rc) return rc;
-        fn<<<gd, bd, size_t(smem), st>>>(da);
+        e = dev::launch_dependent(fn, gd, bd, size_t(smem), st, da);
     } else {
         const GramKernel fn = kernel_of(t);
         const long long smem =
             4 * (table_words(t) + (dv.hist_smem ? up4w(a.ncodes) : 0) + (long long)warps * queue_words(t));
         rc = kernel_smem_attr(reinterpret_cast<const void *>(fn), smem);
         if (rc) return rc;
-        fn<<<gd, bd, size_t(smem), st>>>(a);
+        e = dev::launch_dependent(fn, gd, bd, size_t(smem), st, a);
     }
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
+    if (e != cudaSuccess) { set_cuda_error(int(e)); cudaGetLastError(); return PM_ECUDA; }
     if (!list) return PM_OK;
     if (t.dense) return dense_expand(t, dv, a, ws, dp, d_occ, occ_cap, d_n_occ, occ_base, pos_base, st);
     ExpandTiles tl;
@@ -928,7 +949,7 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
 
 int gram_launch_ws(const GramTables &t, const DevGram &dv, const uint8_t *d_text, int64_t n, bool list,
                    int64_t *d_counts, uint64_t *d_occ, int64_t occ_cap, int64_t *d_n_occ, void *d_ws,
-                   int64_t nterms, int slot_bytes, int per_pos, const unsigned long long *occ_base,
+                   int64_t nterms, int slot_bytes, int per_pos, bool first, const unsigned long long *occ_base,
                    unsigned long long pos_base, void *stream)
 {
     ListParts L;
@@ -940,6 +961,22 @@ int gram_launch_ws(const GramTables &t, const DevGram &dv, const uint8_t *d_text
     ws.slots = L.slots;
     ws.segs = L.segs;
     ws.per_pos = per_pos;
+    ZeroArgs z{};
+    if (list) {
+        z.p[0] = L.seg_sum;
+        z.n[0] = (static_cast<char *>(d_ws) + L.zeroed_bytes - reinterpret_cast<char *>(L.seg_sum)) / 8;
+    }
+    if (first) {
+        z.p[1] = reinterpret_cast<unsigned long long *>(d_counts);
+        z.n[1] = t.d;
+        z.p[2] = static_cast<unsigned long long *>(d_ws);
+        z.n[2] = kWsHeader / 8;
+    }
+    const long long words = std::max<long long>(z.n[0] + z.n[1] + z.n[2], 1);
+    gram_zero_kernel<<<unsigned(std::min<long long>((words + 255) / 256, 1024)), 256, 0,
+                       static_cast<cudaStream_t>(stream)>>>(z, first ? d_n_occ : nullptr);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
     return gram_launch(t, dv, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, ws, occ_base, pos_base, stream);
 }
 

@@ -612,6 +612,9 @@ int wm_launch(const WmTables &t, const DevWm &dv, const uint8_t *d_text, int64_t
     const long long ntiles = warp_tiles(n);
     const int se = t.var ? wmv_slot_bytes(t) : wm_slot_bytes(t);
     const int per_pos = t.var ? t.K : 1;
+    if (dv.dg && n >= t.m && ntiles > 0)
+        return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, 0, se * per_pos,
+                              per_pos, true, nullptr, 0, stream);
     ListParts L;
     list_workspace_parts(d_ws, ntiles, 0, se * per_pos, L);
     const int64_t zeroed = list ? L.zeroed_bytes : kWsHeader;
@@ -620,10 +623,6 @@ int wm_launch(const WmTables &t, const DevWm &dv, const uint8_t *d_text, int64_t
     if (e == cudaSuccess) e = cudaMemsetAsync(d_ws, 0, size_t(zeroed), st);
     if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
     if (n < t.m || ntiles == 0) return PM_OK;
-
-    if (dv.dg)
-        return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, 0, se * per_pos,
-                              per_pos, nullptr, 0, stream);
 
     typedef void (*K)(const WmArgs);
     const int nv = wm_nv(t.m);

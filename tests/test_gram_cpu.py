@@ -49,7 +49,7 @@ def test_one_length(alphabet, m):
                     occ, cnt = pm.pm_selfcheck_gram_walk(h, T)
                 except pm.PmError as e:
                     assert e.code == pm.PM_EINVAL  # no gram fits, or too many matches
-                    assert m < 3 or len(alphabet) ** min(m, 16) < 40 * d
+                    assert m < 3 or len(alphabet) ** min(m, 16) < 80 * d
                     continue
                 assert np.array_equal(occ, want[0]) and np.array_equal(cnt, want[1]), (alphabet, m, d)
             finally:
