@@ -50,14 +50,15 @@ __device__ __forceinline__ void run_item(const BatchArgs &a, const BatchDesc &D,
         ocap = (unsigned long long)D.spill_cap;
     }
     const unsigned long long total = pass(true, staged, 0ull);
-    if (threadIdx.x == 0) {
-        dev::st_relaxed(&pstat[D.part], (1ull << 63) | total);
+    if (threadIdx.x == 0) dev::st_relaxed(&pstat[D.part], (1ull << 63) | total);
+    if (threadIdx.x < 32) {
+        // the parts before this one were taken earlier by running CTAs, and
+        // publish their totals without waiting for anything; a lane waits for
+        // every 32nd of them (one thread after another took 0.7 us a part)
         unsigned long long base = 0;
         if (a.list) {
-            // the parts before this one were taken earlier by running CTAs,
-            // and publish their totals without waiting for anything
             const long long t0c = clock64();
-            for (int q = 0; q < D.part; ++q) {
+            for (int q = threadIdx.x; q < D.part; q += 32) {
                 unsigned long long v = dev::ld_relaxed(&pstat[q]);
                 while (!(v >> 63)) {
                     if (clock64() - t0c > dev::kSpinLimit) {
@@ -69,8 +70,11 @@ __device__ __forceinline__ void run_item(const BatchArgs &a, const BatchDesc &D,
                 }
                 base += v & ~(1ull << 63);
             }
+            __syncwarp();
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(dev::kFull, base, o);
         }
-        s_base = base;
+        if (threadIdx.x == 0) s_base = base;
     }
     __syncthreads();
     if (a.list) {

@@ -505,6 +505,7 @@ struct BatchDesc {                 // one instance, in processing order
     // gram items (gram_batch_kernel): the set's gram tables (see GramTables)
     int gram, tile;                // tile: text bytes a warp takes at a time
     int g_s, g_rank, g_fwords, g_pw;
+    int g_direct, g_pad;           // filter probed in device memory
     uint32_t g_k, g_fshift, g_wshift, g_bshift;
     const uint32_t *g_filter, *g_rank_base, *g_dir, *g_pats, *g_code, *g_grp_off, *g_grp_ids;
     const void *g_ent;

@@ -512,6 +512,13 @@ int64_t batch_fill(const BatchInst *inst, int k, const BatchShape &sh, BatchDesc
     return ccount;
 }
 
+// Most parts an instance is split into: two rounds of tiles each, or 10 KiB of
+// a gram item (whose matches may cost far more than its text)
+static long long max_parts(const InstLayout &L, long long ntiles, int warps)
+{
+    return ntiles / (L.gram ? 4LL : 2LL * warps);
+}
+
 int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool list, std::vector<BatchDesc> &out,
                     int64_t *spill_words)
 {
@@ -532,7 +539,9 @@ int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool lis
         const long long entries = (long long)t.n_rows << t.lw;
         if (L.gram)
             cost[size_t(q)] = double(inst[q].text_len) * (30.0 + inst[q].set->gram.cost) +
-                              30.0 * 4.0 * double(inst[q].set->gram.filter.size()) + 1.0e6;
+                              30.0 * 4.0 * double(inst[q].set->gram.filter.size()) + 1.0e6 +
+                              // each pattern may occur once: a match costs as much as 200 bytes
+                              1.0e4 * std::min(double(t.canon.size()), double(inst[q].text_len) / 4.0);
         else
             cost[size_t(q)] = double(inst[q].text_len) * (L.smem_entries >= entries ? 1.0 : 4.0) +
                               4.0 * double(L.smem_entries * t.entry_bytes);
@@ -556,7 +565,7 @@ int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool lis
         const double share = total[L.gram ? 0 : 1] / ((L.gram ? 8.0 : 4.0) * double(std::max(sh.sm_count, 1)));
         if (cost[size_t(q)] > share && share > 0.0) {
             parts = (long long)std::ceil(cost[size_t(q)] / share);
-            parts = std::min(parts, ntiles / (2LL * sh.warps));  // at least two rounds of tiles each
+            parts = std::min(parts, max_parts(L, ntiles, sh.warps));
             parts = std::max(parts, 1LL);
         }
         int64_t coff = ccount;
@@ -597,7 +606,7 @@ int64_t batch_words_bound(const BatchInst &I, const BatchShape &sh, bool list)
     const AcTables &t = I.set->ac;
     const InstLayout L = layout_of(I.set, sh.region_bytes, sh.policy);
     const long long ntiles = (I.text_len + kWarpTile - 1) / kWarpTile;
-    const long long parts = std::max(1LL, ntiles / (2LL * std::max(sh.warps, 1)));
+    const long long parts = std::max(1LL, max_parts(L, ntiles, std::max(sh.warps, 1)));
     int64_t w = (L.hist_off < 0 || parts > 1) ? int64_t(t.canon.size()) : 0;
     if (parts > 1) {
         w += parts + 1;

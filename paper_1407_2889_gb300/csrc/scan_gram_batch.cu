@@ -14,7 +14,7 @@
 // Against walking the transition tables this removes the per-character
 // lookups, many of which read table rows past the shared-memory prefix from L2
 // or DRAM: 1,024 instances (0.58 GB of text, 10 to 10,000 patterns each) took
-// 2.87 ms, and take 0.61. What is left is latency: warps wait at the round's
+// 2.87 ms, and take 0.43. What is left is latency: warps wait at the round's
 // barrier and for the entries and patterns of candidates, which nothing has
 // brought into L2 (issue slots 29 % in use).
 #include <algorithm>
@@ -29,8 +29,8 @@ namespace {
 using dev::kFull;
 using namespace gramdev;
 
-constexpr int kWarps = 32;
-constexpr int kHits = 96;            // matches a warp keeps per tile
+constexpr int kWarps = 24;           // with 32 (64 registers) the walk spills: 570 us for the batch above against 502
+constexpr int kHits = 192;           // matches a warp keeps per tile
 constexpr int kMaxTile = 32768;      // a match's offset has 16 bits
 
 // rows per load batch, and a warp's queue
@@ -58,9 +58,21 @@ __device__ __noinline__ void run_gram(const BatchArgs &a, const BatchDesc &D, un
     uint32_t *s_rank = s_filter + D.g_fwords;
     uint32_t *s_hist = D.hist_off >= 0 ? s_filter + D.hist_off / 4 : nullptr;
     unsigned long long *g_hist = a.ccount + D.ccount_off;
-    for (int i = threadIdx.x; i < D.g_fwords / 4; i += blockDim.x) {
-        reinterpret_cast<uint4 *>(s_filter)[i] = __ldg(reinterpret_cast<const uint4 *>(D.g_filter) + i);
-        if (RANK) reinterpret_cast<uint4 *>(s_rank)[i] = __ldg(reinterpret_cast<const uint4 *>(D.g_rank_base) + i);
+    // a short item probes the filter where it is: loading it takes longer
+    const uint32_t *filter = D.g_direct ? D.g_filter : s_filter;
+    const uint32_t *rank = D.g_direct ? D.g_rank_base : s_rank;
+    if (!D.g_direct) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(D.g_filter);
+        uint4 *dst = reinterpret_cast<uint4 *>(s_filter);
+        const int nv = D.g_fwords / 4;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < nv; i += kWarps * 32) dst[i] = __ldg(src + i);
+        if (RANK) {
+            const uint4 *rs = reinterpret_cast<const uint4 *>(D.g_rank_base);
+            uint4 *rd = reinterpret_cast<uint4 *>(s_rank);
+#pragma unroll 4
+            for (int i = threadIdx.x; i < nv; i += kWarps * 32) rd[i] = __ldg(rs + i);
+        }
     }
     if (s_hist)
         for (int i = threadIdx.x; i < D.nterms; i += blockDim.x) s_hist[i] = 0u;
@@ -125,7 +137,7 @@ __device__ __noinline__ void run_gram(const BatchArgs &a, const BatchDesc &D, un
 #pragma unroll
                 for (int k = 0; k < NP; ++k) {
                     const uint32_t win = k == 0 ? cl[r] : __funnelshift_r(cl[r], ch[r], 2 * S * k);
-                    const uint32_t w = s_filter[(win * K0) >> D.g_wshift];
+                    const uint32_t w = filter[(win * K0) >> D.g_wshift];
                     m = __funnelshift_r(m, __funnelshift_r(w, 0u, win), 1);
                 }
                 mask[r] = r0 + r < rows ? m >> (32 - NP) : 0u;
@@ -161,7 +173,7 @@ __device__ __noinline__ void run_gram(const BatchArgs &a, const BatchDesc &D, un
                     uint32_t bk;
                     if (RANK) {
                         const uint32_t b = h >> D.g_fshift;
-                        bk = s_rank[b >> 5] + __popc(s_filter[b >> 5] & ~(kFull << (b & 31u)));
+                        bk = rank[b >> 5] + __popc(filter[b >> 5] & ~(kFull << (b & 31u)));
                     } else {
                         bk = h >> D.g_bshift;
                     }
@@ -228,7 +240,7 @@ __device__ __noinline__ void run_gram(const BatchArgs &a, const BatchDesc &D, un
             }
             if (lane == 0) s_tot[warp] = keys;
             __syncthreads();
-            const uint32_t tot = uint32_t(s_tot[lane]);
+            const uint32_t tot = lane < kWarps ? uint32_t(s_tot[lane]) : 0u;
             const uint32_t inc = dev::warp_incl_scan(tot, lane);
             const uint32_t before = __shfl_sync(kFull, inc - tot, warp);
             const unsigned long long base = running + before;
@@ -324,8 +336,8 @@ bool gram_batch_layout(const GramTables &t, int &hist_off, int &tile)
 {
     if (!t.ok || t.var || t.qw != 0) return false;
     const long long room = smem_budget() - rr16((long long)kWarps * bwarp_bytes(t.s));
-    const long long tab = (long long)t.filter.size() * 4 * (t.rank ? 2 : 1);
     const long long nc = (long long)t.code.size();
+    const long long tab = (long long)t.filter.size() * 4 * (t.rank ? 2 : 1);
     if (tab > room || t.filter.size() % 4 != 0) return false;
     hist_off = tab + nc * 4 <= room ? int(tab) : -1;
     // tiles of at most about 48 expected matches
@@ -343,6 +355,7 @@ void gram_batch_fill(const GramTables &t, const DevGram &dv, int tile, BatchDesc
     D.g_s = t.s;
     D.g_rank = t.rank ? 1 : 0;
     D.g_fwords = int(t.filter.size());
+    D.g_direct = 0;
     D.g_pw = t.pw;
     D.g_k = t.K[0];
     D.g_fshift = uint32_t(32 - t.fb);
@@ -359,8 +372,11 @@ void gram_batch_fill(const GramTables &t, const DevGram &dv, int tile, BatchDesc
     D.nterms = int(t.code.size());
 }
 
-int gram_batch_tile(const BatchDesc &D, int most)
+int gram_batch_tile(BatchDesc &D, int most)
 {
+    // 128 KiB of filter load in about 4 us; as many probes from L2 as a text of
+    // a quarter of that makes take less
+    D.g_direct = (D.t_hi - D.t_lo) * kWarpTile <= (long long)D.g_fwords ? 1 : 0;
     // as few rounds as the matches allow, and every warp an equal share
     const long long bytes = std::min(D.t_hi * kWarpTile, D.n) - D.t_lo * kWarpTile;
     const int step = kRow;

@@ -11,8 +11,9 @@ namespace pm {
 // bytes a warp takes at a time.
 bool gram_batch_layout(const GramTables &t, int &hist_off, int &tile);
 void gram_batch_fill(const GramTables &t, const DevGram &dv, int tile, BatchDesc &D);
-// the tile length of an item whose range is set, at most `most`
-int gram_batch_tile(const BatchDesc &D, int most);
+// the tile length of an item whose range is set, at most `most`; also decides
+// whether the item's filter is probed in device memory
+int gram_batch_tile(BatchDesc &D, int most);
 int gram_batch_attr();  // raises the kernel's shared memory limit (before any capture)
 int gram_batch_enqueue(const BatchArgs &a, int grid, void *stream);
 
