@@ -79,8 +79,10 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
             if (off[r + 1] <= off[r] || off[r + 1] - off[r] > 255) return PM_OK;
         bool present[256] = {};
         int lo = 1 << 30, hi = 0;
+        int64_t with_len[256] = {};
         for (int64_t r = 0; r < d; ++r) {
             const int L = len_of(r);
+            ++with_len[L];
             lo = std::min(lo, L);
             hi = std::max(hi, L);
             const uint8_t *p = P + first(r);
@@ -107,33 +109,51 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
         // MiB against 129). The dense form's cost is fitted to 1,000 and 8,000
         // 8-mers; its base is set so that 100 8-mers stay sampled (1 MiB: 18.7
         // us against 21.5).
+        //
+        // 2-bit grams may be longer than the shortest rest m - s + 1: a gram of
+        // which the pattern has only the first L characters enters with all 4^(q
+        // - L) endings. Up to 10 characters the filter is exact, so this turns
+        // away most windows of the longer patterns in a mixed set: 8,000 of 8 to
+        // 16 characters with 8-character grams took 567 us per 256 MiB, 1,000
+        // 121 us per 128 MiB.
         double best = 1e30;
         for (int s = 16; s >= 1; s >>= 1) {
-            int q = std::min(16, lo - s + 1);
-            if (!packed) q &= ~3;
-            if (q < (packed ? 3 : 4)) continue;
-            const double G = double(d) * s;
-            if (G > 8.0e6) continue;
-            const double space = std::pow(double(std::max(letters, 2)), double(q));
-            const double natural = 1.0 - std::exp(-G / space);
-            const bool direct = packed && 2 * q <= 18;
-            const bool dense = direct && s == 1 && !var && q == hi && d < 32768;
-            int fb = direct ? 2 * q : 12;
-            if (!direct)
-                while (fb < 20 && double(1u << fb) < 32.0 * G) ++fb;
-            const double chance = direct ? 0.0 : 1.0 - std::exp(-G / double(1u << fb));
-            const double pass = 1.0 - (1.0 - natural) * (1.0 - chance);
-            const double probes = 16.0 / s;
-            const double cost = dense ? 125.0 + probes * 74.0 * pass
-                                      : 24.0 + probes * ((packed ? 9.0 : 8.0 + q / 4) + 60.0 * pass + 130.0 * G / space);
-            if (cost < best) {
-                best = cost;
-                t.s = s;
-                t.q = q;
-                t.qw = packed ? 0 : q / 4;
-                t.fb = fb;
-                t.rank = direct;
-                t.dense = dense;
+            const int shortest = lo - s + 1;
+            for (int form = 0; form < (packed ? 3 : 1); ++form) {
+                int q = form == 0 ? std::min(16, shortest) : form == 1 ? 9 : 10;
+                if (!packed) q &= ~3;
+                if (q < (packed ? 3 : 4) || shortest < 1 || (form > 0 && q <= shortest)) continue;
+                // entries, and how many of them a gram of random text has
+                double G = 0.0, hits = 0.0;
+                for (int L = lo; L <= hi; ++L)
+                    for (int k = 0; k < s && with_len[L]; ++k) {
+                        const int have = std::min(q, L - k);
+                        G += double(with_len[L]) * std::pow(4.0, double(q - have));
+                        hits += double(with_len[L]) / std::pow(double(std::max(letters, 2)), double(have));
+                    }
+                if (G > (form == 0 ? 8.0e6 : 4.0e5)) continue;
+                const bool direct = packed && 2 * q <= 20 && (form > 0 || 2 * q <= 18);
+                const bool dense = form == 0 && direct && s == 1 && !var && q == hi && d < 32768;
+                int fb = direct ? 2 * q : 12;
+                if (!direct)
+                    while (fb < 20 && double(1u << fb) < 32.0 * G) ++fb;
+                const double natural = 1.0 - std::exp(-hits);
+                const double chance = direct ? 0.0 : 1.0 - std::exp(-G / double(1u << fb));
+                const double pass = 1.0 - (1.0 - natural) * (1.0 - chance);
+                const double probes = 16.0 / s;
+                double cost = dense ? 125.0 + probes * 74.0 * pass
+                                    : 24.0 + probes * ((packed ? 9.0 : 8.0 + q / 4) + 60.0 * pass + 130.0 * hits);
+                if (form == 2) cost += 10.0;  // 128 KiB of filter to load
+                if (cost < best) {
+                    best = cost;
+                    t.s = s;
+                    t.q = q;
+                    t.qw = packed ? 0 : q / 4;
+                    t.fb = fb;
+                    t.direct = direct;
+                    t.rank = direct && 2 * q <= 18;
+                    t.dense = dense;
+                }
             }
         }
         // too short for any gram, too many patterns, or so many candidates that
@@ -148,7 +168,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
         t.m_min = lo;
         t.m_max = hi;
         for (int w = 0; w < 4; ++w) t.K[w] = kMul[w];
-        if (packed) t.K[0] = (t.rank ? 1u : kMul[0]) << (32 - 2 * t.q);
+        if (packed) t.K[0] = (t.direct ? 1u : kMul[0]) << (32 - 2 * t.q);
 
         // distinct patterns of a one-length set (groups of equal patterns, as
         // in the other tables); every pattern of its own in a mixed one
@@ -200,15 +220,31 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
         // entries, bucket-major; inside a bucket by (k descending, pattern
         // ascending), so that the starts t - k come out in ascending order
         // and equal starts in ascending pattern id
-        const size_t G = nc * size_t(t.s);
-        std::vector<uint32_t> h(G);
+        struct Gram {
+            uint32_t h, c, k;
+        };
+        std::vector<Gram> grams;
+        grams.reserve(nc * size_t(t.s));
         t.filter.assign(size_t(1) << (t.fb - 5), 0u);
-        for (int k = 0; k < t.s; ++k)
+        for (int k = t.s - 1; k >= 0; --k)
             for (size_t c = 0; c < nc; ++c) {
-                uint32_t b;
-                h[size_t(k) * nc + c] = gram_hash(t, P + first(rep[c]) + k, &b);
-                t.filter[b >> 5] |= 1u << (b & 31);
+                const uint8_t *p = P + first(rep[c]) + k;
+                const int have = len_of(rep[c]) - k;
+                if (have >= t.q) {
+                    uint32_t b;
+                    const uint32_t x = gram_hash(t, p, &b);
+                    t.filter[b >> 5] |= 1u << (b & 31u);
+                    grams.push_back({x, uint32_t(c), uint32_t(k)});
+                    continue;
+                }
+                const uint32_t head = codes(p, have);   // direct grams: every ending
+                for (uint32_t e = 0; e < 1u << (2 * (t.q - have)); ++e) {
+                    const uint32_t b = head | e << (2 * have);
+                    t.filter[b >> 5] |= 1u << (b & 31u);
+                    grams.push_back({b * t.K[0], uint32_t(c), uint32_t(k)});
+                }
             }
+        const size_t G = grams.size();
         auto bucket = [&](uint32_t x) -> uint32_t {
             if (!t.rank) return x >> (32 - t.db);
             const uint32_t b = x >> (32 - t.fb);
@@ -224,12 +260,14 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
             }
             nb = run;
         } else {
-            t.db = 8;
+            // (a pattern's endings are the top bits of direct grams and at most
+            // as many as there are buckets: they fall into different ones)
+            t.db = 12;
             while (t.db < 24 && (size_t(1) << t.db) < G) ++t.db;
             nb = size_t(1) << t.db;
         }
         std::vector<uint32_t> at(nb + 1, 0u);
-        for (const uint32_t x : h) ++at[bucket(x) + 1];
+        for (const Gram &x : grams) ++at[bucket(x.h) + 1];
         for (size_t b = 0; b < nb; ++b) at[b + 1] += at[b];
         t.dir.assign(2 * (nb + 1), 0u);
         for (size_t b = 0; b <= nb; ++b) {
@@ -237,21 +275,20 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
             t.dir[2 * b] = at[b] | std::min(cnt, 255u) << 24;
         }
         t.ent.resize(G);
-        for (int k = t.s - 1; k >= 0; --k)
-            for (size_t c = 0; c < nc; ++c) {
-                const uint32_t x = h[size_t(k) * nc + c], b = bucket(x), e = at[b]++;
-                GramEntry &en = t.ent[e];
-                en.h = x;
-                if (t.qw == 0) en.h = codes(P + first(rep[c]) + k, len_of(rep[c]) - k);
-                en.idx = uint32_t(c);
-                en.k_len = uint32_t(k) | uint32_t(len_of(rep[c])) << 8;
-                en.code = t.code[c];
-                const uint32_t i = e - (t.dir[2 * b] & 0xFFFFFFu);
-                for (uint32_t u = i; u < 4 && !t.rank; ++u) {
-                    t.dir[2 * b + 1] &= ~(0xFFu << (8 * u));
-                    t.dir[2 * b + 1] |= ((x >> (24 - t.db)) & 0xFFu) << (8 * u);
-                }
+        for (const Gram &x : grams) {
+            const uint32_t b = bucket(x.h), e = at[b]++;
+            const int len = len_of(rep[x.c]);
+            GramEntry &en = t.ent[e];
+            en.h = t.qw == 0 ? codes(P + first(rep[x.c]) + x.k, len - int(x.k)) : x.h;
+            en.idx = x.c;
+            en.k_len = x.k | uint32_t(len) << 8;
+            en.code = t.code[x.c];
+            const uint32_t i = e - (t.dir[2 * b] & 0xFFFFFFu);
+            for (uint32_t u = i; u < 4 && !t.rank; ++u) {
+                t.dir[2 * b + 1] &= ~(0xFFu << (8 * u));
+                t.dir[2 * b + 1] |= ((x.h >> (24 - t.db)) & 0xFFu) << (8 * u);
             }
+        }
         if (t.dense) {
             for (uint32_t c = 0; c < 4; ++c) {
                 uint32_t b = 0;

@@ -158,6 +158,7 @@ struct GramEntry {
 struct GramTables {
     bool ok = false;
     bool var = false;              // mixed lengths: no groups, code = pattern id
+    bool direct = false;           // the hash is the gram itself, shifted to the top: the filter is exact
     bool rank = false;             // buckets by rank in the filter
     int64_t d = 0;
     int32_t m_min = 0, m_max = 0;
