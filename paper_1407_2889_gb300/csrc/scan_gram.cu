@@ -875,19 +875,19 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
     a.n_occ = reinterpret_cast<long long *>(d_n_occ);
     // Tiles: long ones waste fewer lanes on a tile's last batch, short ones
     // spread a short text over the SMs. The workspace holds one count per
-    // kWarpTile bytes, so a tile is longer than that; a mixed-length slot has
-    // 12 bits for the start.
+    // kWarpTile bytes, so a tile is longer than that; the slots of a mixed set
+    // of 2^15 patterns or more have 12 bits for the start.
     int warps = dv.warps;
     const long long lanes = (long long)dp.sm_count * warps;
     int tile = min_tile(t.s);
     static_assert(min_tile(1) >= kWarpTile && min_tile(8) >= kWarpTile, "one count per kWarpTile bytes");
-    const int most = t.var ? tile : 2 * 4096;
+    const int most = t.var && t.d >= 32768 ? tile : 2 * 4096;
     while (2 * tile <= most && (n + 2 * tile - 1) / (2 * tile) >= lanes) tile *= 2;
     a.tile = tile;
     a.ntiles = (n + tile - 1) / tile;
     const int per_pos = t.var ? ws.per_pos : 1;
     const int se = gram_slot_bytes(t);
-    a.slot_kind = se == 8 ? 1 : t.var ? 2 : 0;
+    a.slot_kind = se == 8 ? 1 : t.var && t.d >= 32768 ? 2 : 0;
     a.slot_stride = (long long)tile * per_pos;
     a.slots = ws.slots;
     a.tile_ent = ws.tile_ent;
