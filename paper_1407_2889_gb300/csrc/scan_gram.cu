@@ -873,16 +873,28 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
     a.hist_smem = dv.hist_smem;
     a.counts = reinterpret_cast<long long *>(d_counts);
     a.n_occ = reinterpret_cast<long long *>(d_n_occ);
-    // Tiles: long ones waste fewer lanes on a tile's last batch, short ones
-    // spread a short text over the SMs. The workspace holds one count per
-    // kWarpTile bytes, so a tile is longer than that; the slots of a mixed set
-    // of 2^15 patterns or more have 12 bits for the start.
+    // Tiles: long ones waste fewer lanes on a tile's last batch (about as much as
+    // 500 more bytes), short ones spread a short text over the SMs, and their
+    // number has to fill whole rounds of all warps: 128 MiB in 8 KiB tiles took
+    // four rounds for 3.4 rounds' work (1,000 8-mers as PFAC: 84 us). The
+    // workspace holds one count per kWarpTile bytes, so a tile is longer than
+    // that; the slots of a mixed set of 2^15 patterns or more have 12 bits for
+    // the start, a dense slot 14.
     int warps = dv.warps;
     const long long lanes = (long long)dp.sm_count * warps;
-    int tile = min_tile(t.s);
+    const int step = t.dense ? 2 * kRow : rows_of(t.s) * kRow;
+    const int most = t.var && t.d >= 32768 ? 4096 : t.dense ? 8192 : 16384;
     static_assert(min_tile(1) >= kWarpTile && min_tile(8) >= kWarpTile, "one count per kWarpTile bytes");
-    const int most = t.var && t.d >= 32768 ? tile : 2 * 4096;
-    while (2 * tile <= most && (n + 2 * tile - 1) / (2 * tile) >= lanes) tile *= 2;
+    int tile = min_tile(t.s);
+    double best = 0.0;
+    for (int x = tile; x <= most; x += step) {
+        const long long tiles = (n + x - 1) / x, rounds = (tiles + lanes - 1) / lanes;
+        const double score = double(n) / (double(rounds) * double(lanes) * (x + 500));
+        if (score > best) {
+            best = score;
+            tile = x;
+        }
+    }
     a.tile = tile;
     a.ntiles = (n + tile - 1) / tile;
     const int per_pos = t.var ? ws.per_pos : 1;

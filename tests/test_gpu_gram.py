@@ -64,7 +64,7 @@ def test_every_gram_passes(m):
         s.close()
 
 
-@pytest.mark.parametrize("d,m", [(40000, 12), (70000, 24)])
+@pytest.mark.parametrize("d,m", [(40000, 12), (70000, 24), (20000, 40)])
 def test_wide_codes_and_device_counters(d, m):
     rng = np.random.default_rng(d)
     A = np.frombuffer(b"ACGT", np.uint8)
@@ -73,5 +73,15 @@ def test_wide_codes_and_device_counters(d, m):
     P[::3] = T[(np.arange(0, d, 3) * 4)[:, None] + np.arange(m)[None, :]]
     P[1] = P[0]
     s = pm.PatternSet.ac(P)
-    _check(s, T, oracle.dictionary(T, P, threads=THREADS))
+    want = oracle.dictionary(T, P, threads=THREADS)
+    _check(s, T, want)
+    # the batched form, whole and split, next to a small text
+    d_text = torch.from_numpy(T).cuda()
+    b = pm.Batch.exact([s, s], d_text, [0, 16], [T.size, 5000])
+    b.scan()
+    got = b.results()
+    small = oracle.dictionary(T[16:5016], P, threads=THREADS)
+    for g, w in zip(got, (want, small)):
+        assert np.array_equal(g[0], w[0]) and np.array_equal(g[1], w[1])
+    b.close()
     s.close()

@@ -81,6 +81,19 @@ def test_mixed_lengths(alphabet, lo, hi):
             pm.pm_set_free(h)
 
 
+def test_large_set():
+    rng = np.random.default_rng(3)
+    T = _text(rng, b"ACGT", 60013)
+    P = _rows(rng, T, b"ACGT", 17000, 32)
+    want = oracle.dictionary(T, P, threads=THREADS)
+    h = pm.pm_ac_compile(P, HOST)
+    try:
+        occ, cnt = pm.pm_selfcheck_gram_walk(h, T)
+        assert np.array_equal(occ, want[0]) and np.array_equal(cnt, want[1])
+    finally:
+        pm.pm_set_free(h)
+
+
 def test_text_edges():
     P = np.frombuffer(b"ACGTACGTACGTACGTACGTACGTACGTACGT", np.uint8).reshape(1, 32)
     h = pm.pm_ac_compile(P, HOST)
