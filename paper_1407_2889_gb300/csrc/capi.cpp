@@ -315,7 +315,7 @@ public:
         if (!plan_is_automatic(s)) return;
         const bool limited = s->algo == PM_ALGO_AC;
         auto work = [=]() { rc_ = build_gram(P, off, d, m, limited, s->gram); };
-        if (d >= 2000) {
+        if (d >= 256) {
             try {
                 thread_ = std::thread(work);
                 return;

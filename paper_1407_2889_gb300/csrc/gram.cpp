@@ -131,7 +131,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
                         G += double(with_len[L]) * std::pow(4.0, double(q - have));
                         hits += double(with_len[L]) / std::pow(double(std::max(letters, 2)), double(have));
                     }
-                if (G > (form == 0 ? 8.0e6 : 4.0e5)) continue;
+                if (G > (form == 0 ? 8.0e6 : 1.0e5)) continue;
                 const bool direct = packed && 2 * q <= 20 && (form > 0 || 2 * q <= 18);
                 const bool dense = form == 0 && direct && s == 1 && !var && q == hi && d < 32768;
                 int fb = direct ? 2 * q : 12;
@@ -198,6 +198,12 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
                 t.grp_off.push_back(t.grp_off.back() + mult[c]);
             }
             t.grp_ids.resize(t.grp_off.back());
+            // tiles add up their keys in 32 bits: at most 2^14 positions each
+            t.max_keys = *std::max_element(mult.begin(), mult.end());
+            if (t.max_keys >= 1u << 18) {
+                t = GramTables();
+                return PM_OK;
+            }
             for (int64_t r = 0; r < d; ++r) {
                 const uint32_t c = cls[size_t(r)];
                 if (mult[c] >= 2) t.grp_ids[fill[c]++] = uint32_t(r);

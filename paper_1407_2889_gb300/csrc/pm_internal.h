@@ -162,6 +162,7 @@ struct GramTables {
     bool rank = false;             // buckets by rank in the filter
     int64_t d = 0;
     int32_t m_min = 0, m_max = 0;
+    uint32_t max_keys = 1;         // largest group of equal patterns
     int32_t s = 0, q = 0, qw = 0;  // stride, gram length, words of a byte gram
     int32_t fb = 0, db = 0, pw = 0;
     uint32_t K[4] = {};

@@ -15,13 +15,15 @@
 // settles bytes outside the alphabet). The matches of a tile go to its slot
 // in text order, and the expand kernel of the other scans writes the keys.
 //
-// Bound: instruction issue (54-78 % of the issue slots; DRAM 20-40 % of its
-// peak). 256 MiB of EST-shaped text, list mode, this scan against the one
-// it replaces: 20,000 32-mers 0.10 ms (s = 16) against 1.64 (hybrid
-// transition table), 100,000 32-mers 0.20 against 2.46, 8,000 16-mers
-// compiled as Wu-Manber 0.13 (s = 4) against 2.10, 8,000 patterns of 8-16
-// characters 0.71 (s = 1) against 1.41; counts of 1,000 16-mers 0.075 (s =
-// 8) against 0.18.
+// Bound: instruction issue (62-76 % of the issue slots, 53 % of DRAM at stride 8
+// and 16, 10-38 % below; about 90 warp instructions per row at stride 16, 102 at
+// 8, 153 at 4). Filters of 192 KiB passed fewer grams and were slower (20,000
+// 32-mers 96 us against 75): candidates live on what L1 the filter leaves.
+// 256 MiB of EST-shaped text, list mode, this scan against the one it replaces:
+// 20,000 32-mers 73 us (s = 16) against 1.64 ms (hybrid transition table),
+// 100,000 32-mers 129 us against 2.46 ms, 8,000 16-mers compiled as Wu-Manber 98
+// us (s = 4) against 2.10 ms, 8,000 patterns of 8-16 characters 347 us (s = 1)
+// against 1.41 ms; counts of 1,000 16-mers 62 us (s = 8) against 183.
 #include <algorithm>
 #include <type_traits>
 
@@ -363,9 +365,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
 // word of the pair table, picked by the characters 2 .. m of an (m + 1)-gram,
 // holds for each pair of first characters whether the two m-grams in it are in
 // the set. 64 KB at m = 8; longer grams test the filter's bits. 1 GiB of
-// EST-shaped text, 8,000 8-mers (one position in nine matches), list mode: 1.13
+// EST-shaped text, 8,000 8-mers (one position in nine matches), list mode: 1.12
 // ms, with the transition table 1.38, with sampled grams 2.29; 128 MiB, 1,000
-// 8-mers (PFAC): 93 us, sampled 185. 256 MiB of the first: 73 % of the issue
+// 8-mers (PFAC): 80 us, sampled 185. 256 MiB of the first: 73 % of the issue
 // slots and 78 % of the shared-memory and L1 pipe in use.
 // ---------------------------------------------------------------------------
 struct DenseArgs {

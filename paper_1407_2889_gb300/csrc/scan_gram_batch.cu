@@ -335,6 +335,7 @@ long long smem_budget()
 bool gram_batch_layout(const GramTables &t, int &hist_off, int &tile)
 {
     if (!t.ok || t.var || t.qw != 0) return false;
+    if (t.max_keys > 4096u) return false;   // a round's keys are added up in 32 bits
     const long long room = smem_budget() - rr16((long long)kWarps * bwarp_bytes(t.s));
     const long long nc = (long long)t.code.size();
     const long long tab = (long long)t.filter.size() * 4 * (t.rank ? 2 : 1);

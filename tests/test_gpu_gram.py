@@ -85,3 +85,42 @@ def test_wide_codes_and_device_counters(d, m):
         assert np.array_equal(g[0], w[0]) and np.array_equal(g[1], w[1])
     b.close()
     s.close()
+
+
+@pytest.mark.parametrize("m", [8, 20])
+def test_captured_in_a_graph(m):
+    """A scan's dependent launches captured and replayed over changing texts."""
+    rng = np.random.default_rng(m)
+    A = np.frombuffer(b"ACGT", np.uint8)
+    P = A[rng.integers(0, 4, (200, m))]
+    n = 50000
+    s = pm.PatternSet.ac(P)
+    d_text = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    counts = torch.zeros(200, dtype=torch.int64, device="cuda")
+    occ = torch.zeros(n, dtype=torch.int64, device="cuda")
+    n_occ = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ws = torch.empty(s.workspace_bytes(n), dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+
+    def scan():
+        pm.pm_scan_device(s.h, d_text, n, 0, counts, occ, n, n_occ, ws, ws.numel(), torch.cuda.current_stream())
+
+    with torch.cuda.stream(side):
+        scan()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=side):
+        scan()
+    for k in range(3):
+        T = A[rng.integers(0, 4, n)]
+        T[k * 700:k * 700 + m] = P[k]
+        d_text.copy_(torch.from_numpy(T))
+        torch.cuda.synchronize()
+        g.replay()
+        torch.cuda.synchronize()
+        want = oracle.dictionary(T, P, threads=THREADS)
+        tot = int(n_occ.item())
+        assert tot == want[0].size
+        assert np.array_equal(occ[:tot].cpu().numpy().view(np.uint64), want[0])
+        assert np.array_equal(counts.cpu().numpy(), want[1])
+    s.close()

@@ -117,3 +117,19 @@ def test_pinned_plans_keep_the_automaton(pin):
         assert e.value.code == pm.PM_EINVAL
     finally:
         pm.pm_set_free(h)
+
+
+def test_huge_groups_keep_the_automaton():
+    """A tile's keys are added up in 32 bits: 2^18 equal patterns have no gram plan."""
+    P = np.tile(np.frombuffer(b"ACGTACGTAC", np.uint8), (1 << 18, 1))
+    for d, ok in ((1 << 18, False), ((1 << 18) - 1, True)):
+        h = pm.pm_wm_compile(P[:d], 2, HOST)
+        try:
+            if ok:
+                occ, _ = pm.pm_selfcheck_gram_walk(h, np.frombuffer(b"TACGTACGTACC", np.uint8))
+                assert occ.size == d
+            else:
+                with pytest.raises(pm.PmError):
+                    pm.pm_selfcheck_gram_walk(h, np.frombuffer(b"TACGTACGTACC", np.uint8))
+        finally:
+            pm.pm_set_free(h)
