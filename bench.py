@@ -37,11 +37,13 @@ METRIC = "text GB/s scanned on 1 GB300 (AC & WM), batched vs plain; % of HBM roo
 KERNEL_SOURCES = ["paper_1407_2889_gb300/csrc/scan_ac.cu", "paper_1407_2889_gb300/csrc/scan_ac_wide.cu",
                   "paper_1407_2889_gb300/csrc/ac_scan_kernel.cuh", "paper_1407_2889_gb300/csrc/ac_device.cuh",
                   "paper_1407_2889_gb300/csrc/scan_common.cuh"]
+GRAM_SOURCES = ["paper_1407_2889_gb300/csrc/scan_gram.cu", "paper_1407_2889_gb300/csrc/gram_device.cuh",
+                "paper_1407_2889_gb300/csrc/scan_common.cuh"]
 
 
-def kernel_hash() -> str:
+def kernel_hash(sources=KERNEL_SOURCES) -> str:
     h = hashlib.sha256()
-    for p in KERNEL_SOURCES:
+    for p in sources:
         with open(os.path.join(ROOT, p), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -67,6 +69,12 @@ def plan_key(plan) -> dict:
     return key
 
 
+def takes_gram_scan(plan) -> bool:
+    """Whether a set of the bench's kind (ACGT) with this launch plan takes the
+    gram scan: the automatic plan does, a pinned one walks its automaton."""
+    return plan_key(plan) == plan_key(None)
+
+
 def recorded_traffic(kernel_name: str, workload: str, plan=None):
     """DRAM bytes per launch from a committed ncu summary, if it was taken on
     the current kernel source, the same workload and the same launch plan
@@ -78,7 +86,8 @@ def recorded_traffic(kernel_name: str, workload: str, plan=None):
     with open(p) as f:
         rec = json.load(f)
     e = rec.get(kernel_name)
-    if not e or e.get("kernel_hash") != kernel_hash() or e.get("workload") != workload:
+    sources = GRAM_SOURCES if kernel_name.startswith("gram") else KERNEL_SOURCES
+    if not e or e.get("kernel_hash") != kernel_hash(sources) or e.get("workload") != workload:
         return None
     plans = [e.get("plan")] + list(e.get("same_plans", []))
     if not any(plan_key(q) == plan_key(plan) for q in plans):
@@ -371,12 +380,15 @@ def main():
     avg_launch_s = statistics.mean(per_launch) / 1e3
     alg_bytes = n + 8 * d + (8 * n_occ if args.mode == "list" else 0)
     achieved = alg_bytes / avg_launch_s / 1e9
+    gram = takes_gram_scan(pinned_plan or tuned)
+    kernel = "gram_dense_kernel" if gram else f"{args.algo}_scan_kernel"
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_kind": peak_kind,
-                "traffic": recorded_traffic(f"{args.algo}_scan_kernel", f"est1gib_d{d}_m{args.m}_{args.mode}_n{n}",
+                "traffic": recorded_traffic(kernel, f"est1gib_d{d}_m{args.m}_{args.mode}_n{n}",
                                             pinned_plan or tuned),
                 "algorithmic_bytes_per_launch": alg_bytes,
-                "kernel": (f"{args.algo}_scan_kernel" + (" + expand_kernel (list mode)" if args.mode == "list" else ""))}
+                "kernel": kernel + ((" + dense_expand_kernel" if gram else " + expand_kernel") + " (list mode)"
+                                    if args.mode == "list" else "")}
 
     # end to end through the public API: pinned host text in, pinned host
     # counts and occurrence list out (pm_scan_to_host), copies inside the timing
@@ -430,7 +442,7 @@ def main():
                        "plan": tuned or "planner default"},
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
             # scan + expand kernels per list-mode step (the workspace zeroing is a memset call)
-            "gpu_launches": args.steps * (2 if args.mode == "list" else 1), "clocks": clk, "extras": extras,
+            "gpu_launches": args.steps * ((2 if args.mode == "list" else 1) + (1 if gram else 0)), "clocks": clk, "extras": extras,
         }
         print(json.dumps(line), flush=True)
     if dist:
@@ -471,6 +483,7 @@ def secondary(args, s, P, T, d_text, stream, launch, occ, counts, nocc, ws, pm, 
                 q.tune(d_text, reps=2)
             cnt_q = torch.zeros(dd, dtype=torch.int64, device="cuda")
             ws = torch.zeros(q.workspace_bytes(n), dtype=torch.uint8, device="cuda")
+            torch.cuda.synchronize()  # the fills run on another stream
 
             def timed(flags, buf, cap, reps=3):
                 ev0 = torch.cuda.Event(enable_timing=True)

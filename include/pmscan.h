@@ -105,6 +105,15 @@ typedef struct pm_params {
                                  PM_ETOOBIG otherwise); pm_tune tries both */
 } pm_params;
 
+/*
+ * A set whose plan is left automatic (placement, smem_table_bytes,
+ * warps_per_cta, ctas_per_sm, counters and ids_place 0, stride 0 or 1; for
+ * Wu-Manber sets warps_per_cta and ctas_per_sm 0) also gets sampled-gram
+ * tables where they are planned to be faster, and its scans take them
+ * instead of the automaton or the SHIFT tables: every pattern is entered
+ * under its first s grams, and the grams at multiples of s are looked up in
+ * the text. Results are the same. A pinned plan keeps the method's own scan.
+ */
 typedef struct pm_set pm_set; /* compiled pattern set; owns its device tables */
 
 typedef struct pm_set_info {
@@ -216,7 +225,8 @@ int pm_set_get_info(const pm_set *s, pm_set_info *info);
  * set's own pm_params (placement, warps, counters, ids) apply as at compile
  * time. No device is touched, so this works for host-only sets
  * (pm_params.host_only) and without a GPU: for inspecting what the planner
- * does and testing it. A set compiled for a device runs the plan of that
+ * does and testing it. It is the plan of the transition-table walk, also for
+ * a set whose scans take its gram tables. A set compiled for a device runs the plan of that
  * device's shape (until pm_tune replaces it). PM_EINVAL for other
  * algorithms or non-positive sizes; PM_ETOOBIG when nothing fits.
  */
@@ -293,9 +303,9 @@ int pm_scan_device(const pm_set *s, const uint8_t *d_text, int64_t n, uint32_t f
  * allocated: no cudaMalloc, cudaFree or allocating library call.
  *   - Only plain Aho-Corasick sets (PM_EINVAL for PFAC, mixed-length and
  *     Wu-Manber sets).
- *   - Always the one-character walk, even for a set whose tuned plan takes
- *     two characters per lookup (pm_params.stride = 2): the results are the
- *     same, only the launch plan differs.
+ *   - Never two characters per lookup, even for a set whose plan takes them
+ *     (pm_params.stride = 2): the gram scan where the set has it, else the
+ *     one-character walk. The results are the same.
  *   - PM_ETOOBIG when the scan would need more scratch than the array holds
  *     (large texts in list mode, or very large pattern sets); nothing runs.
  *   - Each call looks up the array's device address on the current device
@@ -325,14 +335,15 @@ int pm_noalloc_scan_status(void *stream);
  * warps per CTA (auto, 16, 12, 8), per-terminal counters (32-bit or 16-bit
  * in shared memory, or device memory) and the terminal-id structure (shared
  * or device memory, or late: codes and counts taken by the expand kernel in
- * list mode), plus the two-character scan (stride 2) when the set
+ * list mode), plus the gram scan where the set has it (the automatic
+ * parameters then) and the two-character scan (stride 2) when the set
  * qualifies, and keeps the fastest for the set: later scans use it. In list
  * mode, late plans that differ only in their counters count as one, and the
  * one kept has the counters that fit best for counts-only scans.
  * Results never depend on the plan. Allocates its own scratch, synchronises
  * `stream`. *best_out / *best_ms (may be NULL) receive the chosen pm_params
- * and its time per scan. Wu-Manber sets tune warps per CTA only (auto, 24,
- * 20, 16, 12, 8; more than 16 for exact-code tables of ACGT sets).
+ * and its time per scan. Wu-Manber sets tune the gram scan and warps per CTA
+ * (auto, 24, 20, 16, 12, 8; more than 16 for exact-code tables of ACGT sets).
  * PM_EINVAL for PFAC and mixed-length sets and for host-only sets.
  */
 int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t reps,
