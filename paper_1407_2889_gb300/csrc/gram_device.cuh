@@ -139,9 +139,17 @@ __device__ __forceinline__ void verify_batch(const GramTile &g, uint32_t e0, uin
 {
     const int lane = threadIdx.x & 31;
     uint32_t nm = 0, first = 0;
-    for (uint32_t k = 0; k < cnt; ++k) {
-        if (!same_code<RAW>(__ldg(g.ent + e0 + k), win)) continue;
-        if (nm++ == 0) first = e0 + k;
+    if (__any_sync(kFull, cnt > 8u)) {
+        // a long list (a run of one letter in many patterns): straight to the
+        // pairs, all lanes on it. With one lane on it, 64 MiB of text with 2 %
+        // of runs of A against 8,000 32-mers took 3.0 ms.
+        nm = cnt;
+        first = e0;
+    } else {
+        for (uint32_t k = 0; k < cnt; ++k) {
+            if (!same_code<RAW>(__ldg(g.ent + e0 + k), win)) continue;
+            if (nm++ == 0) first = e0 + k;
+        }
     }
     if (!__any_sync(kFull, nm != 0u)) return;
     auto one = [&](bool in, uint32_t e, uint32_t w, int p) {

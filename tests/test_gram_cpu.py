@@ -133,3 +133,25 @@ def test_huge_groups_keep_the_automaton():
                     pm.pm_selfcheck_gram_walk(h, np.frombuffer(b"TACGTACGTACC", np.uint8))
         finally:
             pm.pm_set_free(h)
+
+
+def test_repetitive_sets_keep_the_automaton():
+    """A gram with more than 256 entries: an Aho-Corasick set keeps its table."""
+    rng = np.random.default_rng(8)
+    P = np.frombuffer(b"ACGT", np.uint8)[rng.integers(0, 4, (400, 32))]
+    P[:, :24] = ord("A")
+    T = np.full(3000, ord("A"), np.uint8)
+    T[1000:1032] = P[7]
+    want = oracle.dictionary(T, P, threads=1)
+    h = pm.pm_ac_compile(P, HOST)
+    try:
+        with pytest.raises(pm.PmError):
+            pm.pm_selfcheck_gram_walk(h, T)
+        assert np.array_equal(pm.pm_selfcheck_host_walk(h, T)[0], want[0])
+    finally:
+        pm.pm_set_free(h)
+    h = pm.pm_wm_compile(P, 2, HOST)
+    try:
+        assert np.array_equal(pm.pm_selfcheck_gram_walk(h, T)[0], want[0])
+    finally:
+        pm.pm_set_free(h)
