@@ -391,7 +391,8 @@ int pm_scan_batch(const pm_set *const *sets, const uint8_t *const *texts,
  * Counts of instance j land at counts[c_j .. c_j + d_j) with c_j the sum of
  * the d of the instances before j; pm_batch_counts_total gives the sum. The
  * sets must outlive the batch. The batch owns a small device array of
- * descriptors until pm_batch_free.
+ * descriptors until pm_batch_free. Whether an instance takes its set's gram
+ * tables is settled here: a later pm_tune of the set does not change it.
  */
 typedef struct pm_batch pm_batch;
 int pm_batch_prepare(const pm_set *const *sets, int32_t k, const int64_t *text_off,

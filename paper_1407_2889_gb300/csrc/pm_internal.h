@@ -521,16 +521,23 @@ struct BatchShape {                // launch shape and shared-memory split
     int policy = 0;
     int region_bytes = 0;          // per-CTA table / ids / counters region
     long long smem_bytes = 0;
+    long long gram_smem = 0;       // per-CTA shared memory of the gram kernel
     int sm_count = 0;
 };
 
+// gram: the instance is a gram item where its tables fit. Taken from the set
+// once (batch_takes_grams), when the instance is set up: pm_tune may take the
+// set off the gram scan or back to it, and every later layout of the instance
+// has to need the words its workspace was sized for.
 struct BatchInst {
     const pm_set *set;
     int64_t text_off, text_len, count_off, occ_off, occ_cap, out_slot;
+    bool gram;
 };
 
 int batch_shape(int warps, BatchShape &out);
 bool batch_supports(const pm_set *s);   // AC, ACGT-like alphabet, m <= 65, device tables
+bool batch_takes_grams(const pm_set *s);  // do the set's scans take its gram tables now?
 // Descriptors of k instances in the order given, one per instance (out may
 // be NULL); returns the number of global counter words the workspace needs.
 int64_t batch_fill(const BatchInst *inst, int k, const BatchShape &sh, BatchDesc *out);

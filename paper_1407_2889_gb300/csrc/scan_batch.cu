@@ -401,12 +401,13 @@ struct InstLayout {
 // otherwise counters and ids stay in shared memory only while each takes at
 // most a quarter of the region, and the table gets the rest (its
 // breadth-first prefix: the rows a walk visits most).
-static InstLayout layout_of(const pm_set *s, int region, int policy)
+static InstLayout layout_of(const BatchInst &I, const BatchShape &sh)
 {
-    const AcTables &t = s->ac;
-    if (s->dac.dg) {  // sets that take the gram scan take it here too, where their tables fit
+    const AcTables &t = I.set->ac;
+    const int region = sh.region_bytes, policy = sh.policy;
+    if (I.gram) {  // sets that take the gram scan take it here too, where their tables fit
         InstLayout G;
-        G.gram = gram_batch_layout(s->gram, G.hist_off, G.tile);
+        G.gram = gram_batch_layout(I.set->gram, sh.gram_smem, G.hist_off, G.tile);
         if (G.gram) return G;
     }
     const int eb = t.entry_bytes;
@@ -446,6 +447,7 @@ int batch_shape(int warps, BatchShape &out)
     if (room < 4096) room = 4096;
     out.region_bytes = int(room & ~15LL);
     out.smem_bytes = (long long)out.region_bytes + (long long)warps * batch_warp_bytes();
+    out.gram_smem = gram_batch_smem(dp);
     out.sm_count = dp.sm_count;
     return PM_OK;
 }
@@ -454,6 +456,8 @@ bool batch_supports(const pm_set *s)
 {
     return s && !s->host_only && s->algo == PM_ALGO_AC && s->ac.dna && s->ac.m <= kBatchMaxM;
 }
+
+bool batch_takes_grams(const pm_set *s) { return s->dac.dg != nullptr; }
 
 // The descriptor of one instance (or of its part p of P, tiles [t_lo, t_hi)).
 static void fill_desc(const BatchInst &I, const InstLayout &L, long long coff, BatchDesc &D)
@@ -503,7 +507,7 @@ int64_t batch_fill(const BatchInst *inst, int k, const BatchShape &sh, BatchDesc
     for (int q = 0; q < k; ++q) {
         const BatchInst &I = inst[q];
         const AcTables &t = I.set->ac;
-        const InstLayout L = layout_of(I.set, sh.region_bytes, sh.policy);
+        const InstLayout L = layout_of(I, sh);
         const int64_t nt = int64_t(t.canon.size());
         const int64_t coff = ccount;
         if (L.hist_off < 0) ccount += nt;
@@ -530,7 +534,7 @@ int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool lis
     double total[2] = {0.0, 0.0};   // the two kernels run one after the other
     for (int q = 0; q < k; ++q) {
         const AcTables &t = inst[q].set->ac;
-        const InstLayout L = layout_of(inst[q].set, sh.region_bytes, sh.policy);
+        const InstLayout L = layout_of(inst[q], sh);
         lay[size_t(q)] = L;
         // a table read partly through L2 costs several times more per byte;
         // every instance also pays for loading its tables. Gram items by their
@@ -604,7 +608,7 @@ int64_t batch_items(const BatchInst *inst, int k, const BatchShape &sh, bool lis
 int64_t batch_words_bound(const BatchInst &I, const BatchShape &sh, bool list)
 {
     const AcTables &t = I.set->ac;
-    const InstLayout L = layout_of(I.set, sh.region_bytes, sh.policy);
+    const InstLayout L = layout_of(I, sh);
     const long long ntiles = (I.text_len + kWarpTile - 1) / kWarpTile;
     const long long parts = std::max(1LL, max_parts(L, ntiles, std::max(sh.warps, 1)));
     int64_t w = (L.hist_off < 0 || parts > 1) ? int64_t(t.canon.size()) : 0;
@@ -792,7 +796,8 @@ int pm_batch_prepare(const pm_set *const *sets, int32_t k, const int64_t *text_o
         b->inst.resize(size_t(k));
         for (int32_t j = 0; j < k; ++j)
             b->inst[size_t(j)] = BatchInst{sets[j], text_off[j], text_len[j], b->count_off[size_t(j)],
-                                           occ_off[j], occ_off[j + 1] - occ_off[j], j};
+                                           occ_off[j], occ_off[j + 1] - occ_off[j], j,
+                                           batch_takes_grams(sets[j])};
         // the workspace must hold the counters and part words of every
         // warp count the tuner may pick
         int rc = PM_OK;

@@ -326,17 +326,21 @@ __global__ void __launch_bounds__(kWarps * 32, 1) gram_batch_kernel(const BatchA
 long long smem_budget()
 {
     DeviceProps dp;
-    if (device_props(dp)) return 0;
-    return ((long long)dp.smem_optin - 2048) & ~15LL;   // static shared memory and slack
+    return device_props(dp) ? 0 : gram_batch_smem(dp);
 }
 
 }  // namespace
 
-bool gram_batch_layout(const GramTables &t, int &hist_off, int &tile)
+long long gram_batch_smem(const DeviceProps &dp)
+{
+    return ((long long)dp.smem_optin - 2048) & ~15LL;   // static shared memory and slack
+}
+
+bool gram_batch_layout(const GramTables &t, long long smem, int &hist_off, int &tile)
 {
     if (!t.ok || t.var || t.qw != 0) return false;
     if (t.max_keys > 4096u) return false;   // a round's keys are added up in 32 bits
-    const long long room = smem_budget() - rr16((long long)kWarps * bwarp_bytes(t.s));
+    const long long room = smem - rr16((long long)kWarps * bwarp_bytes(t.s));
     const long long nc = (long long)t.code.size();
     const long long tab = (long long)t.filter.size() * 4 * (t.rank ? 2 : 1);
     if (tab > room || t.filter.size() % 4 != 0) return false;

@@ -6,10 +6,11 @@
 
 namespace pm {
 
-// Do the set's gram tables fit the batched kernel? hist_off: byte offset of its
+long long gram_batch_smem(const DeviceProps &dp);  // per-CTA shared memory of the kernel
+// Do the set's gram tables fit it? hist_off: byte offset of its
 // counters behind the filter, -1 when they stay in device memory; tile: text
 // bytes a warp takes at a time.
-bool gram_batch_layout(const GramTables &t, int &hist_off, int &tile);
+bool gram_batch_layout(const GramTables &t, long long smem, int &hist_off, int &tile);
 void gram_batch_fill(const GramTables &t, const DevGram &dv, int tile, BatchDesc &D);
 // the tile length of an item whose range is set, at most `most`; also decides
 // whether the item's filter is probed in device memory

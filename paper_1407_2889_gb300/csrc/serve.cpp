@@ -192,6 +192,7 @@ struct Req {
     int64_t occ_blk = -1, occ_bytes = 0, occ_cap = 0;
     int64_t ws_bytes = 0;              // workspace of a whole-GPU scan (the slot's)
     bool plain = false;
+    bool gram = false;                 // see BatchInst
     void *occ_ext = nullptr;           // re-run buffer outside the arena
     int64_t n_occ = 0;
     int status = PM_OK;
@@ -278,7 +279,7 @@ bool admit(pm_server *s, Req &r)
     r.occ_cap = est_cap(s, r);
     r.occ_bytes = r.list ? std::max<int64_t>(r.occ_cap, 1) * 8 : 0;
     {
-        const BatchInst I{r.set, 0, r.n, 0, 0, r.list ? r.occ_cap : 0, 0};
+        const BatchInst I{r.set, 0, r.n, 0, 0, r.list ? r.occ_cap : 0, 0, r.gram};
         r.plain = batch_words_bound(I, s->shape, r.list) > s->p.counter_words;
     }
     r.ws_bytes = r.plain ? pm_scan_workspace_bytes(r.set, r.n, r.list ? 0u : PM_COUNTS_ONLY) : 0;
@@ -321,7 +322,7 @@ void *release(pm_server *s, Req &r)
 // scan with its own workspace).
 int64_t counter_words(pm_server *s, const Req &r)
 {
-    const BatchInst I{r.set, 0, r.n, 0, 0, r.list ? est_cap(s, r) : 0, 0};
+    const BatchInst I{r.set, 0, r.n, 0, 0, r.list ? est_cap(s, r) : 0, 0, r.gram};
     const int64_t w = batch_words_bound(I, s->shape, r.list);
     return w > s->p.counter_words ? 0 : w;
 }
@@ -366,7 +367,8 @@ int launch_slot(pm_server *s, Slot &sl)
         const Req &r = *sl.reqs[size_t(j)];
         if (r.plain) continue;
         const int64_t occ_off = r.list ? r.occ_blk / 8 : 0;
-        inst.push_back(BatchInst{r.set, r.text_blk, r.n, r.cnt_blk / 8, occ_off, r.list ? r.occ_cap : 0, j});
+        inst.push_back(
+            BatchInst{r.set, r.text_blk, r.n, r.cnt_blk / 8, occ_off, r.list ? r.occ_cap : 0, j, r.gram});
     }
     // queue items: costliest first, large requests split across CTAs
     std::vector<BatchDesc> items;
@@ -548,7 +550,7 @@ int rerun_one(pm_server *s, Slot &sl, Req &r, uint64_t *occ)
         if (rc == PM_OK) rc = launch_plain(s, r, occ, r.occ_cap, sl.d_nocc, sl.d_pws, sl.st);
     } else {
         // split across CTAs when the parts' words fit the slot's workspace
-        BatchInst I{r.set, r.text_blk, r.n, r.cnt_blk / 8, 0, r.occ_cap, 0};
+        BatchInst I{r.set, r.text_blk, r.n, r.cnt_blk / 8, 0, r.occ_cap, 0, r.gram};
         std::vector<BatchDesc> items;
         int64_t spill = 0;
         int64_t words = batch_items(&I, 1, s->shape, true, items, &spill);
@@ -814,6 +816,7 @@ int pm_server_submit(pm_server *s, const pm_set *set, const uint8_t *T, int64_t 
     r->T = T;
     r->n = n;
     r->list = !(flags & PM_COUNTS_ONLY);
+    r->gram = batch_takes_grams(set);
     int64_t need = round_up(std::max<int64_t>(n, 1), kAlign) + round_up(set->ac.d * 8, kAlign) +
                    (r->list ? round_up((est_cap(s, *r) + 1) * 8, kAlign) : 0);
     if (need > s->arena.capacity() || counter_words(s, *r) > s->p.counter_words) {
