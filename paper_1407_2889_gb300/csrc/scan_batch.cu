@@ -698,7 +698,7 @@ struct pm_batch {
     int64_t desc_cap = 0;             // descriptors the device array holds
     pm::BatchDesc *d_desc = nullptr;
     int64_t ccount_total = 0;
-    int64_t ws_bytes = 0;             // enough for every candidate shape
+    int64_t ws_bytes = 0;             // enough for every candidate shape, and for the current one
     int64_t d_total = 0;
     pm::BatchShape shape;
     uint32_t flags = 0;
@@ -708,14 +708,18 @@ struct pm_batch {
 namespace pm {
 
 // Lay the batch out for `warps` warps per CTA and upload the descriptors
-// (into the existing device array once there is one).
+// (into the existing device array once there is one). A layout outside the
+// candidates (fewer than 8 warps) that needs a larger workspace raises
+// ws_bytes, so that scans refuse a smaller one.
 static int apply_plan(pm_batch *b, int warps, int policy)
 {
     int rc = batch_shape(warps, b->shape);
     if (rc) return rc;
     b->shape.policy = policy;
     std::vector<BatchDesc> h;
-    b->ccount_total = batch_items(b->inst.data(), b->k, b->shape, !(b->flags & PM_COUNTS_ONLY), h, nullptr);
+    int64_t spill = 0;
+    b->ccount_total = batch_items(b->inst.data(), b->k, b->shape, !(b->flags & PM_COUNTS_ONLY), h, &spill);
+    b->ws_bytes = std::max<int64_t>(b->ws_bytes, batch_ws_bytes(b->ccount_total) + 8 * spill);
     b->n_items = int32_t(h.size());
     b->n_gram = batch_gram_items(h);
     if (h.empty()) return PM_OK;
@@ -888,6 +892,7 @@ int pm_batch_tune(pm_batch *b, const uint8_t *d_text, int64_t *d_counts, uint64_
     for (int w : kBatchWarpChoices)
     for (int policy : {0, 1}) {
         rc = apply_plan(b, w, policy);
+        if (!rc && workspace_bytes < b->ws_bytes) rc = PM_EINVAL;
         if (!rc) rc = batch_prepare_launch(b->shape);
         if (!rc) rc = batch_enqueue(b, o, st);  // warm-up
         if (!rc) {

@@ -699,8 +699,16 @@ class Batch:
     def tune(self, reps: int = 3, stream=None) -> float:
         return pm_batch_tune(self.b, *self._bufs(), reps=reps, stream=stream)
 
+    def _fit_ws(self) -> None:
+        """A plan outside the tuner's candidates may need a larger workspace."""
+        need = pm_batch_workspace_bytes(self.b)
+        if need > self.ws_bytes:
+            self.ws = self.ws.new_empty(need)
+            self.ws_bytes = need
+
     def set_warps(self, warps: int) -> None:
         pm_batch_set_warps(self.b, warps)
+        self._fit_ws()
 
     @property
     def warps(self) -> int:
@@ -708,6 +716,7 @@ class Batch:
 
     def set_placement(self, placement: int) -> None:
         pm_batch_set_placement(self.b, placement)
+        self._fit_ws()
 
     @property
     def placement(self) -> int:
