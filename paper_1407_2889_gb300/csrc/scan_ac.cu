@@ -137,8 +137,7 @@ struct ExpandLateArgs {
 
 template <typename SE, int kOffShift, uint32_t kGrp, int CM, bool GS, bool ANY>
 __global__ void __launch_bounds__(kExpandThreads)
-expand_kernel(const SE *__restrict__ slots, const uint32_t *__restrict__ tile_ent,
-              const uint32_t *__restrict__ tile_out, const unsigned long long *__restrict__ seg_sum,
+expand_kernel(const SE *slots, const uint32_t *tile_ent, const uint32_t *tile_out, const unsigned long long *seg_sum,
               long long nseg, long long seg_tiles, long long nsub,
               const uint32_t *__restrict__ grp_off, const uint32_t *__restrict__ grp_ids,
               unsigned long long *__restrict__ occ, long long occ_cap, long long *n_occ,

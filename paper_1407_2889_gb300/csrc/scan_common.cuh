@@ -196,7 +196,10 @@ segment_offsets(const uint32_t *tile_ent, const uint32_t *tile_out, const unsign
 // that does not need the one before (table loads): launched as programmatic
 // dependents they do that work while the other still runs. Every such kernel
 // calls grid_wait() before it reads or writes what earlier kernels touch, and
-// the kernels before it let it start early with grid_trigger().
+// the kernels before it let it start early with grid_trigger(). What an earlier
+// kernel of the chain writes is written during this kernel's lifetime, so it is
+// read with ordinary loads: its pointers are not const __restrict__ and not
+// read by __ldg, which may use the non-coherent path.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -626,12 +626,11 @@ constexpr int kDenseExpandThreads = 512;
 
 template <bool SM>
 __global__ void __launch_bounds__(kDenseExpandThreads)
-dense_expand_kernel(const uint32_t *__restrict__ slots, const uint32_t *__restrict__ tile_ent,
-                    const uint32_t *__restrict__ tile_out, const unsigned long long *__restrict__ seg_sum,
-                    long long seg_tiles, long long ntiles, uint32_t tile, const uint16_t *__restrict__ id_off,
-                    const uint16_t *__restrict__ ids, int nc, int d, unsigned long long *__restrict__ occ,
-                    long long occ_cap, long long *n_occ, const unsigned long long *occ_base,
-                    unsigned long long pos_base)
+dense_expand_kernel(const uint32_t *slots, const uint32_t *tile_ent, const uint32_t *tile_out,
+                    const unsigned long long *seg_sum, long long seg_tiles, long long ntiles, uint32_t tile,
+                    const uint16_t *__restrict__ id_off, const uint16_t *__restrict__ ids, int nc, int d,
+                    unsigned long long *__restrict__ occ, long long occ_cap, long long *n_occ,
+                    const unsigned long long *occ_base, unsigned long long pos_base)
 {
     constexpr int T = kDenseExpandThreads, NW = T / 32, R = 8;
     extern __shared__ __align__(16) unsigned char esm[];
