@@ -69,10 +69,11 @@ def plan_key(plan) -> dict:
     return key
 
 
-def takes_gram_scan(plan) -> bool:
-    """Whether a set of the bench's kind (ACGT) with this launch plan takes the
-    gram scan: the automatic plan does, a pinned one walks its automaton."""
-    return plan_key(plan) == plan_key(None)
+def scan_kernels(pm, s, algo):
+    """Names of the scan and expand kernels that the set's scans take."""
+    return {pm.PM_SCAN_METHOD: (f"{algo}_scan_kernel", "expand_kernel"),
+            pm.PM_SCAN_GRAMS: ("gram_scan_kernel", "expand_kernel"),
+            pm.PM_SCAN_DENSE: ("gram_dense_kernel", "dense_expand_kernel")}[s.scan_kind()]
 
 
 def recorded_traffic(kernel_name: str, workload: str, plan=None):
@@ -380,15 +381,14 @@ def main():
     avg_launch_s = statistics.mean(per_launch) / 1e3
     alg_bytes = n + 8 * d + (8 * n_occ if args.mode == "list" else 0)
     achieved = alg_bytes / avg_launch_s / 1e9
-    gram = takes_gram_scan(pinned_plan or tuned)
-    kernel = "gram_dense_kernel" if gram else f"{args.algo}_scan_kernel"
+    gram = s.scan_kind() != pm.PM_SCAN_METHOD
+    kernel, expand = scan_kernels(pm, s, args.algo)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_kind": peak_kind,
                 "traffic": recorded_traffic(kernel, f"est1gib_d{d}_m{args.m}_{args.mode}_n{n}",
                                             pinned_plan or tuned),
                 "algorithmic_bytes_per_launch": alg_bytes,
-                "kernel": kernel + ((" + dense_expand_kernel" if gram else " + expand_kernel") + " (list mode)"
-                                    if args.mode == "list" else "")}
+                "kernel": kernel + (f" + {expand} (list mode)" if args.mode == "list" else "")}
 
     # end to end through the public API: pinned host text in, pinned host
     # counts and occurrence list out (pm_scan_to_host), copies inside the timing
@@ -441,8 +441,9 @@ def main():
                                                       "B", "Bp", "dna_mode") if info.get(k)},
                        "plan": tuned or "planner default"},
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
-            # scan + expand kernels per list-mode step (the workspace zeroing is a memset call)
-            "gpu_launches": args.steps * ((2 if args.mode == "list" else 1) + (1 if gram else 0)), "clocks": clk, "extras": extras,
+            # scan + expand kernels per list-mode step; a gram scan also zeroes by a kernel, the others by memsets
+            "gpu_launches": args.steps * ((2 if args.mode == "list" else 1) + (1 if gram else 0)), "clocks": clk,
+            "extras": extras,
         }
         print(json.dumps(line), flush=True)
     if dist:
@@ -811,12 +812,16 @@ def batched_comparison(args, T, d_text, pm, torch, synth):
         "plain_steady_sample": f"{len(sample)} sets (every {max(1, k // 64)}th instance), each over the first "
                                f"{span >> 20} MiB of the text, list mode, weighted by instance length",
         "tuned_warps": warps, "tune_best_ms": tuned_ms, "compile_s": t_compile,
-        "plan": {"warps_per_cta": warps, "chunk_bytes_per_lane": 80, "placement_policy": placement,
+        "plan": {"gram_sets": sum(s.scan_kind() != pm.PM_SCAN_METHOD for s in sets),
+                 "gram_items": "sets that take the gram scan run in its batch kernel at 24 warps per CTA where their "
+                               "tables fit; the tuned warps and placement apply to the other instances only",
+                 "warps_per_cta": warps, "chunk_bytes_per_lane": 80, "placement_policy": placement,
                  "placement": "per instance: whole table in the CTA's shared memory when it fits, else its "
                               "breadth-first prefix, with ids and counters in shared memory while each takes "
                               "at most a quarter of the region (policy 0) or in device memory (policy 1); "
                               "the tuner picks warps x policy",
-                 "split": "instances above a quarter of a CTA's share split into parts of whole warp tiles"},
+                 "split": "instances above a quarter of a CTA's share (gram items: an eighth) split into parts of "
+                          "whole warp tiles"},
         "workload": "k slices of the EST-shaped text, lengths log-uniform 1 KiB-4 MiB (seed 4000+j), "
                     "own set per instance: d log-uniform 10-10^4, m uniform 8-64, list mode",
     }

@@ -217,6 +217,13 @@ int pm_wmv_compile(const uint8_t *P, const int64_t *offsets, int64_t d, int32_t 
 
 void pm_set_free(pm_set *s);
 int pm_set_get_info(const pm_set *s, pm_set_info *info);
+/* Which scan the set's pm_scan, pm_scan_to_host and pm_scan_device take, until
+ * pm_tune changes it: PM_SCAN_METHOD the method's own (automaton, SHIFT
+ * tables), PM_SCAN_GRAMS sampled grams, PM_SCAN_DENSE grams at every position
+ * (see pm_set above). For a host-only set, the one its tables are planned for.
+ * -1 for NULL. */
+enum { PM_SCAN_METHOD = 0, PM_SCAN_GRAMS = 1, PM_SCAN_DENSE = 2 };
+int32_t pm_set_scan_kind(const pm_set *s);
 
 /*
  * The launch plan the planner picks for an Aho-Corasick or PFAC set on a
@@ -434,7 +441,11 @@ int pm_batch_scan_device(const pm_batch *b, const uint8_t *d_text, int64_t *d_co
 int pm_batch_tune(pm_batch *b, const uint8_t *d_text, int64_t *d_counts, uint64_t *d_occ,
                   int64_t *d_n_occ, void *d_workspace, int64_t workspace_bytes, int32_t reps,
                   void *stream, float *best_ms);
-int pm_batch_set_warps(pm_batch *b, int32_t warps);  /* 1..16; drops a captured graph */
+/* 1..16; drops a captured graph. Warps and placement are those of the
+ * transition-table kernel: instances that take their set's gram tables run in
+ * a kernel of their own with 24 warps per CTA, so for a batch of only such
+ * instances every plan is the same one (and pm_batch_tune times it six times). */
+int pm_batch_set_warps(pm_batch *b, int32_t warps);
 /* Table placement of instances whose tables do not all fit the CTA's shared
  * memory: 0 (default) keeps their terminal ids and counters there while each
  * takes at most a quarter of the region and gives the table's breadth-first

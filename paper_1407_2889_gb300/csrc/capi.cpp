@@ -985,6 +985,17 @@ int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t
     return PM_OK;
 }
 
+int32_t pm_set_scan_kind(const pm_set *s)
+{
+    if (!s) return -1;
+    const DevGram *dg = s->algo == PM_ALGO_WM || s->algo == PM_ALGO_WMV ? s->dwm.dg
+                        : s->algo == PM_ALGO_ACV                        ? s->dacv.dg
+                        : s->algo == PM_ALGO_AC && s->dac2.use          ? nullptr
+                                                                        : s->dac.dg;
+    if (s->host_only ? !s->gram.ok : !dg) return PM_SCAN_METHOD;
+    return s->gram.dense ? PM_SCAN_DENSE : PM_SCAN_GRAMS;
+}
+
 int pm_scan_status(const void *d_workspace, void *stream)
 {
     if (!d_workspace) return PM_EINVAL;

@@ -24,10 +24,11 @@ PM_OK, PM_EINVAL, PM_ENOMEM, PM_ECUDA, PM_ETOOBIG, PM_ETIMEOUT, PM_ECAPACITY, PM
 PM_HOST_TEXT, PM_DEVICE_TEXT, PM_COUNTS_ONLY = 0, 1, 2
 PM_PLACE_AUTO, PM_PLACE_SMEM, PM_PLACE_HYBRID, PM_PLACE_GLOBAL = range(4)
 PM_ALGO_AC, PM_ALGO_WM, PM_ALGO_PFAC, PM_ALGO_ACV, PM_ALGO_WMV = 1, 2, 3, 4, 5
+PM_SCAN_METHOD, PM_SCAN_GRAMS, PM_SCAN_DENSE = range(3)
 
 EXPORTED = [
     "pm_ac_compile", "pm_pfac_compile", "pm_acv_compile", "pm_wm_compile", "pm_wmv_compile", "pm_set_free", "pm_set_get_info",
-    "pm_plan_for_device", "pm_scan",
+    "pm_plan_for_device", "pm_set_scan_kind", "pm_scan",
     "pm_scan_to_host", "pm_result_free", "pm_scan_workspace_bytes", "pm_scan_device",
     "pm_scan_device_noalloc", "pm_noalloc_scratch_bytes", "pm_noalloc_scan_status", "pm_scan_status",
     "pm_scan_batch", "pm_batch_prepare", "pm_batch_free", "pm_batch_counts_total",
@@ -130,6 +131,8 @@ def lib():
         L.pm_set_free.argtypes = [vp]
         L.pm_set_get_info.restype = ctypes.c_int
         L.pm_set_get_info.argtypes = [vp, ctypes.POINTER(pm_set_info)]
+        L.pm_set_scan_kind.restype = ctypes.c_int32
+        L.pm_set_scan_kind.argtypes = [vp]
         L.pm_plan_for_device.restype = ctypes.c_int
         L.pm_plan_for_device.argtypes = [vp, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32,
                                          ctypes.POINTER(pm_plan_info)]
@@ -332,6 +335,10 @@ def pm_set_get_info(h: int) -> dict:
     info = pm_set_info()
     _check(lib().pm_set_get_info(h, ctypes.byref(info)), "pm_set_get_info")
     return {name: getattr(info, name) for name, _ in info._fields_}
+
+
+def pm_set_scan_kind(h: int) -> int:
+    return int(lib().pm_set_scan_kind(h))
 
 
 def pm_plan_for_device(h: int, sm_count: int, smem_optin: int, smem_per_sm: int) -> dict:
@@ -609,6 +616,10 @@ class PatternSet:
 
     def info(self) -> dict:
         return pm_set_get_info(self.h)
+
+    def scan_kind(self) -> int:
+        """PM_SCAN_METHOD, PM_SCAN_GRAMS or PM_SCAN_DENSE: what scans take."""
+        return pm_set_scan_kind(self.h)
 
     def plan_for(self, sm_count: int, smem_optin: int, smem_per_sm: int) -> dict:
         """The planner's launch plan for this AC or PFAC set on a device of the
