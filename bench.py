@@ -57,7 +57,7 @@ def measured_peaks() -> tuple[float, str]:
     return 6800.0, "fallback"
 
 
-PLAN_KEYS = ("placement", "warps_per_cta", "counters", "ids_place", "stride")
+PLAN_KEYS = ("placement", "warps_per_cta", "ctas_per_sm", "counters", "ids_place", "stride")
 
 
 def plan_key(plan) -> dict:
@@ -66,6 +66,7 @@ def plan_key(plan) -> dict:
     plan = plan or {}
     key = {k: int(plan.get(k, 0)) for k in PLAN_KEYS}
     key["stride"] = 2 if key["stride"] == 2 else 1
+    key["ctas_per_sm"] = max(key["ctas_per_sm"], 1)  # 0 is 1 to the planner; the kernel's name tells grams apart
     return key
 
 
@@ -325,7 +326,7 @@ def main():
     if not args.no_tune and not pinned_plan and args.algo == "ac":  # the autotuner picks the launch plan (not timed)
         params, tms = s.tune(d_text, counts_only=args.mode == "counts", reps=3)
         tuned = {"ms_per_scan": tms,
-                 **{k: params[k] for k in ("placement", "warps_per_cta", "counters", "ids_place", "stride")}}
+                 **{k: params[k] for k in PLAN_KEYS}}
     info = s.info()
     ws = torch.zeros(s.workspace_bytes(n), dtype=torch.uint8, device="cuda")
     counts = torch.zeros(d, dtype=torch.int64, device="cuda")

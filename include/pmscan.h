@@ -349,7 +349,9 @@ int pm_noalloc_scan_status(void *stream);
  * one kept has the counters that fit best for counts-only scans.
  * Results never depend on the plan. Allocates its own scratch, synchronises
  * `stream`. *best_out / *best_ms (may be NULL) receive the chosen pm_params
- * and its time per scan. Wu-Manber sets tune the gram scan and warps per CTA
+ * and its time per scan; the same patterns compiled with them take the same
+ * scan (automatic parameters mean the gram scan; where the method's own scan
+ * wins with the plan it has by default, ctas_per_sm is 1). Wu-Manber sets tune the gram scan and warps per CTA
  * (auto, 24, 20, 16, 12, 8; more than 16 for exact-code tables of ACGT sets).
  * PM_EINVAL for PFAC and mixed-length sets and for host-only sets.
  */

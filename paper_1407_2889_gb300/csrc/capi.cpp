@@ -255,12 +255,20 @@ int upload_wm(pm_set *s)
 
 // The gram tables of a set whose launch plan is automatic: scans then take
 // them instead of the automaton or the shift tables (scan_gram.cu).
-bool plan_is_automatic(const pm_set *s)
+bool plan_is_automatic(int algo, const pm_params &p)
 {
-    const pm_params &p = s->params;
-    if (s->algo == PM_ALGO_WM || s->algo == PM_ALGO_WMV) return p.warps_per_cta == 0 && p.ctas_per_sm == 0;
+    if (algo == PM_ALGO_WM || algo == PM_ALGO_WMV) return p.warps_per_cta == 0 && p.ctas_per_sm == 0;
     return p.placement == PM_PLACE_AUTO && p.smem_table_bytes == 0 && p.warps_per_cta == 0 && p.ctas_per_sm == 0 &&
            p.counters == 0 && p.ids_place == 0 && p.stride <= 1;
+}
+
+// The tuners' parameters of a plan that walks the method's own tables: where
+// the set has gram tables, automatic ones would compile to the gram scan.
+// Pinning one CTA per SM, which both planners take anyway, tells them apart.
+pm_params own_scan_params(const pm_set *s, pm_params p)
+{
+    if (s->dgram.use && plan_is_automatic(s->algo, p)) p.ctas_per_sm = 1;
+    return p;
 }
 
 int upload_gram(pm_set *s, const DeviceProps &dp)
@@ -312,7 +320,7 @@ class GramJob {
 public:
     GramJob(pm_set *s, const uint8_t *P, const int64_t *off, int64_t d, int32_t m)
     {
-        if (!plan_is_automatic(s)) return;
+        if (!plan_is_automatic(s->algo, s->params)) return;
         const bool limited = s->algo == PM_ALGO_AC;
         auto work = [=]() { rc_ = build_gram(P, off, d, m, limited, s->gram); };
         if (d >= 256) {
@@ -793,6 +801,8 @@ static int tune_wm(pm_set *s, const uint8_t *d_text, int64_t n, bool list, int32
         if (w < 0 && !s->dgram.use) continue;
         pm_params p = s->params;
         p.warps_per_cta = w < 0 ? 0 : w;
+        if (w < 0) p.ctas_per_sm = 0;
+        else p = own_scan_params(s, p);
         DevWm plan = saved;
         if (wm_plan(t, p, dp, plan) != PM_OK) continue;
         plan.gt = w < 0 ? &s->gram : nullptr;
@@ -881,6 +891,7 @@ int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t
     if (s->dgram.use) cand.push_back(pm_params{});  // the gram scan
     cand.push_back(s->params);
     cand.back().stride = 1;
+    cand.back() = own_scan_params(s, cand.back());
     for (int place : {PM_PLACE_AUTO, PM_PLACE_HYBRID})
         for (int w : {0, 24, 20, 16, 12, 8})
             for (int c : {0, 1, 2, 3})
@@ -892,7 +903,7 @@ int pm_tune(pm_set *s, const uint8_t *d_text, int64_t n, uint32_t flags, int32_t
                     p.counters = c;
                     p.ids_place = idp;
                     p.smem_table_bytes = 0;
-                    cand.push_back(p);
+                    cand.push_back(own_scan_params(s, p));
                 }
     struct Tried { DevAc plan; pm_params params; float ms; };
     std::vector<Tried> tried;
