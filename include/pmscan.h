@@ -547,7 +547,10 @@ int pm_selfcheck_host_walk(const pm_set *s, const uint8_t *T, int64_t n, pm_resu
 /*
  * The same for the set's sampled-gram tables (the ones its scans on a GPU
  * take when the launch plan is automatic): a host walk of them. PM_EINVAL for
- * a set that has none (a pinned launch plan, or patterns too short).
+ * a set that has none (a pinned launch plan, patterns too short, or so many
+ * or so repetitive ones that the method's own scan is planned to be faster; a
+ * Wu-Manber set of repetitive patterns keeps the tables for this walk, see
+ * pm_set_scan_kind).
  */
 int pm_selfcheck_gram_walk(const pm_set *s, const uint8_t *T, int64_t n, pm_result **out);
 

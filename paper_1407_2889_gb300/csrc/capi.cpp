@@ -275,7 +275,7 @@ int upload_gram(pm_set *s, const DeviceProps &dp)
 {
     const GramTables &t = s->gram;
     DevGram &d = s->dgram;
-    if (!t.ok) return PM_OK;
+    if (!t.ok || !t.scan) return PM_OK;
     int rc = gram_plan(t, dp, d);
     if (rc || !d.use) return rc;
     // one allocation and one copy: a small set's compile is mostly these
@@ -318,11 +318,10 @@ int upload_gram(pm_set *s, const DeviceProps &dp)
 // the set is large enough for that to pay (100,000 32-mers: 65 of 355 ms).
 class GramJob {
 public:
-    GramJob(pm_set *s, const uint8_t *P, const int64_t *off, int64_t d, int32_t m)
+    GramJob(pm_set *s, const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32_t B = 0)
     {
         if (!plan_is_automatic(s->algo, s->params)) return;
-        const bool limited = s->algo == PM_ALGO_AC;
-        auto work = [=]() { rc_ = build_gram(P, off, d, m, limited, s->gram); };
+        auto work = [=]() { rc_ = build_gram(P, off, d, m, s->algo, B, s->gram); };
         if (d >= 256) {
             try {
                 thread_ = std::thread(work);
@@ -571,7 +570,7 @@ int pm_wmv_compile(const uint8_t *P, const int64_t *offsets, int64_t d, int32_t 
     if (opt) s->params = *opt;
     s->host_only = s->params.host_only != 0;
     const int bp = s->params.wm_prefix_len > 0 ? s->params.wm_prefix_len : 2;
-    GramJob gram(s, P, offsets, d, 0);
+    GramJob gram(s, P, offsets, d, 0, B);
     int rc = build_wmv(P, offsets, d, B, bp, s->wm);
     const int rg = gram.join();
     if (!rc) rc = rg;
@@ -593,7 +592,7 @@ int pm_wm_compile(const uint8_t *P, int64_t d, int32_t m, int32_t B, const pm_pa
     s->host_only = s->params.host_only != 0;
     int bp = s->params.wm_prefix_len > 0 ? s->params.wm_prefix_len : 2;
     if (bp > m) bp = m;
-    GramJob gram(s, P, nullptr, d, m);
+    GramJob gram(s, P, nullptr, d, m, B);
     int rc = build_wm(P, d, m, B, bp, s->wm);
     const int rg = gram.join();
     if (!rc) rc = rg;
@@ -1003,7 +1002,7 @@ int32_t pm_set_scan_kind(const pm_set *s)
                         : s->algo == PM_ALGO_ACV                        ? s->dacv.dg
                         : s->algo == PM_ALGO_AC && s->dac2.use          ? nullptr
                                                                         : s->dac.dg;
-    if (s->host_only ? !s->gram.ok : !dg) return PM_SCAN_METHOD;
+    if (s->host_only ? !s->gram.ok || !s->gram.scan : !dg) return PM_SCAN_METHOD;
     return s->gram.dense ? PM_SCAN_DENSE : PM_SCAN_GRAMS;
 }
 

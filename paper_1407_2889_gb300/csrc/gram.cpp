@@ -59,15 +59,70 @@ uint32_t codes(const uint8_t *p, int64_t len)
     return x;
 }
 
+// What the method's own scan does with a set whose grams are poor. The figures
+// are one pass over 16 MiB, list mode, unless they say otherwise.
+struct GramLimits {
+    double cost;        // planned instructions per lane and 16 characters (sampled grams)
+    double entries;     // entries compared per position of random text
+    double dense_pass;  // part of all texts' m-grams in a dense set
+    uint32_t longest;   // entries of one gram
+};
+
+// matches: matches per position of random text, hits: entries of a gram of it
+GramLimits gram_limits(int32_t algo, int32_t B, int64_t d, int letters, bool packed, int hi, double matches,
+                       double hits)
+{
+    // Cost. The transition-table walk of a one-length Aho-Corasick set takes, in
+    // units of about 4.6 us per GiB: tables of fewer than about 2,000 patterns in
+    // shared memory 0.8 ms per GiB, larger ones past it 3 ms, general alphabets
+    // 4.4 ms; a PFAC walk 11 ms and more. Wu-Manber compares every candidate of a
+    // window in turn and is never faster (1.2 to 70 times slower).
+    //
+    // Entries. The mixed-length automaton takes about 1,300 M + 120 M^2 us per 4
+    // MiB with M matches a position, grams about 65 per entry. Patterns over ACGT
+    // (entries and M; ms per 4 MiB with grams and without): 3,000 of 3 to 65
+    // letters (47, 1.0) 1.98 and 1.26; 20,000 of 4 to 40 (78, 2.8) 5.8 and 4.3; of
+    // 5 to 30 (20, 1.0) 1.62 and 1.55; of 6 to 20 (5, 0.43) 0.53 and 0.76; 100,000
+    // of 3 to 65 (1,560, 33) 91 and 176.
+    //
+    // Dense sets that hold most m-grams. 8 MiB: 3,000 5-mers (95 % of all) 336 us
+    // and 319 by the automaton (PFAC 338 and 294), 300 4-mers (69 %) 199 and 204
+    // (199 and 189); 3,000 6-mers (52 %) 128 and 181 (127 and 185).
+    //
+    // A gram with hundreds of entries means repetitive patterns (runs of one
+    // letter): in a text with such repeats every occurrence costs them all, and
+    // work grows as text times d. The automata do not care. 4,000 32-mers of
+    // which f begin with 24 A, text with 2 % of such runs (576, 2,304 and 36,000
+    // entries at f = 64, 256 and 4,000): grams 0.18, 0.72 and 16 ms; automaton
+    // 0.09, one or mixed lengths 0.10, PFAC 0.37. The limits are about where the
+    // two meet at 2 %. Wu-Manber depends on its blocks: the exact tables (four
+    // letters or fewer, up to 32 characters) take 0.28, 0.33 and 2.0 ms with B = 2
+    // and 0.10, 0.10 and 0.22 with B = 4; byte-hash tables over 20 letters 0.29,
+    // 0.45 and 4.2 with B = 2, 0.04 with B = 4. Where a block names more than 64
+    // patterns (d / letters^B) every window compares them, and grams win at any
+    // length: 4,000 patterns of 32 to 47 letters over ACGT 0.18, 0.74 and 17 ms,
+    // without 8.1, 13 and 101.
+    // Lists a few times longer than those of random text are no sign of
+    // repetition. (At most 2^18: a tile's keys are added up in 32 bits, at most
+    // 2^14 starts with all patterns of one gram each.)
+    constexpr uint32_t most = (1u << 18) - 1u;
+    auto longest = [&](uint32_t n) { return uint32_t(std::min(std::max(double(n), 4.0 * hits), double(most))); };
+    constexpr double any = 1e30;
+    switch (algo) {
+    case PM_ALGO_AC: return {packed ? (d < 2000 ? 170.0 : 650.0) : 900.0, any, 0.6, longest(256)};
+    case PM_ALGO_PFAC: return {2400.0, any, 0.6, longest(1024)};
+    case PM_ALGO_ACV: return {any, 0.5 + matches * (20.0 + 1.8 * matches), 1.0, longest(256)};
+    default: break;
+    }
+    const bool exact = packed && hi <= 32;
+    if (!exact && double(d) > 64.0 * std::pow(double(letters), double(B))) return {any, any, 1.0, most};
+    return {any, any, 1.0, longest(B < 3 ? 1024 : exact ? 256 : 64)};
+}
+
 }  // namespace
 
-int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool limited, GramTables &t)
+int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32_t algo, int32_t B, GramTables &t)
 {
-    // What the transition-table walk of a one-length Aho-Corasick set costs in
-    // the same unit (about 4.6 us per GiB each): tables of fewer than about
-    // 2,000 patterns in shared memory 0.8 ms per GiB, larger ones past it 3 ms,
-    // general alphabets 4.4 ms. The other scans are always slower.
-    const double small = limited ? 170.0 : 1e30, large = limited ? 650.0 : 1e30, general = limited ? 900.0 : 1e30;
     t = GramTables();
     try {
         const bool var = off != nullptr;
@@ -116,7 +171,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
         // away most windows of the longer patterns in a mixed set: 8,000 of 8 to
         // 16 characters with 8-character grams took 567 us per 256 MiB, 1,000
         // 121 us per 128 MiB.
-        double best = 1e30;
+        double best = 1e30, best_hits = 0.0, dense_pass = 0.0;
         for (int s = 16; s >= 1; s >>= 1) {
             const int shortest = lo - s + 1;
             for (int form = 0; form < (packed ? 3 : 1); ++form) {
@@ -153,12 +208,18 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
                     t.direct = direct;
                     t.rank = direct && 2 * q <= 18;
                     t.dense = dense;
+                    best_hits = hits;
+                    dense_pass = natural;
                 }
             }
         }
         // too short for any gram, too many patterns, or so many candidates that
-        // the automaton is faster
-        if (t.s == 0 || (!t.dense && best > (packed ? (d < 2000 ? small : large) : general))) {
+        // the method's own scan is faster
+        double matches = 0.0;
+        for (int L = lo; L <= hi; ++L)
+            matches += double(with_len[L]) / std::pow(double(std::max(letters, 2)), double(L));
+        const GramLimits lim = gram_limits(algo, B, d, letters, packed, hi, matches, best_hits);
+        if (t.s == 0 || (t.dense ? dense_pass > lim.dense_pass : best > lim.cost || best_hits / t.s > lim.entries)) {
             t = GramTables();
             return PM_OK;
         }
@@ -275,15 +336,14 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool 
         std::vector<uint32_t> at(nb + 1, 0u);
         for (const Gram &x : grams) ++at[bucket(x.h) + 1];
         for (size_t b = 0; b < nb; ++b) at[b + 1] += at[b];
-        // A gram with hundreds of entries means repetitive patterns (runs of one
-        // letter): in a text with such repeats every occurrence costs them all.
-        // The automaton does not care: 64 MiB with 2 % of runs of A, 8,000 32-mers,
-        // 82 of them with such a run (650 entries): 0.63 ms, grams 2.8.
         uint32_t longest = 0;
         for (size_t b = 0; b < nb; ++b) longest = std::max(longest, at[b + 1] - at[b]);
-        if (limited && longest > 256u) {
-            t = GramTables();
-            return PM_OK;
+        if (longest > lim.longest) {
+            if (algo != PM_ALGO_WM && algo != PM_ALGO_WMV) {
+                t = GramTables();
+                return PM_OK;
+            }
+            t.scan = false;
         }
         t.dir.assign(2 * (nb + 1), 0u);
         for (size_t b = 0; b <= nb; ++b) {

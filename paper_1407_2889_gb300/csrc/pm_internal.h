@@ -157,6 +157,7 @@ struct GramEntry {
 
 struct GramTables {
     bool ok = false;
+    bool scan = true;              // false: for the host walk only, scans keep the method's own tables
     bool var = false;              // mixed lengths: no groups, code = pattern id
     bool direct = false;           // the hash is the gram itself, shifted to the top: the filter is exact
     bool rank = false;             // buckets by rank in the filter
@@ -187,9 +188,9 @@ struct GramTables {
 
 int build_ac(const uint8_t *P, int64_t d, int32_t m, AcTables &out);
 // off NULL: d rows of length m; else pattern r is P[off[r] .. off[r+1]).
-// t.ok stays false (and PM_OK is returned) when the set has no gram plan or,
-// `limited`, when walking its transition table is planned to be faster.
-int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, bool limited, GramTables &t);
+// t.ok stays false (and PM_OK is returned) when the set has no gram plan or the
+// scan of its own method (algo, and B for Wu-Manber) is planned to be faster.
+int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32_t algo, int32_t B, GramTables &t);
 void host_walk_gram(const GramTables &t, const uint8_t *T, int64_t n,
                     std::vector<uint64_t> &occ, std::vector<int64_t> &counts);
 // pattern r is P[off[r] .. off[r+1]); lengths 1..kAcvMaxLen

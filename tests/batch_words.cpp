@@ -22,7 +22,7 @@ int main()
         for (auto &c : P) c = "ACGT"[rng() & 3u];
         sets[k].algo = PM_ALGO_AC;
         if (build_ac(P.data(), d, int32_t(m), sets[k].ac) ||
-            build_gram(P.data(), nullptr, d, int32_t(m), true, sets[k].gram) || !sets[k].gram.ok)
+            build_gram(P.data(), nullptr, d, int32_t(m), PM_ALGO_AC, 0, sets[k].gram) || !sets[k].gram.ok)
             return 2;
         sets[k].dac.dg = &sets[k].dgram;   // the scans of a set just compiled take its grams
         inst[k] = BatchInst{&sets[k], 0, texts[k], 0, 0, texts[k], k, batch_takes_grams(&sets[k])};
