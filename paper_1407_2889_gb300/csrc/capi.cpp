@@ -81,10 +81,11 @@ int device_props(DeviceProps &p)
 
 namespace {
 
-// Copy `bytes` to a fresh device allocation padded to a multiple of 16.
-int upload(void **dst, const void *src, size_t bytes, int64_t &total)
+// Copy `bytes` to a fresh, zeroed device allocation of `room` bytes padded to
+// a multiple of 16.
+int upload(void **dst, const void *src, size_t bytes, size_t room, int64_t &total)
 {
-    size_t padded = (bytes + 15) & ~size_t(15);
+    size_t padded = (room + 15) & ~size_t(15);
     if (padded == 0) padded = 16;
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, padded);
@@ -103,6 +104,11 @@ int upload(void **dst, const void *src, size_t bytes, int64_t &total)
     *dst = p;
     total += int64_t(padded);
     return PM_OK;
+}
+
+int upload(void **dst, const void *src, size_t bytes, int64_t &total)
+{
+    return upload(dst, src, bytes, bytes, total);
 }
 
 void free_dev(void *&p)
@@ -292,14 +298,15 @@ int upload_gram(pm_set *s, const DeviceProps &dp)
         {t.ids.data(), t.ids.size() * 2, reinterpret_cast<void **>(&d.ids)}};
     size_t total = 0;
     for (const auto &p : part) total += (p.bytes + 15) & ~size_t(15);
+    const bool staged = total <= size_t(1) << 20;   // more is worth a copy per table
     try {
-        std::vector<uint8_t> all(total, 0);
+        std::vector<uint8_t> all(staged ? total : 0, 0);
         size_t at = 0;
         for (const auto &p : part) {
-            if (p.bytes) std::memcpy(all.data() + at, p.src, p.bytes);
+            if (staged && p.bytes) std::memcpy(all.data() + at, p.src, p.bytes);
             at += (p.bytes + 15) & ~size_t(15);
         }
-        rc = upload(&d.base, all.data(), all.size(), s->device_bytes);
+        rc = upload(&d.base, all.data(), all.size(), total, s->device_bytes);
     } catch (const std::bad_alloc &) {
         return PM_ENOMEM;
     }
@@ -308,6 +315,9 @@ int upload_gram(pm_set *s, const DeviceProps &dp)
     for (const auto &p : part) {
         *p.dst = static_cast<uint8_t *>(d.base) + at;
         at += (p.bytes + 15) & ~size_t(15);
+        if (staged || !p.bytes) continue;
+        const cudaError_t e = cudaMemcpy(*p.dst, p.src, p.bytes, cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) { set_cuda_error(int(e)); return PM_ECUDA; }
     }
     s->dac.gt = s->dwm.gt = s->dacv.gt = &s->gram;
     s->dac.dg = s->dwm.dg = s->dacv.dg = &s->dgram;

@@ -91,10 +91,14 @@ int build_ac(const uint8_t *P, int64_t d, int32_t m, AcTables &t)
         std::vector<int32_t> go;      // state * W + class -> state, -1 = none
         std::vector<int32_t> depth;
         std::vector<int32_t> first_pat, next_pat(size_t(d), -1), last_pat;
-        go.reserve(size_t(std::min<int64_t>(max_states, int64_t(1) << 26)) * W);
+        const size_t expect = size_t(std::min<int64_t>(max_states, int64_t(1) << 26));
+        go.reserve((expect + 256) * W);
+        depth.reserve(expect);
+        first_pat.reserve(expect);
+        last_pat.reserve(expect);
         auto new_state = [&](int32_t dep) {
             int32_t s = int32_t(depth.size());
-            go.insert(go.end(), size_t(W), -1);
+            if (size_t(s) * W == go.size()) go.resize(go.size() + (size_t(W) << 8), -1);  // 256 rows at a time
             depth.push_back(dep);
             first_pat.push_back(-1);
             last_pat.push_back(-1);

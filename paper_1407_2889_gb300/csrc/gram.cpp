@@ -292,7 +292,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
         // ascending), so that the starts t - k come out in ascending order
         // and equal starts in ascending pattern id
         struct Gram {
-            uint32_t h, c, k;
+            uint32_t h, ck;   // hash; distinct pattern (d <= 2^23) | offset << 24
         };
         std::vector<Gram> grams;
         grams.reserve(nc * size_t(t.s));
@@ -305,14 +305,14 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
                     uint32_t b;
                     const uint32_t x = gram_hash(t, p, &b);
                     t.filter[b >> 5] |= 1u << (b & 31u);
-                    grams.push_back({x, uint32_t(c), uint32_t(k)});
+                    grams.push_back({x, uint32_t(c) | uint32_t(k) << 24});
                     continue;
                 }
                 const uint32_t head = codes(p, have);   // direct grams: every ending
                 for (uint32_t e = 0; e < 1u << (2 * (t.q - have)); ++e) {
                     const uint32_t b = head | e << (2 * have);
                     t.filter[b >> 5] |= 1u << (b & 31u);
-                    grams.push_back({b * t.K[0], uint32_t(c), uint32_t(k)});
+                    grams.push_back({b * t.K[0], uint32_t(c) | uint32_t(k) << 24});
                 }
             }
         const size_t G = grams.size();
@@ -356,13 +356,13 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
         }
         t.ent.resize(G);
         for (const Gram &x : grams) {
-            const uint32_t b = bucket(x.h), e = at[b]++;
-            const int len = len_of(rep[x.c]);
+            const uint32_t b = bucket(x.h), e = at[b]++, c = x.ck & 0xFFFFFFu, k = x.ck >> 24;
+            const int len = len_of(rep[c]);
             GramEntry &en = t.ent[e];
-            en.h = t.qw == 0 ? codes(P + first(rep[x.c]) + x.k, len - int(x.k)) : x.h;
-            en.idx = x.c;
-            en.k_len = x.k | uint32_t(len) << 8;
-            en.code = t.code[x.c];
+            en.h = t.qw == 0 ? codes(P + first(rep[c]) + k, len - int(k)) : x.h;
+            en.idx = c;
+            en.k_len = k | uint32_t(len) << 8;
+            en.code = t.code[c];
             const uint32_t i = e - (t.dir[2 * b] & 0xFFFFFFu);
             for (uint32_t u = i; u < 4 && !t.rank; ++u) {
                 t.dir[2 * b + 1] &= ~(0xFFu << (8 * u));
