@@ -12,11 +12,24 @@ using dev::kFull;
 
 constexpr int kRow = 512;        // text bytes per warp row
 
-// bytes [off, off + 16) of the text, zeros from n on
+// Four bytes in place of those at o, past a text's end: mixed bits (the last
+// steps of MurmurHash3), which pass the filter as seldom as other text. Zeros
+// are the codes of A, and with a gram of A only in the set one warp looked at
+// every position of the last tile's rest: 48 MiB and 100 bytes against 600
+// 16-mers, counts, 28.5 us, with A^16 among them 147, now 28.
+__device__ __forceinline__ uint32_t past_end(long long o)
+{
+    uint32_t x = uint32_t(o) * 0x85EBCA6Bu;
+    x = (x ^ x >> 13) * 0xC2B2AE35u;
+    return x ^ x >> 16;
+}
+
+// bytes [off, off + 16) of the text, past_end from n on (a match is compared
+// with the text itself and ends inside it)
 __device__ __forceinline__ uint4 load16(const uint8_t *text, long long n, bool aligned, long long off)
 {
     if (aligned && off + 16 <= n) return __ldg(reinterpret_cast<const uint4 *>(text + off));
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    uint4 v;
     if (off + 20 <= n) {
         // unaligned text: five aligned words (the last one ends inside the text)
         const uint8_t *p = text + off;
@@ -31,10 +44,15 @@ __device__ __forceinline__ uint4 load16(const uint8_t *text, long long n, bool a
             return v;
         }
     }
-    uint32_t b[4] = {0u, 0u, 0u, 0u};
+    uint32_t b[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) b[j] = past_end(off + 4 * j);
 #pragma unroll
     for (int j = 0; j < 16; ++j)
-        if (off + j < n) b[j >> 2] |= uint32_t(text[off + j]) << (8 * (j & 3));
+        if (off + j < n) {
+            const uint32_t sh = 8u * (j & 3);
+            b[j >> 2] = (b[j >> 2] & ~(0xFFu << sh)) | uint32_t(text[off + j]) << sh;
+        }
     return make_uint4(b[0], b[1], b[2], b[3]);
 }
 
