@@ -316,6 +316,10 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
                 }
             }
         const size_t G = grams.size();
+        uint32_t run[4];   // (K is odd: different grams have different hashes)
+        for (uint32_t c = 0; c < 4; ++c) run[c] = (0x55555555u >> (32 - 2 * t.q)) * c * t.K[0];
+        for (const Gram &x : grams)
+            t.runs = t.runs || (packed && (x.h == run[0] || x.h == run[1] || x.h == run[2] || x.h == run[3]));
         auto bucket = [&](uint32_t x) -> uint32_t {
             if (!t.rank) return x >> (32 - t.db);
             const uint32_t b = x >> (32 - t.fb);
@@ -369,13 +373,13 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
                 t.dir[2 * b + 1] |= ((x.h >> (24 - t.db)) & 0xFFu) << (8 * u);
             }
         }
+        for (uint32_t c = 0; packed && c < 4; ++c) {
+            uint32_t b = 0;
+            while (b < 256 && !(present[b] && code2(b) == c)) ++b;
+            // an absent letter: a byte with another code never equals the text's
+            t.lut |= (b < 256 ? b : (c ^ 1u) << 1) << (8 * c);
+        }
         if (t.dense) {
-            for (uint32_t c = 0; c < 4; ++c) {
-                uint32_t b = 0;
-                while (b < 256 && !(present[b] && code2(b) == c)) ++b;
-                // an absent letter: a byte with another code never equals the text's
-                t.lut |= (b < 256 ? b : (c ^ 1u) << 1) << (8 * c);
-            }
             t.id_off.push_back(0);
             for (const GramEntry &e : t.ent) {
                 const uint32_t gi = e.code & 0x7FFFFFFFu;

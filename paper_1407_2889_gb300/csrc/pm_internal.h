@@ -161,6 +161,7 @@ struct GramTables {
     bool var = false;              // mixed lengths: no groups, code = pattern id
     bool direct = false;           // the hash is the gram itself, shifted to the top: the filter is exact
     bool rank = false;             // buckets by rank in the filter
+    bool runs = false;             // 2-bit grams: one of them is of a single letter
     int64_t d = 0;
     int32_t m_min = 0, m_max = 0;
     uint32_t max_keys = 1;         // largest group of equal patterns
@@ -180,9 +181,9 @@ struct GramTables {
     std::vector<uint32_t> grp_off, grp_ids;
     // Dense form (one-length sets of fewer than 2^15 patterns, s = 1, q = m):
     // the gram is the pattern, so its rank is the distinct pattern's number,
-    // whose ids are ids[id_off[c] .. id_off[c + 1]). lut: the byte of code c in byte c.
+    // whose ids are ids[id_off[c] .. id_off[c + 1]).
     bool dense = false;
-    uint32_t lut = 0;
+    uint32_t lut = 0;                 // 2-bit grams: the letter of code c in byte c
     std::vector<uint16_t> id_off, ids;
 };
 

@@ -47,6 +47,7 @@ struct GramArgs {
     long long n;
     int aligned;
     uint32_t K[4];
+    uint32_t lut;                 // the letter of code c in byte c
     int fshift, wshift, bshift;   // 32 - fb, 32 - (fb - 5), 32 - db
     int fwords;                   // filter words
     const uint32_t *filter_g;
@@ -75,8 +76,9 @@ __host__ __device__ constexpr int qcap(int s) { return 32 + rows_of(s) * kRow / 
 
 // S: stride; QW: 0 2-bit grams, else words of a byte gram; RANK: buckets by
 // rank in the filter, else by hash. The queue holds each passing gram's offset
-// and the codes of the 16 characters from it on (a byte gram's hash).
-template <int S, int QW, bool RANK>
+// and the codes of the 16 characters from it on (a byte gram's hash). RUNS: see
+// letter_probes.
+template <int S, int QW, bool RANK, bool RUNS>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const GramArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -199,13 +201,21 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_scan_kernel(const Gram
             // (32 lanes x NP; four rows only up to two grams each).
             constexpr int F = R == 4 ? 8 : 16;
             uint32_t ex = 0, tot = 0;
-            if (NP > 1) {
+            auto places = [&]() {
                 uint32_t cnt = 0;
 #pragma unroll
                 for (int r = 0; r < R; ++r) cnt |= uint32_t(__popc(mask[r])) << (F * r);
                 const uint32_t inc = dev::warp_incl_scan(cnt, lane);
                 ex = inc - cnt;
                 tot = __shfl_sync(kFull, inc, 31);
+            };
+            if (NP > 1) places();
+            if (RUNS && (NP > 1 ? (tot & ((1u << F) - 1u)) == 32u * NP : __all_sync(kFull, mask[0]))) {
+                const long long base = (long long)st * a.tile + g * (kRow * R) + lane * 16;
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    mask[r] &= letter_probes<S>(a.text, a.n, base + r * kRow, a.lut);
+                if (NP > 1) places();
             }
 #pragma unroll
             for (int r = 0; r < R; ++r) {
@@ -376,7 +386,6 @@ struct DenseArgs {
     uint32_t pmask;               // (pwords - 1) * 4
     uint32_t gmask;               // 4^m - 1
     int m;
-    uint32_t lut;                 // the byte of code c in byte c
     const uint16_t *id_off, *ids; // each distinct pattern's ids
 };
 
@@ -408,7 +417,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_dense_kernel(const Den
     }
     for (int i = threadIdx.x; i < 256; i += blockDim.x) {
         uint32_t x = 0;
-        for (int j = 0; j < 4; ++j) x |= ((da.lut >> (8 * ((i >> (2 * j)) & 3))) & 0xFFu) << (8 * j);
+        for (int j = 0; j < 4; ++j) x |= ((a.lut >> (8 * ((i >> (2 * j)) & 3))) & 0xFFu) << (8 * j);
         s_exp[i] = x;
     }
     __syncthreads();
@@ -496,8 +505,16 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_dense_kernel(const Den
         // ---- hits -> queue (offsets in the tile), lane by lane: both rows'
         // counts in one scan ----
         {
-            const uint32_t cnt = __popc(m0) | __popc(m1) << 16;
-            const uint32_t inc = dev::warp_incl_scan(cnt, lane), tot = __shfl_sync(kFull, inc, 31);
+            uint32_t cnt = __popc(m0) | __popc(m1) << 16;
+            uint32_t inc = dev::warp_incl_scan(cnt, lane), tot = __shfl_sync(kFull, inc, 31);
+            if ((tot & 0xFFFFu) == uint32_t(kRow)) {   // (see letter_probes)
+                const long long base = (long long)row * kRow + lane * 16;
+                m0 &= __brev(letter_probes<1>(a.text, a.n, base, a.lut));
+                m1 &= __brev(letter_probes<1>(a.text, a.n, base + kRow, a.lut));
+                cnt = __popc(m0) | __popc(m1) << 16;
+                inc = dev::warp_incl_scan(cnt, lane);
+                tot = __shfl_sync(kFull, inc, 31);
+            }
             uint32_t at = uint32_t(qn) + ((inc - cnt) & 0xFFFFu);
             uint32_t off = r * kRow + uint32_t(lane) * 16u;
             while (m0) {
@@ -552,7 +569,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 1) gram_dense_kernel(const Den
                     ok = ok && off <= fits;
                     for (int j = 0; ok && j < m; ++j) {
                         const uint32_t b = tp[off + j], c = (b >> 1) & 3u;
-                        ok = b == ((da.lut >> (8 * c)) & 0xFFu);
+                        ok = b == ((a.lut >> (8 * c)) & 0xFFu);
                         gram |= c << (2 * j);
                     }
                 }
@@ -774,26 +791,28 @@ typedef void (*GramKernel)(const GramArgs);
 
 inline long long up4w(long long x) { return (x + 3) & ~3LL; }
 
-template <int QW, bool RANK>
+template <int QW, bool RANK, bool RUNS>
 GramKernel by_stride(int s)
 {
     switch (s) {
-    case 1: return gram_scan_kernel<1, QW, RANK>;
-    case 2: return gram_scan_kernel<2, QW, RANK>;
-    case 4: return gram_scan_kernel<4, QW, RANK>;
-    case 8: return gram_scan_kernel<8, QW, RANK>;
-    default: return gram_scan_kernel<16, QW, RANK>;
+    case 1: return gram_scan_kernel<1, QW, RANK, RUNS>;
+    case 2: return gram_scan_kernel<2, QW, RANK, RUNS>;
+    case 4: return gram_scan_kernel<4, QW, RANK, RUNS>;
+    case 8: return gram_scan_kernel<8, QW, RANK, RUNS>;
+    default: return gram_scan_kernel<16, QW, RANK, RUNS>;
     }
 }
 
 GramKernel kernel_of(const GramTables &t)
 {
     switch (t.qw) {
-    case 0: return t.rank ? by_stride<0, true>(t.s) : by_stride<0, false>(t.s);
-    case 1: return by_stride<1, false>(t.s);
-    case 2: return by_stride<2, false>(t.s);
-    case 3: return by_stride<3, false>(t.s);
-    default: return by_stride<4, false>(t.s);
+    case 0:
+        if (t.runs) return t.rank ? by_stride<0, true, true>(t.s) : by_stride<0, false, true>(t.s);
+        return t.rank ? by_stride<0, true, false>(t.s) : by_stride<0, false, false>(t.s);
+    case 1: return by_stride<1, false, false>(t.s);
+    case 2: return by_stride<2, false, false>(t.s);
+    case 3: return by_stride<3, false, false>(t.s);
+    default: return by_stride<4, false, false>(t.s);
     }
 }
 
@@ -856,6 +875,7 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
     a.n = n;
     a.aligned = (reinterpret_cast<uintptr_t>(d_text) & 15) == 0;
     for (int j = 0; j < 4; ++j) a.K[j] = t.K[j];
+    a.lut = t.lut;
     a.fshift = 32 - t.fb;
     a.wshift = 37 - t.fb;
     a.bshift = 32 - t.db;
@@ -927,7 +947,6 @@ int gram_launch(const GramTables &t, const DevGram &dv, const uint8_t *d_text, i
         da.pmask = uint32_t(da.pwords - 1) * 4u;
         da.gmask = (1u << (2 * t.q)) - 1u;
         da.m = t.q;
-        da.lut = t.lut;
         da.id_off = dv.id_off;
         da.ids = dv.ids;
         const long long smem = dense_smem(t, pair, warps);
