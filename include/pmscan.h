@@ -217,8 +217,9 @@ int pm_wmv_compile(const uint8_t *P, const int64_t *offsets, int64_t d, int32_t 
 
 void pm_set_free(pm_set *s);
 int pm_set_get_info(const pm_set *s, pm_set_info *info);
-/* Which scan the set's pm_scan, pm_scan_to_host and pm_scan_device take, until
- * pm_tune changes it: PM_SCAN_METHOD the method's own (automaton, SHIFT
+/* Which scan the set's pm_scan, pm_scan_to_host and pm_scan_device take in list
+ * mode (and with PM_COUNTS_ONLY, but for mixed-length automata, whose counts
+ * are often faster without grams), until pm_tune changes it: PM_SCAN_METHOD the method's own (automaton, SHIFT
  * tables), PM_SCAN_GRAMS sampled grams, PM_SCAN_DENSE grams at every position
  * (see pm_set above). For a host-only set, the one its tables are planned for.
  * -1 for NULL. */

@@ -281,7 +281,7 @@ int upload_gram(pm_set *s, const DeviceProps &dp)
 {
     const GramTables &t = s->gram;
     DevGram &d = s->dgram;
-    if (!t.ok || !t.scan) return PM_OK;
+    if (!t.ok || (!t.list && !t.counts)) return PM_OK;
     int rc = gram_plan(t, dp, d);
     if (rc || !d.use) return rc;
     // one allocation and one copy: a small set's compile is mostly these
@@ -1012,7 +1012,8 @@ int32_t pm_set_scan_kind(const pm_set *s)
                         : s->algo == PM_ALGO_ACV                        ? s->dacv.dg
                         : s->algo == PM_ALGO_AC && s->dac2.use          ? nullptr
                                                                         : s->dac.dg;
-    if (s->host_only ? !s->gram.ok || !s->gram.scan : !dg) return PM_SCAN_METHOD;
+    if (s->host_only ? !s->gram.ok : !dg) return PM_SCAN_METHOD;
+    if (!s->gram.list) return PM_SCAN_METHOD;
     return s->gram.dense ? PM_SCAN_DENSE : PM_SCAN_GRAMS;
 }
 

@@ -59,18 +59,26 @@ uint32_t codes(const uint8_t *p, int64_t len)
     return x;
 }
 
-// What the method's own scan does with a set whose grams are poor. The figures
-// are one pass over 16 MiB, list mode, unless they say otherwise.
+// What a set and its gram plan are like, per position of random text.
+struct GramShape {
+    int64_t d;
+    int letters, hi;
+    bool packed;
+    double matches;     // matches
+    double hits;        // entries of one gram
+    double pass;        // grams that pass the filter, per probe
+    double states;      // the set's trie
+};
+
+// When the method's own scan is taken all the same. Times are of one pass over
+// 64 MiB, list mode, unless they say otherwise.
 struct GramLimits {
     double cost;        // planned instructions per lane and 16 characters (sampled grams)
-    double entries;     // entries compared per position of random text
     double dense_pass;  // part of all texts' m-grams in a dense set
     uint32_t longest;   // entries of one gram
 };
 
-// matches: matches per position of random text, hits: entries of a gram of it
-GramLimits gram_limits(int32_t algo, int32_t B, int64_t d, int letters, bool packed, int hi, double matches,
-                       double hits)
+GramLimits gram_limits(int32_t algo, int32_t B, const GramShape &g)
 {
     // Cost. The transition-table walk of a one-length Aho-Corasick set takes, in
     // units of about 4.6 us per GiB: tables of fewer than about 2,000 patterns in
@@ -78,21 +86,14 @@ GramLimits gram_limits(int32_t algo, int32_t B, int64_t d, int letters, bool pac
     // 4.4 ms; a PFAC walk 11 ms and more. Wu-Manber compares every candidate of a
     // window in turn and is never faster (1.2 to 70 times slower).
     //
-    // Entries. The mixed-length automaton takes about 1,300 M + 120 M^2 us per 4
-    // MiB with M matches a position, grams about 65 per entry. Patterns over ACGT
-    // (entries and M; ms per 4 MiB with grams and without): 3,000 of 3 to 65
-    // letters (47, 1.0) 1.98 and 1.26; 20,000 of 4 to 40 (78, 2.8) 5.8 and 4.3; of
-    // 5 to 30 (20, 1.0) 1.62 and 1.55; of 6 to 20 (5, 0.43) 0.53 and 0.76; 100,000
-    // of 3 to 65 (1,560, 33) 91 and 176.
-    //
     // Dense sets that hold most m-grams. 8 MiB: 3,000 5-mers (95 % of all) 336 us
     // and 319 by the automaton (PFAC 338 and 294), 300 4-mers (69 %) 199 and 204
     // (199 and 189); 3,000 6-mers (52 %) 128 and 181 (127 and 185).
     //
     // A gram with hundreds of entries means repetitive patterns (runs of one
     // letter): in a text with such repeats every occurrence costs them all, and
-    // work grows as text times d. The automata do not care. 4,000 32-mers of
-    // which f begin with 24 A, text with 2 % of such runs (576, 2,304 and 36,000
+    // work grows as text times d. The automata do not care. 16 MiB with 2 % of
+    // runs of A, 4,000 32-mers of which f begin with 24 A (576, 2,304 and 36,000
     // entries at f = 64, 256 and 4,000): grams 0.18, 0.72 and 16 ms; automaton
     // 0.09, one or mixed lengths 0.10, PFAC 0.37. The limits are about where the
     // two meet at 2 %. Wu-Manber depends on its blocks: the exact tables (four
@@ -106,17 +107,36 @@ GramLimits gram_limits(int32_t algo, int32_t B, int64_t d, int letters, bool pac
     // repetition. (At most 2^18: a tile's keys are added up in 32 bits, at most
     // 2^14 starts with all patterns of one gram each.)
     constexpr uint32_t most = (1u << 18) - 1u;
-    auto longest = [&](uint32_t n) { return uint32_t(std::min(std::max(double(n), 4.0 * hits), double(most))); };
+    auto longest = [&](uint32_t n) { return uint32_t(std::min(std::max(double(n), 4.0 * g.hits), double(most))); };
     constexpr double any = 1e30;
     switch (algo) {
-    case PM_ALGO_AC: return {packed ? (d < 2000 ? 170.0 : 650.0) : 900.0, any, 0.6, longest(256)};
-    case PM_ALGO_PFAC: return {2400.0, any, 0.6, longest(1024)};
-    case PM_ALGO_ACV: return {any, 0.5 + matches * (20.0 + 1.8 * matches), 1.0, longest(256)};
+    case PM_ALGO_AC: return {g.packed ? (g.d < 2000 ? 170.0 : 650.0) : 900.0, 0.6, longest(256)};
+    case PM_ALGO_PFAC: return {2400.0, 0.6, longest(1024)};
+    case PM_ALGO_ACV: return {any, 1.0, longest(256)};
     default: break;
     }
-    const bool exact = packed && hi <= 32;
-    if (!exact && double(d) > 64.0 * std::pow(double(letters), double(B))) return {any, any, 1.0, most};
-    return {any, any, 1.0, longest(B < 3 ? 1024 : exact ? 256 : 64)};
+    const bool exact = g.packed && g.hi <= 32;
+    if (!exact && double(g.d) > 64.0 * std::pow(double(g.letters), double(B))) return {any, 1.0, most};
+    return {any, 1.0, longest(B < 3 ? 1024 : exact ? 256 : 64)};
+}
+
+// Mixed lengths: the automaton against grams, in list mode and for counts, by
+// estimates in us per 64 MiB of random text. Both were fitted to some 100 sets
+// (30 to 100,000 patterns from 3 to 65 characters, 2, 4 and 20 letters): grams
+// cost by windows that pass, entries compared and keys, the automaton by
+// matches, far more in list mode, and by whether its table is small. Counts with
+// grams and without: 3,000 patterns of 3 to 65 letters over ACGT 11,600 us and
+// 3,800, 8,000 of 5 to 8 3,740 and 3,050, 8,000 of 6 to 9 1,370 and 3,080, 8,000
+// of 8 to 16 95 and 340; list mode 12,800 and 7,700, 4,440 and 11,050, 1,530 and
+// 6,130, 102 and 406.
+void acv_modes(const GramShape &g, int s, bool &list, bool &counts)
+{
+    const double M = g.matches, grams = 40.0 + 1000.0 * g.pass / s + 300.0 * g.hits / s;
+    const double base = g.packed ? 75.0 : 150.0;
+    const bool small = g.states < 8192.0;
+    counts = grams <= (small ? base + 900.0 * M : 250.0 + 3400.0 * std::sqrt(M));
+    list = grams + 500.0 * M <=
+           (small ? base + M * (1500.0 + 3000.0 * M) : 250.0 + 8000.0 * std::sqrt(M) + 1000.0 * M * M);
 }
 
 }  // namespace
@@ -171,7 +191,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
         // away most windows of the longer patterns in a mixed set: 8,000 of 8 to
         // 16 characters with 8-character grams took 567 us per 256 MiB, 1,000
         // 121 us per 128 MiB.
-        double best = 1e30, best_hits = 0.0, dense_pass = 0.0;
+        double best = 1e30, best_hits = 0.0, best_pass = 0.0;
         for (int s = 16; s >= 1; s >>= 1) {
             const int shortest = lo - s + 1;
             for (int form = 0; form < (packed ? 3 : 1); ++form) {
@@ -213,17 +233,21 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
                     t.rank = direct && 2 * q <= 18;
                     t.dense = dense;
                     best_hits = hits;
-                    dense_pass = natural;
+                    best_pass = dense ? natural : pass;
                 }
             }
         }
         // too short for any gram, too many patterns, or so many candidates that
         // the method's own scan is faster
-        double matches = 0.0;
-        for (int L = lo; L <= hi; ++L)
-            matches += double(with_len[L]) / std::pow(double(std::max(letters, 2)), double(L));
-        const GramLimits lim = gram_limits(algo, B, d, letters, packed, hi, matches, best_hits);
-        if (t.s == 0 || (t.dense ? dense_pass > lim.dense_pass : best > lim.cost || best_hits / t.s > lim.entries)) {
+        GramShape shape{d, letters, hi, packed, 0.0, best_hits, best_pass, 1.0};
+        for (int L = hi, longer = 0; L >= 1; --L) {
+            const double grams = std::pow(double(std::max(letters, 2)), double(L));
+            longer += int(with_len[L]);
+            shape.matches += double(with_len[L]) / grams;
+            shape.states += std::min(grams, double(longer));
+        }
+        const GramLimits lim = gram_limits(algo, B, shape);
+        if (t.s == 0 || (t.dense ? best_pass > lim.dense_pass : best > lim.cost)) {
             t = GramTables();
             return PM_OK;
         }
@@ -351,7 +375,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
                 t = GramTables();
                 return PM_OK;
             }
-            t.scan = false;
+            t.list = t.counts = false;
         }
         t.dir.assign(2 * (nb + 1), 0u);
         for (size_t b = 0; b <= nb; ++b) {
@@ -389,6 +413,7 @@ int build_gram(const uint8_t *P, const int64_t *off, int64_t d, int32_t m, int32
                 t.id_off.push_back(uint16_t(t.ids.size()));
             }
         }
+        if (algo == PM_ALGO_ACV) acv_modes(shape, t.s, t.list, t.counts);
         t.ok = true;
         return PM_OK;
     } catch (const std::bad_alloc &) {

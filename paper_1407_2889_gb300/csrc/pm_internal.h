@@ -157,7 +157,8 @@ struct GramEntry {
 
 struct GramTables {
     bool ok = false;
-    bool scan = true;              // false: for the host walk only, scans keep the method's own tables
+    // which scans take the tables (neither: the host walk only)
+    bool list = true, counts = true;
     bool var = false;              // mixed lengths: no groups, code = pattern id
     bool direct = false;           // the hash is the gram itself, shifted to the top: the filter is exact
     bool rank = false;             // buckets by rank in the filter

@@ -516,7 +516,7 @@ int acv_launch(const AcvTables &v, const DevAcv &dv, const uint8_t *d_text, int6
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long nsub = warp_tiles(n);
     const int se = acv_slot_bytes(v);
-    if (dv.dg && n >= v.m_min && nsub > 0)
+    if (dv.dg && (list ? dv.gt->list : dv.gt->counts) && n >= v.m_min && nsub > 0)
         return gram_launch_ws(*dv.gt, *dv.dg, d_text, n, list, d_counts, d_occ, occ_cap, d_n_occ, d_ws, 0, se * v.K,
                               v.K, true, nullptr, 0, stream);
     ListParts L;

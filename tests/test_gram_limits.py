@@ -94,3 +94,10 @@ def test_mixed_lengths_with_many_short_patterns(lo, hi, d, kind):
     assert _kind(pm.pm_acv_compile(V, HOST)) == kind
     if d <= 3000:
         assert _kind(pm.pm_wmv_compile(V, 2, HOST)) == pm.PM_SCAN_GRAMS
+
+
+@pytest.mark.parametrize("lo,hi,d,kind", [(10, 20, 1000, pm.PM_SCAN_METHOD), (16, 24, 1000, pm.PM_SCAN_GRAMS),
+                                          (8, 20, 2000, pm.PM_SCAN_GRAMS)])
+def test_mixed_lengths_over_two_letters(lo, hi, d, kind):
+    """A small automaton and few matches beat grams that half of all windows pass."""
+    assert _kind(pm.pm_acv_compile(_mixed(b"AC", d, lo, hi), HOST)) == kind
