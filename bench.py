@@ -38,7 +38,7 @@ KERNEL_SOURCES = ["paper_1407_2889_gb300/csrc/scan_ac.cu", "paper_1407_2889_gb30
                   "paper_1407_2889_gb300/csrc/ac_scan_kernel.cuh", "paper_1407_2889_gb300/csrc/ac_device.cuh",
                   "paper_1407_2889_gb300/csrc/scan_common.cuh"]
 GRAM_SOURCES = ["paper_1407_2889_gb300/csrc/scan_gram.cu", "paper_1407_2889_gb300/csrc/gram_device.cuh",
-                "paper_1407_2889_gb300/csrc/scan_common.cuh"]
+                "paper_1407_2889_gb300/csrc/gram.cpp", "paper_1407_2889_gb300/csrc/scan_common.cuh"]
 
 
 def kernel_hash(sources=KERNEL_SOURCES) -> str:
@@ -78,23 +78,24 @@ def scan_kernels(pm, s, algo):
 
 
 def recorded_traffic(kernel_name: str, workload: str, plan=None):
-    """DRAM bytes per launch from a committed ncu summary, if it was taken on
-    the current kernel source, the same workload and the same launch plan
-    (or one the record lists as resolving to the same kernels and launch
-    shapes for this workload); else None."""
+    """DRAM bytes per launch from a committed ncu summary and how they were
+    taken (a smaller capture, scaled), if that was on the current kernel
+    source, the same workload and the same launch plan (or one the record
+    lists as resolving to the same kernels and launch shapes for this
+    workload); else None, None."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
-        return None
+        return None, None
     with open(p) as f:
         rec = json.load(f)
     e = rec.get(kernel_name)
     sources = GRAM_SOURCES if kernel_name.startswith("gram") else KERNEL_SOURCES
     if not e or e.get("kernel_hash") != kernel_hash(sources) or e.get("workload") != workload:
-        return None
+        return None, None
     plans = [e.get("plan")] + list(e.get("same_plans", []))
     if not any(plan_key(q) == plan_key(plan) for q in plans):
-        return None
-    return e.get("dram_bytes_per_launch")
+        return None, None
+    return e.get("dram_bytes_per_launch"), e.get("how")
 
 
 class ClockSampler:
@@ -384,10 +385,10 @@ def main():
     achieved = alg_bytes / avg_launch_s / 1e9
     gram = s.scan_kind() != pm.PM_SCAN_METHOD
     kernel, expand = scan_kernels(pm, s, args.algo)
+    traffic, traffic_how = recorded_traffic(kernel, f"est1gib_d{d}_m{args.m}_{args.mode}_n{n}", pinned_plan or tuned)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "peak_kind": peak_kind,
-                "traffic": recorded_traffic(kernel, f"est1gib_d{d}_m{args.m}_{args.mode}_n{n}",
-                                            pinned_plan or tuned),
+                "traffic": traffic, "traffic_how": traffic_how,
                 "algorithmic_bytes_per_launch": alg_bytes,
                 "kernel": kernel + (f" + {expand} (list mode)" if args.mode == "list" else "")}
 

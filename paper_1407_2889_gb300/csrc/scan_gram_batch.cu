@@ -29,7 +29,9 @@ namespace {
 using dev::kFull;
 using namespace gramdev;
 
-constexpr int kWarps = 24;           // with 32 (64 registers) the walk spills: 570 us for the batch above against 502
+// Most walks spill at 24 warps (80 registers; 8 to 220 bytes by ptxas, stride 16
+// most), more at 32 (64 registers): 570 us for the batch above against 502.
+constexpr int kWarps = 24;
 constexpr int kHits = 192;           // matches a warp keeps per tile
 constexpr int kMaxTile = 32768;      // a match's offset has 16 bits
 
@@ -345,7 +347,7 @@ bool gram_batch_layout(const GramTables &t, long long smem, int &hist_off, int &
     const long long tab = (long long)t.filter.size() * 4 * (t.rank ? 2 : 1);
     if (tab > room || t.filter.size() % 4 != 0) return false;
     hist_off = tab + nc * 4 <= room ? int(tab) : -1;
-    // tiles of at most about 48 expected matches
+    // tiles of at most kHits / 2 = 96 expected matches
     const double density = double(nc) / std::pow(4.0, double(std::min(t.m_min, 16)));
     const int step = kRow;
     tile = step;
