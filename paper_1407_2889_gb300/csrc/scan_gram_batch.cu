@@ -120,7 +120,7 @@ __device__ __noinline__ void run_gram(const BatchArgs &a, const BatchDesc &D, un
             } else {
 #pragma unroll
                 for (int r = 0; r <= R; ++r)
-                    if (r < R || lane == 0) v[r] = load16(text, n, aligned, lo + off + r * kRow + lane * 16);
+                    if (r < R || lane == 0) v[r] = load16<false>(text, n, aligned, lo + off + r * kRow + lane * 16);
             }
         };
         v[R] = make_uint4(0u, 0u, 0u, 0u);
